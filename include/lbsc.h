@@ -396,8 +396,9 @@ int lb_set_step_variant(lb_ctx* ctx, int variant, int stages);
  * discrete adjoint of the step (Sec. 2: the reverse of streaming with
  * bounce-back, BGK with Eq. Equil, the velocity shift and Eq. SCforce with
  * the wall as a species). States are checkpointed every ckpt_every steps
- * and recomputed one segment at a time (device memory: nsteps/ckpt_every + 1
- * + ckpt_every states). Planar walls only (LB_ERR_UNSUPPORTED otherwise).
+ * and recomputed one segment at a time (device memory: a state per segment,
+ * two more, and 10 floats a node for each of ckpt_every + 1 time levels).
+ * Planar walls only (LB_ERR_UNSUPPORTED otherwise).
  * The paper calibrates the wall parameter by repeated runs; the gradient
  * replaces that search. J may be NULL. */
 int lb_step_backward(lb_ctx* ctx, int nsteps, int ckpt_every, int observable, double* dJ_deta, double* J);

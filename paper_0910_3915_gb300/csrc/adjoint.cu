@@ -17,15 +17,19 @@
 // to psi^abar of its 18 neighbours (or to eta_abar where the neighbour is a
 // wall); a second pass gathers those contributions.
 //
-// Adjoint arrays are dense, index x + nx*(y + ny*z), FP32; gradient sums FP64.
+// The adjoint of n_k(t) is kept as
+//   lambda_k(t) = M_k + E_k,  M_k = (1 - omega) mu_k,  E_k = rhobar + c_k . jbar,
+// so a reverse step writes E's 4 values per component (32 bytes a node)
+// where writing and re-reading lambda itself took 3 passes over 38 values.
+// At tau = 1 M vanishes and is neither stored nor read: lambda lives in E
+// alone. All fields are dense, index x + nx*(y + ny*z), and hold both
+// components of a node side by side (one 8-byte access for the two).
+// Gradient sums are FP64.
 #include "lb_fields.cuh"
 
 namespace lbsc {
 
-__device__ __forceinline__ long long didx(int x, int y, int z, int nx, int ny)
-{
-    return (long long)x + (long long)nx * (y + (long long)ny * z);
-}
+__device__ __forceinline__ int didx(int x, int y, int z, int nx, int ny) { return x + nx * (y + ny * z); }
 __device__ __forceinline__ bool wall_z(int z, int nz) { return z == 0 || z == nz - 1; }
 // coordinates of dense node index i (32-bit: node counts stay below 2^31)
 __device__ __forceinline__ void node_xyz(int i, int nx, int ny, int& x, int& y, int& z)
@@ -35,133 +39,171 @@ __device__ __forceinline__ void node_xyz(int i, int nx, int ny, int& x, int& y, 
     z = t / ny;
     y = t - z * ny;
 }
+__device__ __forceinline__ float lane(const float2& v, int a) { return a ? v.y : v.x; }
+// s + c v for a velocity component c in {-1, 0, 1} known at compile time after unrolling
+__device__ __forceinline__ float add_c(float s, int c, float v) { return c == 0 ? s : (c > 0 ? s + v : s - v); }
 
-// forward rho, j, psi of the stored state (lattice layout L)
+// Forward rho, j, psi of the stored state (lattice layout L), one thread per
+// node, both components of a velocity in one load. Bound by the read of the
+// populations (152 bytes a node, from L2 when it follows the step that wrote
+// them): 8.5 us at 64^3 FP32 (cold caches), 11.4 with a grid-stride grid of 512
+// blocks and one component at a time.
 template <class S>
-__global__ void adj_forward_kernel(Layout L, KParams P, const S* __restrict__ f, AdjFields A)
+__global__ void __launch_bounds__(kAdjThreads) adj_forward_kernel(Layout L, KParams P, const S* __restrict__ f, AdjState A)
 {
-    const long long N = (long long)L.nx * L.ny * L.nz;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        int x, y, z;
-        node_xyz((int)i, L.nx, L.ny, x, y, z);
-        const bool solid = wall_z(z, L.nz);
+    const int N = L.nx * L.ny * L.nz;
+    const int i = blockIdx.x * kAdjThreads + threadIdx.x;
+    if (i >= N) return;
+    int x, y, z;
+    node_xyz(i, L.nx, L.ny, x, y, z);
+    const bool solid = wall_z(z, L.nz);
+    float2 w[Q];
+    if (!solid) {
         const long long off = L.off(x, y, z);
-        #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            float r = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
-            if (!solid) {
-                #pragma unroll
-                for (int k = 0; k < Q; ++k) {
-                    float v = Codec<S>::load(f + L.at(a, k, off));
-                    if constexpr (Codec<S>::kDeviation) v = zeta(k) * (P.ref[a] + v);
-                    r += v;
-                    jx += cx(k) * v;
-                    jy += cy(k) * v;
-                    jz += cz(k) * v;
-                }
-            }
-            A.rho[a][i] = r;
-            A.j[a][0][i] = jx;
-            A.j[a][1][i] = jy;
-            A.j[a][2][i] = jz;
-            A.psi[a][i] = solid ? P.eta[a] : -expm1f(-r);
-        }
+#pragma unroll
+        for (int k = 0; k < Q; ++k) w[k] = Codec<S>::load2(f + L.at(0, k, off));
     }
+    float r[2], j[2][3], psi[2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+        float s = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
+        if (!solid) {
+#pragma unroll
+            for (int k = 0; k < Q; ++k) {
+                float v = lane(w[k], a);
+                if constexpr (Codec<S>::kDeviation) v = zeta(k) * (P.ref[a] + v);
+                s += v;
+                jx += cx(k) * v;
+                jy += cy(k) * v;
+                jz += cz(k) * v;
+            }
+        }
+        r[a] = s;
+        j[a][0] = jx;
+        j[a][1] = jy;
+        j[a][2] = jz;
+        psi[a] = solid ? P.eta[a] : -expm1f(-s);
+    }
+    A.rho[i] = make_float2(r[0], r[1]);
+    A.psi[i] = make_float2(psi[0], psi[1]);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) A.j[d][i] = make_float2(j[0][d], j[1][d]);
 }
 
-// Pass A: per fluid node, mu from lambda(t+1), the local adjoint of BGK,
-// equilibrium, shift, u' and force; lambda(t) gets (1 - omega) mu; the wall
-// gradient is reduced into part[block][2] (FP64).
-__global__ void __launch_bounds__(256)
-    adj_local_kernel(AdjArgs G, AdjFields A, const float* __restrict__ lam_next, float* __restrict__ lam_cur,
-                     double* __restrict__ part)
+// Pass A of a reverse step, one thread per fluid node: mu from lambda(t+1),
+// the local adjoint of BGK, equilibrium, shift, u' and force. Writes jbar and
+// (before the psi term) rhobar into E(t), M(t) where tau != 1, and V and psibar
+// for pass B. The wall gradient of the block is added to its own row of
+// part[block][2] (FP64), which one pass sums after the last step.
+// Issue-bound (about 1500 FP32 operations a node, 25 of them divisions): the
+// neighbours' E and psi are L1/L2 hits, 8-byte loads of both components.
+// 25 us at 64^3; 75 when it read and wrote lambda's 38 values. One thread summed
+// the blocks' rows after every step before (32 us).
+template <bool kTauOne>
+__global__ void __launch_bounds__(kAdjThreads)
+    adj_local_kernel(AdjArgs G, AdjState A, AdjE En, const float* __restrict__ Mn, AdjE Ec, float* __restrict__ Mc,
+                     AdjV W, double* __restrict__ part)
 {
     const int nx = G.nx, ny = G.ny, nz = G.nz;
-    const long long N = (long long)nx * ny * nz;
+    const int N = nx * ny * nz;
+    const int i = blockIdx.x * kAdjThreads + threadIdx.x;
     double geta[2] = {0.0, 0.0};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        int x, y, z;
-        node_xyz((int)i, nx, ny, x, y, z);
-        if (wall_z(z, nz)) {
-            #pragma unroll
-            for (int k = 0; k < 2 * Q; ++k) lam_cur[(long long)k * N + i] = 0.f;
-            #pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                A.rhob[a][i] = 0.f;
-                A.psib[a][i] = 0.f;
-                #pragma unroll
-                for (int d = 0; d < 3; ++d) A.jb[a][d][i] = A.V[a][d][i] = 0.f;
-            }
-            continue;
-        }
+    bool at_wall = false;
+    int x = 0, y = 0, z = 0;
+    if (i < N) node_xyz(i, nx, ny, x, y, z);
+    if (i < N && !wall_z(z, nz)) {
+        const int xo[3] = {wrapi(x - 1, nx), x, wrapi(x + 1, nx)};
+        const int yo[3] = {wrapi(y - 1, ny), y, wrapi(y + 1, ny)};
+        const bool zwall[3] = {wall_z(z - 1, nz), false, wall_z(z + 1, nz)};
+        at_wall = zwall[0] || zwall[2];
         float rho[2], j[2][3], psi[2], S[2][3], F[2][3];
-        #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            rho[a] = A.rho[a][i];
-            psi[a] = A.psi[a][i];
-            #pragma unroll
-            for (int d = 0; d < 3; ++d) j[a][d] = A.j[a][d][i];
-        }
-        // S^a = sum_m G_m psi~^abar(y + c_m) c_m, wall links flagged
-        #pragma unroll
-        for (int a = 0; a < 2; ++a) S[a][0] = S[a][1] = S[a][2] = 0.f;
-        #pragma unroll
-        for (int m = 1; m < Q; ++m) {
-            const long long n = didx(wrapi(x + cx(m), nx), wrapi(y + cy(m), ny), z + cz(m), nx, ny);
-            #pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                const float ps = G.G[m] * A.psi[1 - a][n];
-                S[a][0] += ps * cx(m);
-                S[a][1] += ps * cy(m);
-                S[a][2] += ps * cz(m);
+        {
+            const float2 r2 = A.rho[i], p2 = A.psi[i];
+            rho[0] = r2.x, rho[1] = r2.y, psi[0] = p2.x, psi[1] = p2.y;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const float2 t = A.j[d][i];
+                j[0][d] = t.x, j[1][d] = t.y;
             }
         }
-        #pragma unroll
+        // S^a = sum_m G_m psi~^abar(y + c_m) c_m
+#pragma unroll
+        for (int a = 0; a < 2; ++a) S[a][0] = S[a][1] = S[a][2] = 0.f;
+#pragma unroll
+        for (int m = 1; m < Q; ++m) {
+            const float2 pn = A.psi[didx(xo[cx(m) + 1], yo[cy(m) + 1], z + cz(m), nx, ny)];
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const float ps = G.G[m] * lane(pn, 1 - a);
+                S[a][0] = add_c(S[a][0], cx(m), ps);
+                S[a][1] = add_c(S[a][1], cy(m), ps);
+                S[a][2] = add_c(S[a][2], cz(m), ps);
+            }
+        }
+#pragma unroll
         for (int a = 0; a < 2; ++a)
-            #pragma unroll
+#pragma unroll
             for (int d = 0; d < 3; ++d) F[a][d] = -G.gk * psi[a] * S[a][d];
         const float D = G.omega[0] * rho[0] + G.omega[1] * rho[1];
         float up[3] = {0.f, 0.f, 0.f};
         if (D > 0.f)
-            #pragma unroll
+#pragma unroll
             for (int d = 0; d < 3; ++d) up[d] = (G.omega[0] * j[0][d] + G.omega[1] * j[1][d]) / D;
 
-        float rhob[2] = {0.f, 0.f}, ub[2][3], upb[3] = {0.f, 0.f, 0.f};
-        #pragma unroll
+        float rhob[2] = {0.f, 0.f}, ub[2][3], upb[3] = {0.f, 0.f, 0.f}, u[2][3], usq[2];
+#pragma unroll
         for (int a = 0; a < 2; ++a) {
             const bool shift = rho[a] > 1e-12f;
-            float u[3];
-            #pragma unroll
-            for (int d = 0; d < 3; ++d) u[d] = up[d] + (shift ? G.tau[a] * F[a][d] / rho[a] : 0.f);
-            const float usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) u[a][d] = up[d] + (shift ? G.tau[a] * F[a][d] / rho[a] : 0.f);
+            usq[a] = u[a][0] * u[a][0] + u[a][1] * u[a][1] + u[a][2] * u[a][2];
             ub[a][0] = ub[a][1] = ub[a][2] = 0.f;
-            #pragma unroll
-            for (int k = 0; k < Q; ++k) {
-                // mu_k = lambda_k(y + c_k), or lambda_kbar(y) when y + c_k is a wall
-                const int zt = z + cz(k);
-                float mu;
-                if (wall_z(zt, nz)) mu = lam_next[(long long)(a * Q + opp(k)) * N + i];
-                else mu = lam_next[(long long)(a * Q + k) * N + didx(wrapi(x + cx(k), nx), wrapi(y + cy(k), ny), zt, nx, ny)];
-                lam_cur[(long long)(a * Q + k) * N + i] = (1.0f - G.omega[a]) * mu;
-                const float qb = G.omega[a] * mu;
-                const float cu = cx(k) * u[0] + cy(k) * u[1] + cz(k) * u[2];
-                const float P = 3.f * cu + 4.5f * cu * cu - 1.5f * usq + 4.5f * cu * cu * cu - 4.5f * usq * cu;
-                rhob[a] += qb * zeta(k) * (1.0f + P);
-                const float Ak = 3.f + 9.f * cu + 13.5f * cu * cu - 4.5f * usq, Bk = -3.f - 9.f * cu;
-                const float w = qb * zeta(k) * rho[a];
-                ub[a][0] += w * (cx(k) * Ak + u[0] * Bk);
-                ub[a][1] += w * (cy(k) * Ak + u[1] * Bk);
-                ub[a][2] += w * (cz(k) * Ak + u[2] * Bk);
-            }
-            #pragma unroll
-            for (int d = 0; d < 3; ++d) upb[d] += ub[a][d];
         }
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            // mu_k = lambda_k(y + c_k), or lambda_kbar(y) when y + c_k is a wall
+            const bool wall = cz(k) != 0 && zwall[cz(k) + 1];
+            const int n = wall ? i : didx(xo[cx(k) + 1], yo[cy(k) + 1], z + cz(k), nx, ny);
+            float2 lam = En.rb[n];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int c = d == 0 ? cx(k) : (d == 1 ? cy(k) : cz(k));
+                if (c == 0) continue;
+                float2 e = En.j[d][n];
+                if (cz(k) != 0 && wall) e = make_float2(-e.x, -e.y);  // c_kbar = -c_k
+                lam.x = add_c(lam.x, c, e.x);
+                lam.y = add_c(lam.y, c, e.y);
+            }
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                float mu = lane(lam, a);
+                if constexpr (!kTauOne) {
+                    mu += Mn[(long long)(a * Q + (wall ? opp(k) : k)) * N + n];
+                    Mc[(long long)(a * Q + k) * N + i] = (1.0f - G.omega[a]) * mu;
+                }
+                const float qb = G.omega[a] * mu;
+                // the zero products stay: without them the compiler shares terms between opposite
+                // velocities and fuses others, which moves the gradient by 1e-8 of itself
+                const float cu = cx(k) * u[a][0] + cy(k) * u[a][1] + cz(k) * u[a][2];
+                const float P = 3.f * cu + 4.5f * cu * cu - 1.5f * usq[a] + 4.5f * cu * cu * cu - 4.5f * usq[a] * cu;
+                rhob[a] += qb * zeta(k) * (1.0f + P);
+                const float Ak = 3.f + 9.f * cu + 13.5f * cu * cu - 4.5f * usq[a], Bk = -3.f - 9.f * cu;
+                const float w = qb * zeta(k) * rho[a];
+                ub[a][0] += w * (cx(k) * Ak + u[a][0] * Bk);
+                ub[a][1] += w * (cy(k) * Ak + u[a][1] * Bk);
+                ub[a][2] += w * (cz(k) * Ak + u[a][2] * Bk);
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) upb[d] += ub[a][d];
         float Fb[2][3];
-        #pragma unroll
+#pragma unroll
         for (int a = 0; a < 2; ++a) {
             const bool shift = rho[a] > 1e-12f;
             float dot = 0.f;
-            #pragma unroll
+#pragma unroll
             for (int d = 0; d < 3; ++d) {
                 Fb[a][d] = shift ? ub[a][d] * G.tau[a] / rho[a] : 0.f;
                 dot += ub[a][d] * F[a][d];
@@ -171,42 +213,52 @@ __global__ void __launch_bounds__(256)
         float jb[2][3];
         if (D > 0.f) {
             const float updot = upb[0] * up[0] + upb[1] * up[1] + upb[2] * up[2];
-            #pragma unroll
+#pragma unroll
             for (int a = 0; a < 2; ++a) {
-                #pragma unroll
+#pragma unroll
                 for (int d = 0; d < 3; ++d) jb[a][d] = G.omega[a] * upb[d] / D;
                 rhob[a] -= G.omega[a] * updot / D;
             }
         } else {
-            #pragma unroll
+#pragma unroll
             for (int a = 0; a < 2; ++a) jb[a][0] = jb[a][1] = jb[a][2] = 0.f;
         }
         // force: psi^a(y) factor and the neighbour sum
-        #pragma unroll
+        float V[2][3], psib[2];
+#pragma unroll
         for (int a = 0; a < 2; ++a) {
-            float V[3];
             float sdot = 0.f;
-            #pragma unroll
+#pragma unroll
             for (int d = 0; d < 3; ++d) {
-                V[d] = -G.gk * psi[a] * Fb[a][d];
+                V[a][d] = -G.gk * psi[a] * Fb[a][d];
                 sdot += Fb[a][d] * S[a][d];
             }
-            A.psib[a][i] = -G.gk * sdot;
-            #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                A.V[a][d][i] = V[d];
-                A.jb[a][d][i] = jb[a][d];
-            }
-            A.rhob[a][i] = rhob[a];
+            psib[a] = -G.gk * sdot;
             // wall links of the neighbour sum feed d J / d eta_abar
-            #pragma unroll
-            for (int m = 1; m < Q; ++m)
-                if (wall_z(z + cz(m), nz)) geta[1 - a] += (double)(G.G[m] * (V[0] * cx(m) + V[1] * cy(m) + V[2] * cz(m)));
+            if (at_wall) {
+#pragma unroll
+                for (int m = 1; m < Q; ++m) {
+                    if (cz(m) == 0 || !zwall[cz(m) + 1]) continue;
+                    float t = 0.f;
+                    t = add_c(t, cx(m), V[a][0]);
+                    t = add_c(t, cy(m), V[a][1]);
+                    t = add_c(t, cz(m), V[a][2]);
+                    geta[1 - a] += (double)(G.G[m] * t);
+                }
+            }
+        }
+        Ec.rb[i] = make_float2(rhob[0], rhob[1]);
+        W.psib[i] = make_float2(psib[0], psib[1]);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            Ec.j[d][i] = make_float2(jb[0][d], jb[1][d]);
+            W.v[d][i] = make_float2(V[0][d], V[1][d]);
         }
     }
-    // block reduction of the wall gradient
-    __shared__ double sh[8][2];
-    #pragma unroll
+    // block sum of the wall gradient, in blocks that hold a node next to a wall
+    if (!__syncthreads_or(at_wall)) return;
+    __shared__ double sh[kAdjThreads / 32][2];
+#pragma unroll
     for (int a = 0; a < 2; ++a) {
         double v = geta[a];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -215,38 +267,67 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
     if (threadIdx.x < 2) {
         double v = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w][threadIdx.x];
-        part[blockIdx.x * 2 + threadIdx.x] = v;
+        for (int w = 0; w < kAdjThreads / 32; ++w) v += sh[w][threadIdx.x];
+        part[blockIdx.x * 2 + threadIdx.x] += v;  // this block's row, step after step
     }
 }
 
 // Pass B: gather the neighbours' force adjoints into psibar, then finish
-// lambda(t) = (1 - omega) mu + rhobar + c . jbar with rhobar including psibar psi'.
-__global__ void adj_gather_kernel(AdjArgs G, AdjFields A, float* __restrict__ lam_cur)
+// E(t)'s rhobar with psibar psi'. A neighbour's V is read only along the
+// nonzero entries of its link (30 loads of 8 bytes a node, L1/L2 hits).
+// 7.8 us at 64^3; 83 when it loaded all of V and rewrote lambda's 38 values.
+__global__ void __launch_bounds__(kAdjThreads) adj_gather_kernel(AdjArgs G, AdjState A, AdjV W, AdjE Ec)
 {
     const int nx = G.nx, ny = G.ny, nz = G.nz;
-    const long long N = (long long)nx * ny * nz;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        int x, y, z;
-        node_xyz((int)i, nx, ny, x, y, z);
-        if (wall_z(z, nz)) continue;
-        #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            // psi^a(x) is used by F^abar(x - c_m) for every fluid x - c_m
-            float pb = A.psib[a][i];
-            #pragma unroll
-            for (int m = 1; m < Q; ++m) {
-                const int zs = z - cz(m);
-                if (wall_z(zs, nz)) continue;
-                const long long s = didx(wrapi(x - cx(m), nx), wrapi(y - cy(m), ny), zs, nx, ny);
-                pb += G.G[m] * (A.V[1 - a][0][s] * cx(m) + A.V[1 - a][1][s] * cy(m) + A.V[1 - a][2][s] * cz(m));
-            }
-            const float rb = A.rhob[a][i] + pb * expf(-A.rho[a][i]);
-            const float jb[3] = {A.jb[a][0][i], A.jb[a][1][i], A.jb[a][2][i]};
-            #pragma unroll
-            for (int k = 0; k < Q; ++k)
-                lam_cur[(long long)(a * Q + k) * N + i] += rb + cx(k) * jb[0] + cy(k) * jb[1] + cz(k) * jb[2];
+    const int N = nx * ny * nz;
+    const int i = blockIdx.x * kAdjThreads + threadIdx.x;
+    if (i >= N) return;
+    int x, y, z;
+    node_xyz(i, nx, ny, x, y, z);
+    if (wall_z(z, nz)) return;
+    const int xo[3] = {wrapi(x - 1, nx), x, wrapi(x + 1, nx)};
+    const int yo[3] = {wrapi(y - 1, ny), y, wrapi(y + 1, ny)};
+    const bool zwall[3] = {wall_z(z - 1, nz), false, wall_z(z + 1, nz)};
+    const float2 p2 = W.psib[i], r2 = A.rho[i], b2 = Ec.rb[i];
+    float pb[2] = {p2.x, p2.y};
+    // psi^a(x) is used by F^abar(x - c_m) for every fluid x - c_m
+#pragma unroll
+    for (int m = 1; m < Q; ++m) {
+        if (cz(m) != 0 && zwall[1 - cz(m)]) continue;
+        const int s = didx(xo[1 - cx(m)], yo[1 - cy(m)], z - cz(m), nx, ny);
+        float2 t = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int c = d == 0 ? cx(m) : (d == 1 ? cy(m) : cz(m));
+            if (c == 0) continue;
+            const float2 v = W.v[d][s];
+            t.x = add_c(t.x, c, v.x);
+            t.y = add_c(t.y, c, v.y);
         }
+        pb[0] += G.G[m] * t.y;
+        pb[1] += G.G[m] * t.x;
+    }
+    float rb[2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a) rb[a] = lane(b2, a) + pb[a] * expf(-lane(r2, a));
+    Ec.rb[i] = make_float2(rb[0], rb[1]);
+}
+
+// out[a] = sum over the blocks' rows of part: thread t rows t, t + 256, ... in
+// order, a fixed shuffle tree per warp, then the warps in order (a = blockIdx.x)
+__global__ void __launch_bounds__(256) rows_sum_kernel(const double* __restrict__ part, int nblocks, double* __restrict__ out)
+{
+    const int a = blockIdx.x;
+    double v = 0;
+    for (int b = threadIdx.x; b < nblocks; b += 256) v += part[2 * b + a];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    __shared__ double sh[8];
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0;
+        for (int w = 0; w < 8; ++w) t += sh[w];
+        out[a] = t;
     }
 }
 
@@ -256,8 +337,8 @@ __global__ void adj_gather_kernel(AdjArgs G, AdjFields A, float* __restrict__ la
 // obs 2: wetted area, sum over the first fluid layer of sigma(phi / eps)
 __device__ __forceinline__ double sigmoid(double s) { return 1.0 / (1.0 + exp(-s)); }
 
-__global__ void obs_sums_kernel(int nx, int ny, int nz, int obs, double eps, const float* __restrict__ rr,
-                                const float* __restrict__ rb, double* __restrict__ part)
+__global__ void obs_sums_kernel(int nx, int ny, int nz, int obs, double eps, const float2* __restrict__ rho,
+                                double* __restrict__ part)
 {
     const long long N = (long long)nx * ny * nz;
     double s0 = 0, s1 = 0;
@@ -266,10 +347,10 @@ __global__ void obs_sums_kernel(int nx, int ny, int nz, int obs, double eps, con
         if (wall_z(z, nz)) continue;
         const double h = z - 0.5;
         if (obs == 0) {
-            s0 += rr[i];
-            s1 += h * rr[i];
+            s0 += rho[i].x;
+            s1 += h * rho[i].x;
         } else {
-            const double w = sigmoid(((double)rr[i] - (double)rb[i]) / eps);
+            const double w = sigmoid(((double)rho[i].x - (double)rho[i].y) / eps);
             if (obs == 1) {
                 s0 += w;
                 s1 += h * w;
@@ -295,22 +376,15 @@ __global__ void obs_sums_kernel(int nx, int ny, int nz, int obs, double eps, con
     }
 }
 
-// sums[0..1] = reduced (s0, s1); J = s1/s0 (obs 0, 1) or s0 (obs 2), written to sums[2]
-__global__ void obs_finish_kernel(const double* __restrict__ part, int nblocks, int obs, double* __restrict__ sums)
+// J = s1/s0 (obs 0, 1) or s0 (obs 2) from the reduced sums[0..1], written to sums[2]
+__global__ void obs_finish_kernel(int obs, double* __restrict__ sums)
 {
-    if (threadIdx.x != 0) return;
-    double s0 = 0, s1 = 0;
-    for (int b = 0; b < nblocks; ++b) {
-        s0 += part[2 * b];
-        s1 += part[2 * b + 1];
-    }
-    sums[0] = s0;
-    sums[1] = s1;
-    sums[2] = obs == 2 ? s0 : s1 / s0;
+    if (threadIdx.x == 0) sums[2] = obs == 2 ? sums[0] : sums[1] / sums[0];
 }
 
-__global__ void obs_grad_kernel(int nx, int ny, int nz, int obs, double eps, const float* __restrict__ rr,
-                                const float* __restrict__ rb, const double* __restrict__ sums, float* __restrict__ lam)
+// lambda(T) = dJ/dn(T) as E: the same for every velocity, so rhobar = dJ/drho and jbar = 0
+__global__ void obs_grad_kernel(int nx, int ny, int nz, int obs, double eps, const float2* __restrict__ rho,
+                                const double* __restrict__ sums, AdjE E)
 {
     const long long N = (long long)nx * ny * nz;
     const double s0 = sums[0], J = sums[2];
@@ -322,7 +396,7 @@ __global__ void obs_grad_kernel(int nx, int ny, int nz, int obs, double eps, con
             if (obs == 0) {
                 gr = (h - J) / s0;
             } else {
-                const double w = sigmoid(((double)rr[i] - (double)rb[i]) / eps);
+                const double w = sigmoid(((double)rho[i].x - (double)rho[i].y) / eps);
                 const double dw = w * (1.0 - w) / eps;  // d w / d phi
                 double gphi = 0;
                 if (obs == 1) gphi = (h - J) * dw / s0;
@@ -331,52 +405,50 @@ __global__ void obs_grad_kernel(int nx, int ny, int nz, int obs, double eps, con
                 gb = -gphi;
             }
         }
-        #pragma unroll
-        for (int k = 0; k < Q; ++k) {
-            lam[(long long)k * N + i] = (float)gr;
-            lam[(long long)(Q + k) * N + i] = (float)gb;
-        }
+        E.rb[i] = make_float2((float)gr, (float)gb);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) E.j[d][i] = make_float2(0.f, 0.f);
     }
 }
 
-// accumulate the per-block wall gradient of one backward step into acc[2] (block order)
-__global__ void adj_acc_kernel(const double* __restrict__ part, int nblocks, double* __restrict__ acc)
-{
-    const int a = threadIdx.x;
-    if (a >= 2) return;
-    double v = 0;
-    for (int b = 0; b < nblocks; ++b) v += part[2 * b + a];
-    acc[a] += v;
-}
+static int adj_blocks(long long n) { return (int)((n + kAdjThreads - 1) / kAdjThreads); }
 
 template <class S>
-cudaError_t launch_adj_forward(const Layout& L, const KParams& P, const S* f, const AdjFields& A, cudaStream_t st)
+cudaError_t launch_adj_forward(const Layout& L, const KParams& P, const S* f, const AdjState& A, cudaStream_t st)
 {
-    adj_forward_kernel<S><<<kAdjBlocks, 256, 0, st>>>(L, P, f, A);
+    adj_forward_kernel<S><<<adj_blocks((long long)L.nx * L.ny * L.nz), kAdjThreads, 0, st>>>(L, P, f, A);
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_backstep(const AdjArgs& G, const AdjFields& A, const float* lam_next, float* lam_cur,
-                                double* part, double* acc, cudaStream_t st)
+cudaError_t launch_adj_backstep(const AdjArgs& G, const AdjState& A, bool tau_one, const AdjE& En, const float* Mn,
+                                const AdjE& Ec, float* Mc, const AdjV& W, double* part, cudaStream_t st)
 {
-    adj_local_kernel<<<kAdjBlocks, 256, 0, st>>>(G, A, lam_next, lam_cur, part);
-    adj_gather_kernel<<<kAdjBlocks, 256, 0, st>>>(G, A, lam_cur);
-    adj_acc_kernel<<<1, 32, 0, st>>>(part, kAdjBlocks, acc);
+    const int blocks = adj_blocks((long long)G.nx * G.ny * G.nz);
+    if (tau_one) adj_local_kernel<true><<<blocks, kAdjThreads, 0, st>>>(G, A, En, Mn, Ec, Mc, W, part);
+    else adj_local_kernel<false><<<blocks, kAdjThreads, 0, st>>>(G, A, En, Mn, Ec, Mc, W, part);
+    adj_gather_kernel<<<blocks, kAdjThreads, 0, st>>>(G, A, W, Ec);
     return cudaGetLastError();
 }
 
-cudaError_t launch_observable(int nx, int ny, int nz, int obs, double eps, const float* rr, const float* rb,
-                              double* part, double* sums, float* lam, cudaStream_t st)
+cudaError_t launch_rows_sum(const double* part, int nblocks, double* out, cudaStream_t st)
 {
-    obs_sums_kernel<<<kAdjBlocks, 256, 0, st>>>(nx, ny, nz, obs, eps, rr, rb, part);
-    obs_finish_kernel<<<1, 32, 0, st>>>(part, kAdjBlocks, obs, sums);
-    if (lam) obs_grad_kernel<<<kAdjBlocks, 256, 0, st>>>(nx, ny, nz, obs, eps, rr, rb, sums, lam);
+    rows_sum_kernel<<<2, 256, 0, st>>>(part, nblocks, out);
     return cudaGetLastError();
 }
 
-template cudaError_t launch_adj_forward<float>(const Layout&, const KParams&, const float*, const AdjFields&, cudaStream_t);
-template cudaError_t launch_adj_forward<__half>(const Layout&, const KParams&, const __half*, const AdjFields&, cudaStream_t);
+cudaError_t launch_observable(int nx, int ny, int nz, int obs, double eps, const float2* rho, double* part,
+                              double* sums, const AdjE* E, cudaStream_t st)
+{
+    obs_sums_kernel<<<kObsBlocks, 256, 0, st>>>(nx, ny, nz, obs, eps, rho, part);
+    rows_sum_kernel<<<2, 256, 0, st>>>(part, kObsBlocks, sums);
+    obs_finish_kernel<<<1, 32, 0, st>>>(obs, sums);
+    if (E) obs_grad_kernel<<<kObsBlocks, 256, 0, st>>>(nx, ny, nz, obs, eps, rho, sums, *E);
+    return cudaGetLastError();
+}
+
+template cudaError_t launch_adj_forward<float>(const Layout&, const KParams&, const float*, const AdjState&, cudaStream_t);
+template cudaError_t launch_adj_forward<__half>(const Layout&, const KParams&, const __half*, const AdjState&, cudaStream_t);
 template cudaError_t launch_adj_forward<__nv_bfloat16>(const Layout&, const KParams&, const __nv_bfloat16*,
-                                                       const AdjFields&, cudaStream_t);
+                                                       const AdjState&, cudaStream_t);
 
 }  // namespace lbsc

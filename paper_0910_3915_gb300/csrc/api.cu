@@ -261,10 +261,8 @@ static EncodeTiledFn encode_fn()
 // 16 bytes of columns, TY + 2 rows; y row = the main box's columns, one row;
 // corner = 16 bytes of columns, one row. Every box spans one plane and all 19
 // slots.
-static int tensor_map(lb_ctx* c, int buf, int ty)
+static int encode_maps(lb_ctx* c, void* f, int ty, CUtensorMap (&maps)[4])
 {
-    const int ti = tile_index(ty);
-    if (c->tmap_ok[buf][ti]) return LB_OK;
     EncodeTiledFn enc = encode_fn();
     if (!enc) return fail(c, LB_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
     const size_t es = elem_size(c->prec);
@@ -283,13 +281,22 @@ static int tensor_map(lb_ctx* c, int buf, int ty)
                                    : c->prec == LB_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                                        : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     for (int kind = 0; kind < 4; ++kind) {
-        const CUresult r = enc(&c->tmap[buf][ti][kind], dt, 4, c->f[buf], dims, strides, boxes[kind], estr,
+        const CUresult r = enc(&maps[kind], dt, 4, f, dims, strides, boxes[kind], estr,
                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return fail(c, LB_ERR_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
     }
-    c->tmap_ok[buf][ti] = true;
     return LB_OK;
+}
+
+// the maps of the lattice's own buffer `buf`, encoded on first use
+static int tensor_map(lb_ctx* c, int buf, int ty)
+{
+    const int ti = tile_index(ty);
+    if (c->tmap_ok[buf][ti]) return LB_OK;
+    const int rc = encode_maps(c, c->f[buf], ty, c->tmap[buf][ti]);
+    c->tmap_ok[buf][ti] = rc == LB_OK;
+    return rc;
 }
 
 template <class S>
@@ -1460,19 +1467,36 @@ struct AdjScratch {
 };
 }  // namespace
 
+// one step from src into dst (states outside the context) by the lattice's step
+// kernel: the TMA-staged one with src's maps, or (ns = 0) the load-from-global one
 template <class S>
-static cudaError_t adj_step_into(lb_ctx* c, const void* src, void* dst, cudaStream_t st)
+static cudaError_t adj_step_into(lb_ctx* c, const void* src, void* dst, int ns, const CUtensorMap* maps, cudaStream_t st)
 {
     StepArgs<S> A = step_args<S>(c, 0);
     A.src = (const S*)src;
     A.dst = (S*)dst;
+    if (ns) return (cudaError_t)tma_step<S>(0, c->tile_y, ns, tau_one(c), maps, &A, st);
     return launch_step<S>(A, c->tile_y, c->general, tau_one(c), st);
 }
 
 template <class S>
-static cudaError_t adj_forward_of(lb_ctx* c, const void* f, const AdjFields& A, cudaStream_t st)
+static cudaError_t adj_forward_of(lb_ctx* c, const void* f, const AdjState& A, cudaStream_t st)
 {
     return launch_adj_forward<S>(c->L, c->kp, (const S*)f, A, st);
+}
+static cudaError_t adj_forward(lb_ctx* c, const void* f, const AdjState& A, cudaStream_t st)
+{
+    switch (c->prec) {
+    case LB_F32: return adj_forward_of<float>(c, f, A, st);
+    case LB_F16: return adj_forward_of<__half>(c, f, A, st);
+    default: return adj_forward_of<__nv_bfloat16>(c, f, A, st);
+    }
+}
+// the adjoint's forward fields of one state at p (kAdjStateVals * N floats)
+static AdjState adj_state(float* p, size_t N)
+{
+    float2* q = (float2*)p;
+    return AdjState{q, q + N, {q + 2 * N, q + 3 * N, q + 4 * N}};
 }
 
 extern "C" int lb_step_backward(lb_ctx* c, int nsteps, int ckpt_every, int observable, double* dJ_deta, double* J)
@@ -1481,38 +1505,44 @@ extern "C" int lb_step_backward(lb_ctx* c, int nsteps, int ckpt_every, int obser
         return fail(c, LB_ERR_ARG, "lb_step_backward: bad argument");
     if (c->general) return fail(c, LB_ERR_UNSUPPORTED, "lb_step_backward: planar walls only");
     cudaStream_t st = c->stream;
-    const long long N = (long long)c->nx * c->ny * c->nz;
+    const size_t N = (size_t)c->nx * c->ny * c->nz;
     const size_t sb = payload_bytes(c);
+    const bool t1 = tau_one(c);
     const int nseg = (nsteps + ckpt_every - 1) / ckpt_every;
-    const int slen = nsteps < ckpt_every ? (nsteps > 0 ? nsteps : 1) : ckpt_every;
+    const int slen = nsteps < ckpt_every ? nsteps : ckpt_every;  // steps of the longest segment
+    const int blocks = (int)((N + kAdjThreads - 1) / kAdjThreads);
+    // Device memory of the call: the states at the starts of all segments but
+    // the last, two states the recompute steps between, the forward fields
+    // (10 values a node) of one segment's states and of the final one, and
+    // the adjoint's fields
     AdjScratch M;
     char* ck = nullptr;
     char* store = nullptr;
-    float* lam = nullptr;
-    float* aux = nullptr;
+    float* fields = nullptr;
+    float* adj = nullptr;
+    float* mom = nullptr;
     double* dsc = nullptr;
-    if (nseg > 0) LB_CUDA(c, M.alloc((void**)&ck, sb * (size_t)nseg));
-    LB_CUDA(c, M.alloc((void**)&store, sb * (size_t)(slen + 1)));
-    LB_CUDA(c, M.alloc((void**)&lam, sizeof(float) * 2 * 2 * Q * (size_t)N));
-    LB_CUDA(c, M.alloc((void**)&aux, sizeof(float) * 26 * (size_t)N));
-    LB_CUDA(c, M.alloc((void**)&dsc, sizeof(double) * (2 * kAdjBlocks + 8)));
-    double* part = dsc;
-    double* acc = dsc + 2 * kAdjBlocks;
+    if (nseg > 1) LB_CUDA(c, M.alloc((void**)&ck, sb * (size_t)(nseg - 1)));
+    if (nseg > 0) LB_CUDA(c, M.alloc((void**)&store, 2 * sb));
+    LB_CUDA(c, M.alloc((void**)&fields, sizeof(float) * kAdjStateVals * N * (size_t)(slen + 1)));
+    LB_CUDA(c, M.alloc((void**)&adj, sizeof(float) * (2 * kAdjEVals + kAdjVVals) * N));
+    if (!t1) LB_CUDA(c, M.alloc((void**)&mom, sizeof(float) * 2 * 2 * Q * N));
+    LB_CUDA(c, M.alloc((void**)&dsc, sizeof(double) * (2 * (size_t)blocks + 2 * kObsBlocks + 8)));
+    double* part = dsc;                  // the wall gradient, one row a block
+    double* opart = dsc + 2 * (size_t)blocks;
+    double* acc = opart + 2 * kObsBlocks;
     double* sums = acc + 2;
-    AdjFields A;
+    AdjE E[2];
+    AdjV V;
     {
-        float* q = aux;
-        for (int a = 0; a < 2; ++a) A.rho[a] = q, q += N;
-        for (int a = 0; a < 2; ++a) A.psi[a] = q, q += N;
-        for (int a = 0; a < 2; ++a)
-            for (int d = 0; d < 3; ++d) A.j[a][d] = q, q += N;
-        for (int a = 0; a < 2; ++a) A.rhob[a] = q, q += N;
-        for (int a = 0; a < 2; ++a)
-            for (int d = 0; d < 3; ++d) A.jb[a][d] = q, q += N;
-        for (int a = 0; a < 2; ++a)
-            for (int d = 0; d < 3; ++d) A.V[a][d] = q, q += N;
-        for (int a = 0; a < 2; ++a) A.psib[a] = q, q += N;
+        float2* q = (float2*)adj;
+        for (AdjE& e : E) {
+            e = AdjE{q, {q + N, q + 2 * N, q + 3 * N}};
+            q += 4 * N;
+        }
+        V = AdjV{{q, q + N, q + 2 * N}, q + 3 * N};
     }
+    float* Mm[2] = {mom, t1 ? nullptr : mom + 2 * Q * N};
     AdjArgs G;
     G.nx = c->nx;
     G.ny = c->ny;
@@ -1524,87 +1554,111 @@ extern "C" int lb_step_backward(lb_ctx* c, int nsteps, int ckpt_every, int obser
         G.omega[a] = c->kp.itau[a];
         G.eta[a] = c->kp.eta[a];
     }
-    auto fwd_on = [&](const void* f, cudaStream_t s2) -> cudaError_t {
+    const int ns = tma_stages(c);
+    CUtensorMap maps[2][4];
+    if (ns && nseg > 0)
+        for (int b = 0; b < 2; ++b) {
+            const int rc = encode_maps(c, store + sb * (size_t)b, c->tile_y, maps[b]);
+            if (rc != LB_OK) return rc;
+        }
+    auto step_of = [&](int b, cudaStream_t s2) -> cudaError_t {  // store[b] -> store[1 - b]
+        char *src = store + sb * (size_t)b, *dst = store + sb * (size_t)(1 - b);
         switch (c->prec) {
-        case LB_F32: return adj_forward_of<float>(c, f, A, s2);
-        case LB_F16: return adj_forward_of<__half>(c, f, A, s2);
-        default: return adj_forward_of<__nv_bfloat16>(c, f, A, s2);
+        case LB_F32: return adj_step_into<float>(c, src, dst, ns, maps[b], s2);
+        case LB_F16: return adj_step_into<__half>(c, src, dst, ns, maps[b], s2);
+        default: return adj_step_into<__nv_bfloat16>(c, src, dst, ns, maps[b], s2);
         }
     };
-    auto fwd = [&](const void* f) { return fwd_on(f, st); };
-    auto step_into = [&](const void* src, void* dst, cudaStream_t s2) -> cudaError_t {
-        switch (c->prec) {
-        case LB_F32: return adj_step_into<float>(c, src, dst, s2);
-        case LB_F16: return adj_step_into<__half>(c, src, dst, s2);
-        default: return adj_step_into<__nv_bfloat16>(c, src, dst, s2);
-        }
-    };
-    // One segment's recompute and reverse sweep, as launched on stream s2. The
-    // launches depend only on the segment length and on which lambda buffer
-    // holds lambda(t+1) at its end, so each such pair is captured once into a
-    // CUDA graph and replayed (about 5 launches per step otherwise).
-    auto segment = [&](int len, float* ln, float* lc, cudaStream_t s2) -> cudaError_t {
+    auto fields_of = [&](int i) { return adj_state(fields + kAdjStateVals * N * (size_t)i, N); };
+    // the forward fields of a segment's `len` states, stepping on from store[0]
+    // (the fields pass reads the state while it is in L2); with `end` also the
+    // step that ends the segment
+    auto recompute = [&](int len, bool end, cudaStream_t s2) -> cudaError_t {
         cudaError_t e = cudaSuccess;
-        for (int i = 0; i < len && e == cudaSuccess; ++i) e = step_into(store + sb * (size_t)i, store + sb * (size_t)(i + 1), s2);
-        for (int i = len - 1; i >= 0 && e == cudaSuccess; --i) {
-            e = fwd_on(store + sb * (size_t)i, s2);
-            if (e == cudaSuccess) e = launch_adj_backstep(G, A, ln, lc, part, acc, s2);
-            std::swap(ln, lc);
+        for (int i = 0; i < len && e == cudaSuccess; ++i) {
+            e = adj_forward(c, store + sb * (size_t)(i & 1), fields_of(i), s2);
+            if (e == cudaSuccess && (end || i + 1 < len)) e = step_of(i & 1, s2);
         }
         return e;
     };
+    // lambda(t0 + len) -> lambda(t0); E[en] holds lambda(t0 + len)
+    auto reverse = [&](int len, int en, cudaStream_t s2) -> cudaError_t {
+        cudaError_t e = cudaSuccess;
+        for (int i = len - 1; i >= 0 && e == cudaSuccess; --i, en ^= 1)
+            e = launch_adj_backstep(G, fields_of(i), t1, E[en], Mm[en], E[1 - en], Mm[1 - en], V, part, s2);
+        return e;
+    };
     struct SegGraphs {
-        std::vector<std::pair<long long, cudaGraphExec_t>> g;
+        cudaGraphExec_t g[2] = {nullptr, nullptr};  // by the E buffer that holds lambda at the segment's end
         ~SegGraphs()
         {
-            for (auto& p : g) cudaGraphExecDestroy(p.second);
+            for (cudaGraphExec_t x : g)
+                if (x) cudaGraphExecDestroy(x);
         }
     } graphs;
-    auto run_segment = [&](int len, float* ln, float* lc) -> cudaError_t {
-        const long long key = 2LL * len + (ln == lam ? 0 : 1);
-        for (auto& p : graphs.g)
-            if (p.first == key) return cudaGraphLaunch(p.second, st);
-        cudaGraph_t gr = nullptr;
-        cudaError_t e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) return e;
-        const cudaError_t e1 = segment(len, ln, lc, c->cap);
-        e = cudaStreamEndCapture(c->cap, &gr);
-        if (e1 != cudaSuccess) e = e1;
-        cudaGraphExec_t ex = nullptr;
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, gr, 0);
-        if (gr) cudaGraphDestroy(gr);
-        if (e != cudaSuccess) return e;
-        graphs.g.emplace_back(key, ex);
-        return cudaGraphLaunch(ex, st);
+    // The segments before the last are all ckpt_every long: their launches
+    // depend only on which E buffer holds lambda at their end, so with several
+    // of them each such sequence is captured once and replayed (capturing costs
+    // about as much as launching it twice).
+    auto segment = [&](int len, int en) -> cudaError_t {
+        if (nseg < 5) {
+            cudaError_t e = recompute(len, false, st);
+            return e == cudaSuccess ? reverse(len, en, st) : e;
+        }
+        if (!graphs.g[en]) {
+            cudaGraph_t gr = nullptr;
+            cudaError_t e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
+            if (e != cudaSuccess) return e;
+            cudaError_t e1 = recompute(len, false, c->cap);
+            if (e1 == cudaSuccess) e1 = reverse(len, en, c->cap);
+            e = cudaStreamEndCapture(c->cap, &gr);
+            if (e1 != cudaSuccess) e = e1;
+            if (e == cudaSuccess) e = cudaGraphInstantiate(&graphs.g[en], gr, 0);
+            if (gr) cudaGraphDestroy(gr);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaGraphLaunch(graphs.g[en], st);
     };
 
     // forward: a checkpoint at the start of every segment (with the step count,
     // which keys the 16-bit rounding dither, so the recompute replays it)
     std::vector<long long> ck_steps(nseg > 0 ? nseg : 1);
-    for (int s = 0; s < nseg; ++s) {
+    for (int s = 0; s + 1 < nseg; ++s) {
         ck_steps[s] = c->steps;
         LB_CUDA(c, cudaMemcpyAsync(ck + sb * (size_t)s, c->f[c->cur], sb, cudaMemcpyDeviceToDevice, st));
-        const int len = nsteps - s * ckpt_every < ckpt_every ? nsteps - s * ckpt_every : ckpt_every;
-        const int rc = lb_step(c, len);
+        const int rc = lb_step(c, ckpt_every);
         if (rc != LB_OK) return rc;
+    }
+    // the last segment steps with its forward fields kept, so it needs no recompute
+    const int llen = nseg > 0 ? nsteps - (nseg - 1) * ckpt_every : 0;
+    if (nseg > 0) {
+        LB_CUDA(c, cudaMemcpyAsync(store, c->f[c->cur], sb, cudaMemcpyDeviceToDevice, st));
+        LB_CUDA(c, recompute(llen, true, st));
+        c->cur ^= llen & 1;  // as lb_step leaves it
+        c->steps += llen;
+        LB_CUDA(c, cudaMemcpyAsync(c->f[c->cur], store + sb * (size_t)(llen & 1), sb, cudaMemcpyDeviceToDevice, st));
     }
     // observable of the final state and lambda(T) = dJ/dn(T)
     const double eps = 0.05;
-    float* lam_next = lam;
-    float* lam_cur = lam + 2 * Q * (size_t)N;
-    LB_CUDA(c, fwd(c->f[c->cur]));
-    LB_CUDA(c, launch_observable(c->nx, c->ny, c->nz, observable, eps, A.rho[0], A.rho[1], part, sums, lam_next, st));
-    LB_CUDA(c, cudaMemsetAsync(acc, 0, 2 * sizeof(double), st));
-    // backward, segment by segment: recompute the segment's states, then sweep them in reverse
-    for (int s = nseg - 1; s >= 0; --s) {
-        const int t0 = s * ckpt_every;
-        const int len = nsteps - t0 < ckpt_every ? nsteps - t0 : ckpt_every;
+    const AdjState last = fields_of(slen);
+    LB_CUDA(c, adj_forward(c, c->f[c->cur], last, st));
+    LB_CUDA(c, launch_observable(c->nx, c->ny, c->nz, observable, eps, last.rho, opart, sums, &E[0], st));
+    LB_CUDA(c, cudaMemsetAsync(part, 0, 2 * sizeof(double) * (size_t)blocks, st));
+    if (!t1) LB_CUDA(c, cudaMemsetAsync(Mm[0], 0, sizeof(float) * 2 * Q * N, st));
+    // backward, segment by segment: recompute the segment's forward fields, then sweep them in reverse
+    int en = 0;
+    if (nseg > 0) {
+        LB_CUDA(c, reverse(llen, en, st));
+        en ^= llen & 1;
+    }
+    for (int s = nseg - 2; s >= 0; --s) {
         LB_CUDA(c, cudaMemcpyAsync(store, ck + sb * (size_t)s, sb, cudaMemcpyDeviceToDevice, st));
         LB_CUDA(c, launch_clock_set(c->clock, (uint32_t)ck_steps[s], st));
-        LB_CUDA(c, run_segment(len, lam_next, lam_cur));
-        if (len & 1) std::swap(lam_next, lam_cur);
+        LB_CUDA(c, segment(ckpt_every, en));
+        en ^= ckpt_every & 1;
     }
     LB_CUDA(c, launch_clock_set(c->clock, (uint32_t)c->steps, st));
+    LB_CUDA(c, launch_rows_sum(part, blocks, acc, st));
     double h[3] = {0, 0, 0};
     LB_CUDA(c, cudaMemcpyAsync(h, acc, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
     LB_CUDA(c, cudaMemcpyAsync(h + 2, sums + 2, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1619,28 +1673,17 @@ extern "C" int lb_observable(lb_ctx* c, int observable, double* J)
 {
     if (!c || !J || observable < 0 || observable > 2) return fail(c, LB_ERR_ARG, "lb_observable: bad argument");
     if (c->general) return fail(c, LB_ERR_UNSUPPORTED, "lb_observable: planar walls only");
-    const long long N = (long long)c->nx * c->ny * c->nz;
+    const size_t N = (size_t)c->nx * c->ny * c->nz;
     AdjScratch M;
     float* aux = nullptr;
     double* dsc = nullptr;
-    LB_CUDA(c, M.alloc((void**)&aux, sizeof(float) * 10 * (size_t)N));
-    LB_CUDA(c, M.alloc((void**)&dsc, sizeof(double) * (2 * kAdjBlocks + 8)));
-    AdjFields A{};
-    float* q = aux;
-    for (int a = 0; a < 2; ++a) A.rho[a] = q, q += N;
-    for (int a = 0; a < 2; ++a) A.psi[a] = q, q += N;
-    for (int a = 0; a < 2; ++a)
-        for (int d = 0; d < 3; ++d) A.j[a][d] = q, q += N;
-    cudaError_t e;
-    switch (c->prec) {
-    case LB_F32: e = adj_forward_of<float>(c, c->f[c->cur], A, c->stream); break;
-    case LB_F16: e = adj_forward_of<__half>(c, c->f[c->cur], A, c->stream); break;
-    default: e = adj_forward_of<__nv_bfloat16>(c, c->f[c->cur], A, c->stream); break;
-    }
-    LB_CUDA(c, e);
-    LB_CUDA(c, launch_observable(c->nx, c->ny, c->nz, observable, 0.05, A.rho[0], A.rho[1], dsc,
-                                 dsc + 2 * kAdjBlocks, nullptr, c->stream));
-    LB_CUDA(c, cudaMemcpyAsync(J, dsc + 2 * kAdjBlocks + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    LB_CUDA(c, M.alloc((void**)&aux, sizeof(float) * kAdjStateVals * N));
+    LB_CUDA(c, M.alloc((void**)&dsc, sizeof(double) * (2 * kObsBlocks + 8)));
+    const AdjState A = adj_state(aux, N);
+    LB_CUDA(c, adj_forward(c, c->f[c->cur], A, c->stream));
+    LB_CUDA(c, launch_observable(c->nx, c->ny, c->nz, observable, 0.05, A.rho, dsc, dsc + 2 * kObsBlocks, nullptr,
+                                 c->stream));
+    LB_CUDA(c, cudaMemcpyAsync(J, dsc + 2 * kObsBlocks + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     LB_CUDA(c, cudaStreamSynchronize(c->stream));
     return LB_OK;
 }

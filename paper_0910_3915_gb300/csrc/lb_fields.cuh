@@ -31,29 +31,37 @@ struct Scratch {
     float* u[3];
 };
 
-// Dense FP32 fields of the adjoint (index x + nx*(y + ny*z)).
-struct AdjFields {
-    float* rho[2];   // forward: densities
-    float* psi[2];   // forward: psi (wall pseudo-density on solid nodes)
-    float* j[2][3];  // forward: momenta
-    float* rhob[2];  // adjoint of rho before the psi term
-    float* jb[2][3]; // adjoint of j
-    float* V[2][3];  // adjoint of the neighbour sum S^a: -g kappa psi^a Fbar^a
-    float* psib[2];  // adjoint of psi^a from the node's own force
+// Dense FP32 fields of the adjoint (index x + nx*(y + ny*z)), both components
+// of a node side by side.
+struct AdjState {  // forward: densities, psi (wall pseudo-density on solid nodes), momenta
+    float2 *rho, *psi, *j[3];
 };
+struct AdjE {  // adjoint of the populations, lambda_k = rb + c_k . j (+ M_k where tau != 1)
+    float2 *rb, *j[3];
+};
+struct AdjV {  // adjoint of the neighbour sum S^a, -g kappa psi^a Fbar^a, and of psi^a from the node's own force
+    float2 *v[3], *psib;
+};
+constexpr int kAdjStateVals = 10, kAdjEVals = 8, kAdjVVals = 8;  // floats a node
 struct AdjArgs {
     int nx, ny, nz;
     float gk, G[Q];  // G[k]: neighbour weight of link k (G[0] unused)
     float tau[2], omega[2];
     float eta[2];
 };
-constexpr int kAdjBlocks = 512;
+constexpr int kAdjThreads = 128;  // threads a block of the adjoint passes, one node each
+constexpr int kObsBlocks = 512;   // fixed grid of the observable's sums
 template <class S>
-cudaError_t launch_adj_forward(const Layout& L, const KParams& P, const S* f, const AdjFields& A, cudaStream_t st);
-cudaError_t launch_adj_backstep(const AdjArgs& G, const AdjFields& A, const float* lam_next, float* lam_cur,
-                                double* part, double* acc, cudaStream_t st);
-cudaError_t launch_observable(int nx, int ny, int nz, int obs, double eps, const float* rr, const float* rb,
-                              double* part, double* sums, float* lam, cudaStream_t st);
+cudaError_t launch_adj_forward(const Layout& L, const KParams& P, const S* f, const AdjState& A, cudaStream_t st);
+// one reverse step: E(t+1), M(t+1) -> E(t), M(t) (M only where tau != 1); adds the
+// wall gradient to the blocks' rows of part (2 doubles a block of kAdjThreads nodes)
+cudaError_t launch_adj_backstep(const AdjArgs& G, const AdjState& A, bool tau_one, const AdjE& En, const float* Mn,
+                                const AdjE& Ec, float* Mc, const AdjV& W, double* part, cudaStream_t st);
+// out[0..1] = the sums of nblocks rows of two doubles, in a fixed order
+cudaError_t launch_rows_sum(const double* part, int nblocks, double* out, cudaStream_t st);
+// J of the densities into sums[2], with E non-NULL also lambda(T); part: 2 kObsBlocks doubles
+cudaError_t launch_observable(int nx, int ny, int nz, int obs, double eps, const float2* rho, double* part,
+                              double* sums, const AdjE* E, cudaStream_t st);
 
 template <class S>
 cudaError_t launch_step(const StepArgs<S>& A, int tile_y, bool general, bool tau_one, cudaStream_t st);

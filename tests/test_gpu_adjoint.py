@@ -157,3 +157,24 @@ def test_autograd_function_chain_rule(lbsc):
     assert J.item() == J2
     assert math.isclose(w.grad.item(), g[1] - g[0], rel_tol=1e-12)
     lat.close()
+
+
+@pytest.mark.parametrize("tau", [(1.0, 1.0), (0.9, 1.15)])
+@pytest.mark.parametrize("ckpt", [1, 2, 3, 6, 13, 40])
+def test_adjoint_segments_change_nothing(lbsc, tau, ckpt):
+    """13 steps in 13, 7, 5, 3 and 1 segments (launched one by one and as replayed graphs, the last one shorter or
+    longer than none, odd and even lengths): the same gradient and J, and the state that plain stepping gives."""
+    nx, ny, nz = 35, 9, 7  # no multiple of a block, both walls next to each other's neighbours
+    rr, rb = W.droplet_fields(nx, ny, nz, 4.0, seed=2)
+    prm = dict(CONTACT, tau_r=tau[0], tau_b=tau[1], eta_wall_r=-0.04, eta_wall_b=0.04)
+
+    def run(every):
+        lat = lbsc.Lattice(rr, rb).set_params(**prm)
+        J, g = lat.step_backward(13, every, "com_soft")
+        return J, g, lat.step(2).populations()
+
+    J0, g0, n0 = run(100)
+    J, g, n = run(ckpt)
+    assert J == J0 and np.array_equal(g, g0)
+    assert np.array_equal(n, n0)
+    assert np.array_equal(n, lbsc.Lattice(rr, rb).set_params(**prm).step(15).populations())
