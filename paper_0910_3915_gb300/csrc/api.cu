@@ -1695,9 +1695,15 @@ static cudaError_t pressure_field_of(lb_ctx* c, double* out)
     return launch_pressure_field<S>(field_args(c), (const S*)c->f[c->cur], c->W, out, c->stream);
 }
 template <class S>
-static cudaError_t pressure_planes_of(lb_ctx* c, double* out)
+static cudaError_t pressure_planes_of(lb_ctx* c, int split, double* part, double* out)
 {
-    return launch_pressure_planes<S>(field_args(c), (const S*)c->f[c->cur], c->W, out, c->stream);
+    return launch_pressure_planes<S>(field_args(c), (const S*)c->f[c->cur], c->W, split, part, out, c->stream);
+}
+template <class S>
+static cudaError_t pressure_radial_of(lb_ctx* c, const double* centre, double dr, int nbins, double zmin,
+                                      unsigned long long* out)
+{
+    return launch_pressure_radial<S>(field_args(c), (const S*)c->f[c->cur], c->W, centre, dr, nbins, zmin, out, c->stream);
 }
 
 extern "C" int lb_pressure_tensor(lb_ctx* c, double* P)
@@ -1707,7 +1713,7 @@ extern "C" int lb_pressure_tensor(lb_ctx* c, double* P)
     AdjScratch M;
     double* d = nullptr;
     LB_CUDA(c, M.alloc((void**)&d, 6 * N * sizeof(double)));
-    LB_CUDA(c, dispatch_fields(c, true));
+    LB_CUDA(c, dispatch_fields(c, false));
     switch (c->prec) {
     case LB_F32: LB_CUDA(c, pressure_field_of<float>(c, d)); break;
     case LB_F16: LB_CUDA(c, pressure_field_of<__half>(c, d)); break;
@@ -1722,14 +1728,22 @@ extern "C" int lb_pressure_profile(lb_ctx* c, double* prof, double* gamma_sum)
 {
     if (!c || !prof) return fail(c, LB_ERR_ARG, "lb_pressure_profile: NULL argument");
     const int nz = c->nz;
+    // about 8 blocks an SM, none below 128 nodes: ranges of a plane in as many blocks as that leaves
+    const long long nxy = (long long)c->nx * c->ny;
+    long long split = (8LL * c->nsm + nz - 1) / nz;
+    const long long smax = (nxy + kPressThreads - 1) / kPressThreads;
+    split = split > smax ? smax : split;
+    // the sums live in the context's partials area, or (very tall lattices) in memory of their own
+    const size_t need = (size_t)nz * 8 * (size_t)(split + 1);
     AdjScratch M;
-    double* d = nullptr;
-    LB_CUDA(c, M.alloc((void**)&d, (size_t)nz * 8 * sizeof(double)));
-    LB_CUDA(c, dispatch_fields(c, true));
+    double* d = c->part;
+    if (need > (size_t)kPartRows * kAngleVals) LB_CUDA(c, M.alloc((void**)&d, need * sizeof(double)));
+    double* part = d + (size_t)nz * 8;
+    LB_CUDA(c, dispatch_fields(c, false));
     switch (c->prec) {
-    case LB_F32: LB_CUDA(c, pressure_planes_of<float>(c, d)); break;
-    case LB_F16: LB_CUDA(c, pressure_planes_of<__half>(c, d)); break;
-    default: LB_CUDA(c, pressure_planes_of<__nv_bfloat16>(c, d)); break;
+    case LB_F32: LB_CUDA(c, pressure_planes_of<float>(c, (int)split, part, d)); break;
+    case LB_F16: LB_CUDA(c, pressure_planes_of<__half>(c, (int)split, part, d)); break;
+    default: LB_CUDA(c, pressure_planes_of<__nv_bfloat16>(c, (int)split, part, d)); break;
     }
     LB_CUDA(c, cudaMemcpyAsync(prof, d, (size_t)nz * 8 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     LB_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -1753,12 +1767,14 @@ extern "C" int lb_pressure_radial(lb_ctx* c, const double* centre, double dr, in
     if (!c || !centre || !bins || !(dr > 0) || nbins < 1 || nbins > kRadialBinsMax || !std::isfinite(zmin) ||
         !std::isfinite(r_max) || !std::isfinite(centre[0]) || !std::isfinite(centre[1]) || !std::isfinite(centre[2]))
         return fail(c, LB_ERR_ARG, "lb_pressure_radial: bad argument (dr > 0, 1 <= nbins <= 1024, finite centre)");
-    AdjScratch M;
-    unsigned long long* d = nullptr;
-    LB_CUDA(c, M.alloc((void**)&d, (size_t)nbins * 4 * sizeof(unsigned long long)));
-    LB_CUDA(c, dispatch_fields(c, true));
-    LB_CUDA(c, launch_pressure_radial(field_args(c), c->f[c->cur], c->prec, c->W, centre, dr, nbins, zmin, d,
-                                      c->stream));
+    static_assert((size_t)kRadialBinsMax * 4 <= (size_t)kPartRows * kAngleVals, "the bins fit the partials area");
+    unsigned long long* d = (unsigned long long*)c->part;
+    LB_CUDA(c, dispatch_fields(c, false));
+    switch (c->prec) {
+    case LB_F32: LB_CUDA(c, pressure_radial_of<float>(c, centre, dr, nbins, zmin, d)); break;
+    case LB_F16: LB_CUDA(c, pressure_radial_of<__half>(c, centre, dr, nbins, zmin, d)); break;
+    default: LB_CUDA(c, pressure_radial_of<__nv_bfloat16>(c, centre, dr, nbins, zmin, d)); break;
+    }
     std::vector<unsigned long long> h((size_t)nbins * 4);
     LB_CUDA(c, cudaMemcpyAsync(h.data(), d, h.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
     LB_CUDA(c, cudaStreamSynchronize(c->stream));

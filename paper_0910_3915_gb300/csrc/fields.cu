@@ -22,27 +22,6 @@ __device__ __forceinline__ double warp_max(double v)
     return v;
 }
 
-// Reduce NV values per thread into out[blockIdx.x*NV + i]; entries listed in
-// `is_max` are max-reduced, all others summed. blockDim.x must be kRedThreads.
-template <int NV>
-__device__ __forceinline__ void block_reduce(double (&acc)[NV], uint32_t is_max, double* out)
-{
-    __shared__ double sh[kRedThreads / 32][NV];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        const double v = ((is_max >> i) & 1u) ? warp_max(acc[i]) : warp_sum(acc[i]);
-        if (lane == 0) sh[warp][i] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        const int i = threadIdx.x;
-        double v = sh[0][i];
-        for (int w = 1; w < kRedThreads / 32; ++w) v = ((is_max >> i) & 1u) ? fmax(v, sh[w][i]) : v + sh[w][i];
-        out[(long long)blockIdx.x * NV + i] = v;
-    }
-}
-
 // Sum (or max) nrows partial rows of NV values: block v reduces value v,
 // thread t taking rows t, t + 256, ... in order, then a fixed shuffle tree per
 // warp and the warps in order. Launched as NV blocks of 256 threads.
@@ -81,11 +60,15 @@ static int grid_for(long long n, int threads, int cap)
 }
 
 template <class S>
-__device__ __forceinline__ float decode(const S* p, int k, float ref)
+__device__ __forceinline__ float decode_val(float v, int k, float ref)
 {
-    const float v = Codec<S>::load(p);
     if constexpr (Codec<S>::kDeviation) return zeta(k) * (ref + v);
     else return v;
+}
+template <class S>
+__device__ __forceinline__ float decode(const S* p, int k, float ref)
+{
+    return decode_val<S>(Codec<S>::load(p), k, ref);
 }
 
 // both components' n_k of one node from their paired storage
@@ -236,20 +219,32 @@ __global__ void __launch_bounds__(kRedThreads) cons_kernel(FieldArgs F, const S*
 }
 
 // ---------------------------------------------------------------- moment fields
-// rho^r, rho^b, total j and psi of every node (psi = wall pseudo-density on solid)
+// rho^r, rho^b, total j and psi of every node (psi = wall pseudo-density on
+// solid). Bound by the read of the populations and the write of the fields. A
+// 16-bit velocity's two components come in one load (256x256x128 BF16: 136
+// us, 178 with one load each); FP32 takes them apart, the second from L1, with
+// 32 registers instead of 48 (128^3: 54 us against 64).
 template <class S>
-__global__ void fields_kernel(FieldArgs F, const S* __restrict__ f, Scratch W)
+__global__ void __launch_bounds__(kRedThreads) fields_kernel(FieldArgs F, const S* __restrict__ f, Scratch W)
 {
-    const long long N = (long long)F.L.nx * F.L.ny * F.L.nz;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % F.L.nx), y = (int)((i / F.L.nx) % F.L.ny), z = (int)(i / ((long long)F.L.nx * F.L.ny));
+    const unsigned nx = (unsigned)F.L.nx, nxy = nx * (unsigned)F.L.ny, N = nxy * (unsigned)F.L.nz;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        const int z = (int)(i / nxy), y = (int)((i - z * nxy) / nx), x = (int)(i - z * nxy - y * nx);
         const long long off = F.L.off(x, y, z);
         float rho[2] = {0.f, 0.f}, j[3] = {0.f, 0.f, 0.f};
         const bool solid = node_solid(F, x, y, z, off);
         if (!solid) {
+            float2 v[Q];
+            if constexpr (sizeof(S) == 2)
+#pragma unroll
+                for (int k = 0; k < Q; ++k) v[k] = Codec<S>::load2(f + F.L.at(0, k, off));
+#pragma unroll
             for (int a = 0; a < 2; ++a)
+#pragma unroll
                 for (int k = 0; k < Q; ++k) {
-                    const float n = decode<S>(f + F.L.at(a, k, off), k, F.P.ref[a]);
+                    float n;
+                    if constexpr (sizeof(S) == 2) n = decode_val<S>(a ? v[k].y : v[k].x, k, F.P.ref[a]);
+                    else n = Codec<S>::load(f + F.L.at(a, k, off));
                     rho[a] += n;
                     j[0] += cx(k) * n;
                     j[1] += cy(k) * n;
@@ -263,34 +258,44 @@ __global__ void fields_kernel(FieldArgs F, const S* __restrict__ f, Scratch W)
     }
 }
 
-// u = (j + F/2) / (rho_r + rho_b), F the total Shan-Chen force (Eq. SCforce)
-__global__ void velocity_kernel(FieldArgs F, Scratch W)
+// u = (j + F/2) / (rho_r + rho_b) of the fluid node (x, y, z) at index i, F the
+// total Shan-Chen force (Eq. SCforce)
+__device__ __forceinline__ void node_velocity(const FieldArgs& F, const Scratch& W, int x, int y, int z, unsigned i,
+                                              float (&u)[3])
 {
     const int nx = F.L.nx, ny = F.L.ny, nz = F.L.nz;
-    const long long N = (long long)nx * ny * nz;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % nx), y = (int)((i / nx) % ny), z = (int)(i / ((long long)nx * ny));
-        const long long off = F.L.off(x, y, z);
-        const float tot = W.rho[0][i] + W.rho[1][i];
-        float u[3] = {0.f, 0.f, 0.f};
-        if (!node_solid(F, x, y, z, off) && tot > 0.f) {
-            float Ft[3] = {0.f, 0.f, 0.f};
-            for (int a = 0; a < 2; ++a) {
-                float s[3] = {0.f, 0.f, 0.f};
-                for (int k = 1; k < Q; ++k) {
-                    const long long ip = (long long)wrapi(x + cx(k), nx) +
-                                         (long long)nx * (wrapi(y + cy(k), ny) + (long long)ny * wrapi(z + cz(k), nz));
-                    const float G = is_axis(k) ? F.P.Gax : F.P.Gdi;
-                    const float ps = W.psi[1 - a][ip];
-                    s[0] += G * ps * cx(k);
-                    s[1] += G * ps * cy(k);
-                    s[2] += G * ps * cz(k);
-                }
-                const float pre = -F.P.gk * W.psi[a][i];
-                for (int d = 0; d < 3; ++d) Ft[d] += pre * s[d];
-            }
-            for (int d = 0; d < 3; ++d) u[d] = (W.j[d][i] + 0.5f * Ft[d]) / tot;
+    const int xo[3] = {wrapi(x - 1, nx), x, wrapi(x + 1, nx)};
+    const int yo[3] = {nx * wrapi(y - 1, ny), nx * y, nx * wrapi(y + 1, ny)};
+    const int zo[3] = {nx * ny * wrapi(z - 1, nz), nx * ny * z, nx * ny * wrapi(z + 1, nz)};
+    const float tot = W.rho[0][i] + W.rho[1][i];
+    u[0] = u[1] = u[2] = 0.f;
+    if (!(tot > 0.f)) return;
+    float Ft[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+        float s[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int k = 1; k < Q; ++k) {
+            const int ip = xo[cx(k) + 1] + yo[cy(k) + 1] + zo[cz(k) + 1];
+            const float G = is_axis(k) ? F.P.Gax : F.P.Gdi;
+            const float ps = W.psi[1 - a][ip];
+            s[0] += G * ps * cx(k);
+            s[1] += G * ps * cy(k);
+            s[2] += G * ps * cz(k);
         }
+        const float pre = -F.P.gk * W.psi[a][i];
+        for (int d = 0; d < 3; ++d) Ft[d] += pre * s[d];
+    }
+    for (int d = 0; d < 3; ++d) u[d] = (W.j[d][i] + 0.5f * Ft[d]) / tot;
+}
+
+__global__ void __launch_bounds__(kRedThreads) velocity_kernel(FieldArgs F, Scratch W)
+{
+    const unsigned nx = (unsigned)F.L.nx, nxy = nx * (unsigned)F.L.ny, N = nxy * (unsigned)F.L.nz;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        const int z = (int)(i / nxy), y = (int)((i - z * nxy) / nx), x = (int)(i - z * nxy - y * nx);
+        float u[3] = {0.f, 0.f, 0.f};
+        if (!node_solid(F, x, y, z, F.L.off(x, y, z))) node_velocity(F, W, x, y, z, i, u);
         for (int d = 0; d < 3; ++d) W.u[d][i] = u[d];
     }
 }
@@ -506,7 +511,7 @@ __global__ void __launch_bounds__(kRedThreads) angle_kernel(FieldArgs F, Scratch
 }
 
 // ---------------------------------------------------------------- pressure tensor
-// Pressure tensor of Sec. 4.1 at a node, in FP64 from the FP32 fields:
+// Pressure tensor of Sec. 4.1 at a node:
 //   P_ij = sum_a sum_k (c_ki - u_i)(c_kj - u_j) n_k^a
 //        + 1/4 sum over the two ordered component pairs (a, abar) of
 //          g kappa sum_k G_k [psi^a(x) psi^abar(x+c_k) + psi^abar(x) psi^a(x+c_k)] c_ki c_kj,
@@ -514,16 +519,77 @@ __global__ void __launch_bounds__(kRedThreads) angle_kernel(FieldArgs F, Scratch
 // pseudo-density (the force's reading of the wall). Both ordered pairs give the
 // same bracket, so the interaction is 1/2 g kappa sum_k G_k [..] c_ki c_kj.
 // Components xx, yy, zz, xy, xz, yz; zero on solid nodes.
+//
+// FP64 runs at a sixtieth of the FP32 rate on this GPU, so the sums are taken
+// in pairs of FP32 numbers (Dekker 1971, Knuth's two-sum): a value is h + l
+// with l far below h, a sum carries the rounding error of h in l. That keeps
+// about 46 bits of the sums over exact FP32 inputs, 20 more than the stored
+// populations hold. With u common to both components the kinetic term is
+//   S_ij - u_i K_j - u_j J_i,  S = sum c c m,  J = sum c m,  K = J - u R,
+//   R = sum m,  m_k = n_k^r + n_k^b,
+// and S, J need the sums and differences of opposite velocities only. A node
+// whose result is not finite is taken again in FP64, so that infinities and
+// NaN come out as they always did.
+struct Two {
+    float h, l;
+};
+__device__ __forceinline__ Two two(float a) { return Two{a, 0.f}; }
+__device__ __forceinline__ Two two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return Two{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+// l may grow to a few roundings of h: normalised by norm2 before a product
+__device__ __forceinline__ Two operator+(Two a, Two b)
+{
+    const Two s = two_sum(a.h, b.h);
+    return Two{s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ Two operator-(Two a) { return Two{-a.h, -a.l}; }
+__device__ __forceinline__ Two operator-(Two a, Two b) { return a + (-b); }
+__device__ __forceinline__ Two norm2(Two a)
+{
+    const float s = __fadd_rn(a.h, a.l);
+    return Two{s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
+}
+__device__ __forceinline__ Two mul2f(Two a, float f)  // a normalised
+{
+    const float p = __fmul_rn(a.h, f);
+    return Two{p, __fmaf_rn(a.l, f, __fmaf_rn(a.h, f, -p))};
+}
+__device__ __forceinline__ Two mul22(Two a, Two b)  // both normalised
+{
+    const float p = __fmul_rn(a.h, b.h);
+    return Two{p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ double to_f64(Two a) { return (double)a.h + (double)a.l; }
+
+// S_ij of values s[k] = v_k + v_kbar (k odd; entry (k - 1) / 2): xx, yy, zz, xy, xz, yz
+__device__ __forceinline__ void second_moment(const Two (&s)[9], Two (&S)[6], Two& XY, Two& XZ, Two& YZ)
+{
+    XY = s[3] + s[4];
+    XZ = s[5] + s[6];
+    YZ = s[7] + s[8];
+    S[0] = (s[0] + XY) + XZ;
+    S[1] = (s[1] + XY) + YZ;
+    S[2] = (s[2] + XZ) + YZ;
+    S[3] = s[3] - s[4];
+    S[4] = s[5] - s[6];
+    S[5] = s[7] - s[8];
+}
+
+// the tensor in FP64, operation by operation
 template <class S>
-__device__ bool node_pressure(const FieldArgs& F, const S* __restrict__ f, const Scratch& W, int x, int y, int z,
-                              double (&P)[6])
+__device__ __noinline__ void node_pressure_f64(const FieldArgs& F, const S* __restrict__ f, const Scratch& W, int x, int y,
+                                               int z, double* P)
 {
     const int nx = F.L.nx, ny = F.L.ny, nz = F.L.nz;
     for (int c = 0; c < 6; ++c) P[c] = 0.0;
     const long long off = F.L.off(x, y, z);
-    if (node_solid(F, x, y, z, off)) return false;
     const long long i = (long long)x + (long long)nx * (y + (long long)ny * z);
-    const double u[3] = {W.u[0][i], W.u[1][i], W.u[2][i]};
+    float uf[3];
+    node_velocity(F, W, x, y, z, (unsigned)i, uf);
+    const double u[3] = {uf[0], uf[1], uf[2]};
     for (int a = 0; a < 2; ++a)
         for (int k = 0; k < Q; ++k) {
             const double n = decode<S>(f + F.L.at(a, k, off), k, F.P.ref[a]);
@@ -551,41 +617,161 @@ __device__ bool node_pressure(const FieldArgs& F, const S* __restrict__ f, const
     }
     const double h = 0.5 * (double)F.P.gk;
     for (int c = 0; c < 6; ++c) P[c] += h * I[c];
-    return true;
+}
+
+// the tensor at the fluid node (x, y, z), normalised; false where a component
+// is not finite (the caller then takes node_pressure_f64)
+template <class S>
+__device__ __forceinline__ bool node_pressure(const FieldArgs& F, const S* __restrict__ f, const Scratch& W, int x, int y,
+                                              int z, Two (&P)[6])
+{
+    const int nx = F.L.nx, ny = F.L.ny, nz = F.L.nz;
+    const long long off = F.L.off(x, y, z);
+    const int i = x + nx * (y + ny * z);
+    float u[3];
+    node_velocity(F, W, x, y, z, (unsigned)i, u);
+    const float ref[2] = {F.P.ref[0], F.P.ref[1]};
+    Two XY, XZ, YZ;
+    {
+        Two s[9], d[9];
+        auto m = [&](int k) {
+            float n0, n1;
+            decode2<S>(f + F.L.at(0, k, off), k, ref, n0, n1);
+            return two_sum(n0, n1);
+        };
+#pragma unroll
+        for (int p = 0; p < 9; ++p) {
+            const Two a = m(2 * p + 1), b = m(2 * p + 2);
+            s[p] = a + b;
+            d[p] = a - b;
+        }
+        second_moment(s, P, XY, XZ, YZ);
+        const Two R = norm2(((m(0) + s[0]) + (s[1] + s[2])) + ((XY + XZ) + YZ));
+        // pairs 3.. are (1,1,0), (1,-1,0), (1,0,1), (1,0,-1), (0,1,1), (0,1,-1)
+        const Two J[3] = {norm2((d[0] + (d[3] + d[4])) + (d[5] + d[6])), norm2((d[1] + (d[3] - d[4])) + (d[7] + d[8])),
+                          norm2((d[2] + (d[5] - d[6])) + (d[7] - d[8]))};
+        Two K[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) K[q] = norm2(J[q] - mul2f(R, u[q]));
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const int a = c < 3 ? c : (c < 5 ? 0 : 1), b = c < 3 ? c : (c == 3 ? 1 : 2);
+            P[c] = P[c] - (mul2f(K[b], u[a]) + mul2f(J[a], u[b]));
+        }
+    }
+    const int xo[3] = {wrapi(x - 1, nx), x, wrapi(x + 1, nx)};
+    const int yo[3] = {nx * wrapi(y - 1, ny), nx * y, nx * wrapi(y + 1, ny)};
+    const int zo[3] = {nx * ny * wrapi(z - 1, nz), nx * ny * z, nx * ny * wrapi(z + 1, nz)};
+    const float h = 0.5f * F.P.gk;  // exact
+    Two I[6];
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+        Two s[9], T[6];
+#pragma unroll
+        for (int p = 0; p < 9; ++p) {
+            const int k = 2 * p + 1;
+            const float v0 = W.psi[1 - a][xo[cx(k) + 1] + yo[cy(k) + 1] + zo[cz(k) + 1]];
+            const float v1 = W.psi[1 - a][xo[1 - cx(k)] + yo[1 - cy(k)] + zo[1 - cz(k)]];
+            const float G = p < 3 ? F.P.Gax : F.P.Gdi;  // 1 or 2: exact
+            s[p] = two_sum(__fmul_rn(G, v0), __fmul_rn(G, v1));
+        }
+        second_moment(s, T, XY, XZ, YZ);
+        const float own = W.psi[a][i];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const Two t = mul2f(norm2(T[c]), own);
+            I[c] = a ? I[c] + t : t;
+        }
+    }
+    bool finite = true;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        P[c] = norm2(P[c] + mul2f(norm2(I[c]), h));
+        finite = finite && isfinite(P[c].h) && isfinite(P[c].l);
+    }
+    return finite;
 }
 
 // every node: P[c*N + i] (FP64)
 template <class S>
-__global__ void pressure_field_kernel(FieldArgs F, const S* __restrict__ f, Scratch W, double* __restrict__ out)
+__global__ void __launch_bounds__(kPressThreads) pressure_field_kernel(FieldArgs F, const S* __restrict__ f, Scratch W,
+                                                                       double* __restrict__ out)
 {
-    const int nx = F.L.nx, ny = F.L.ny, nz = F.L.nz;
-    const long long N = (long long)nx * ny * nz;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % nx), y = (int)((i / nx) % ny), z = (int)(i / ((long long)nx * ny));
-        double P[6];
-        node_pressure<S>(F, f, W, x, y, z, P);
-        for (int c = 0; c < 6; ++c) out[c * N + i] = P[c];
+    const unsigned nx = (unsigned)F.L.nx, nxy = nx * (unsigned)F.L.ny, N = nxy * (unsigned)F.L.nz;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        const int z = (int)(i / nxy), y = (int)((i - z * nxy) / nx), x = (int)(i - z * nxy - y * nx);
+        double D[6] = {0, 0, 0, 0, 0, 0};
+        if (!node_solid(F, x, y, z, F.L.off(x, y, z))) {
+            Two P[6];
+            if (node_pressure<S>(F, f, W, x, y, z, P)) {
+                for (int c = 0; c < 6; ++c) D[c] = to_f64(P[c]);
+            } else {
+                node_pressure_f64<S>(F, f, W, x, y, z, D);
+            }
+        }
+        for (int c = 0; c < 6; ++c) out[(size_t)c * N + i] = D[c];
     }
 }
 
-// one block per z plane: sums over the plane's fluid nodes of the six
-// components, phi = rho_r - rho_b and the count -> out[z*8 + v]
+// Sums over the fluid nodes of a plane (blockIdx.x) and a range of its nodes
+// (one of `split` equal ones, blockIdx.y) of the six components, phi = rho_r -
+// rho_b and the count -> out[(z * split + range) * 8 + v]. A thread sums its
+// nodes in FP32 pairs (as node_pressure), then FP64 across threads.
+// Bound by the pairs' arithmetic (2180 instructions a node at half the issue rate, five blocks an SM): 110 us at 96^3; the
+// sums in FP64, one block a plane, took 1480.
 template <class S>
-__global__ void __launch_bounds__(kRedThreads) pressure_plane_kernel(FieldArgs F, const S* __restrict__ f, Scratch W,
-                                                                     double* __restrict__ out)
+__global__ void __launch_bounds__(kPressThreads, 5) pressure_plane_kernel(FieldArgs F, const S* __restrict__ f, Scratch W,
+                                                                       int split, double* __restrict__ out)
 {
-    const int nx = F.L.nx, ny = F.L.ny, z = blockIdx.x;
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int c = threadIdx.x; c < nx * ny; c += blockDim.x) {
-        const int x = c % nx, y = c / nx;
-        double P[6];
-        if (!node_pressure<S>(F, f, W, x, y, z, P)) continue;
-        const long long i = (long long)c + (long long)nx * ny * z;
-        for (int v = 0; v < 6; ++v) acc[v] += P[v];
-        acc[6] += (double)W.rho[0][i] - (double)W.rho[1][i];
-        acc[7] += 1.0;
+    const int nx = F.L.nx, nxy = nx * F.L.ny, z = blockIdx.x;
+    const int lo = (int)((long long)blockIdx.y * nxy / split), hi = (int)((long long)(blockIdx.y + 1) * nxy / split);
+    Two sum[7];
+    for (int v = 0; v < 7; ++v) sum[v] = two(0.f);
+    double odd[6] = {0, 0, 0, 0, 0, 0};  // nodes taken in FP64
+    int count = 0;
+    for (int c = lo + threadIdx.x; c < hi; c += kPressThreads) {
+        const int y = c / nx, x = c - y * nx;
+        if (node_solid(F, x, y, z, F.L.off(x, y, z))) continue;
+        const int i = c + nxy * z;
+        Two P[6];
+        if (node_pressure<S>(F, f, W, x, y, z, P)) {
+#pragma unroll
+            for (int v = 0; v < 6; ++v) sum[v] = norm2(sum[v] + P[v]);
+        } else {
+            double D[6];
+            node_pressure_f64<S>(F, f, W, x, y, z, D);
+            for (int v = 0; v < 6; ++v) odd[v] += D[v];
+        }
+        sum[6] = norm2(sum[6] + two_sum(W.rho[0][i], -W.rho[1][i]));
+        ++count;
     }
-    block_reduce<8>(acc, 0u, out);
+    double acc[8];
+#pragma unroll
+    for (int v = 0; v < 7; ++v) acc[v] = to_f64(sum[v]) + (v < 6 ? odd[v] : 0.0);
+    acc[7] = (double)count;
+    __shared__ double sh[kPressThreads / 32][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+        const double t = warp_sum(acc[v]);
+        if (lane == 0) sh[warp][v] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        double t = 0;
+        for (int w = 0; w < kPressThreads / 32; ++w) t += sh[w][threadIdx.x];
+        out[((size_t)z * split + blockIdx.y) * 8 + threadIdx.x] = t;
+    }
+}
+
+// out[z*8 + v] = the sum of plane z's `split` rows, in order
+__global__ void plane_rows_kernel(const double* __restrict__ part, int nz, int split, double* __restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nz * 8) return;
+    double t = 0;
+    for (int r = 0; r < split; ++r) t += part[((size_t)(i / 8) * split + r) * 8 + i % 8];
+    out[i] = t;
 }
 
 // Radial bins about a centre: per fluid node with z >= zmin at distance
@@ -594,49 +780,106 @@ __global__ void __launch_bounds__(kRedThreads) pressure_plane_kernel(FieldArgs F
 // P_T = (tr P - P_N)/2, phi and 1. Sums are kept in 64-bit fixed point
 // (units of 2^-30) so that the atomic accumulation is exact and the result
 // does not depend on the order the nodes are added in.
-__global__ void __launch_bounds__(kRedThreads) pressure_radial_kernel(FieldArgs F, const void* f, int prec, Scratch W,
-                                                                      double cxx, double cyy, double czz, double dr,
-                                                                      int nbins, double zmin,
-                                                                      unsigned long long* __restrict__ out)
+// The bin comes from an FP32 root of the FP64 r^2; only where that lies within
+// its rounding of a bin's edge is it taken from the FP64 root and quotient. A
+// block gathers its nodes' sums in shared memory as 32-bit words (the low 16
+// and the high bits of a value apart: 64-bit adds in shared memory are loops)
+// and adds them to the global bins at its end; a value too large for that
+// goes to the global bins at once.
+// As the plane sums, plus about 30 FP64 operations a node for the radius and the split into words: 155 us at 96^3, 1230 with
+// the tensor, three divisions and 64-bit shared-memory adds in FP64.
+constexpr int kRadialNodes = 32000;  // most nodes a block takes: its 32-bit sums cannot overflow (below 2^15 nodes of 2^16)
+
+template <class S>
+__global__ void __launch_bounds__(kPressThreads, 5) pressure_radial_kernel(FieldArgs F, const S* __restrict__ f, Scratch W,
+                                                                        double cxx, double cyy, double czz, double dr,
+                                                                        int nbins, double zmin, unsigned per,
+                                                                        unsigned long long* __restrict__ out)
 {
-    __shared__ unsigned long long sh[kRadialBinsMax * 4];
-    for (int b = threadIdx.x; b < nbins * 4; b += blockDim.x) sh[b] = 0ull;
+    extern __shared__ unsigned radial_sh[];  // [nbins][7]: low and high words of the three sums, count
+    for (int b = threadIdx.x; b < nbins * 7; b += kPressThreads) radial_sh[b] = 0u;
     __syncthreads();
     const int nx = F.L.nx, ny = F.L.ny, nz = F.L.nz;
-    const long long N = (long long)nx * ny * nz;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % nx), y = (int)((i / nx) % ny), z = (int)(i / ((long long)nx * ny));
+    const unsigned nxy = (unsigned)nx * (unsigned)ny, N = nxy * (unsigned)nz;
+    const unsigned lo = blockIdx.x * per, hi = N - lo < per ? N : lo + per;
+    const float idr = (float)(1.0 / dr);
+    const bool plain_dr = dr > 1e-6 && dr < 1e6;
+    for (unsigned i = lo + threadIdx.x; i < hi; i += kPressThreads) {
+        const int z = (int)(i / nxy), y = (int)((i - z * nxy) / (unsigned)nx), x = (int)(i - z * nxy - y * nx);
         if (z < zmin) continue;
         double d[3] = {x - cxx, y - cyy, z - czz};
-        d[0] -= nx * rint(d[0] / nx);
-        d[1] -= ny * rint(d[1] / ny);
-        if (F.general) d[2] -= nz * rint(d[2] / nz);
-        const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-        if (!(r > 0)) continue;
-        const double bf = floor(r / dr);
-        if (bf >= nbins) continue;
-        double P[6];
-        bool fluid;
-        if (prec == 0) fluid = node_pressure<float>(F, (const float*)f, W, x, y, z, P);
-        else if (prec == 1) fluid = node_pressure<__half>(F, (const __half*)f, W, x, y, z, P);
-        else fluid = node_pressure<__nv_bfloat16>(F, (const __nv_bfloat16*)f, W, x, y, z, P);
-        if (!fluid) continue;
-        const double n[3] = {d[0] / r, d[1] / r, d[2] / r};
-        const double T[3][3] = {{P[0], P[3], P[4]}, {P[3], P[1], P[5]}, {P[4], P[5], P[2]}};
-        double pn = 0;
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) pn += n[a] * T[a][b] * n[b];
-        const double pt = 0.5 * (P[0] + P[1] + P[2] - pn);
+        // v - n rint(v / n): rint is 0 up to |v| = n / 2 (a tie goes to even), where no quotient is needed
+        auto image = [](double v, int n) { return 2 * fabs(v) <= (double)n ? v : v - n * rint(v / n); };
+        d[0] = image(d[0], nx);
+        d[1] = image(d[1], ny);
+        if (F.general) d[2] = image(d[2], nz);
+        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        if (!(r2 > 0)) continue;
+        const float q = sqrtf((float)r2) * idr;  // r / dr within 3e-7 of itself for the moderate r2 and dr that `fast` asks for
+        const bool fast = plain_dr && r2 > 1e-12 && r2 < 1e12;
+        float bf = floorf(q);
+        if (!fast || fabsf(q - rintf(q)) <= 1e-6f * q) {
+            const double be = floor(sqrt(r2) / dr);
+            if (be >= nbins) continue;
+            bf = (float)be;
+        }
+        if (!(bf < (float)nbins)) continue;
+        if (node_solid(F, x, y, z, F.L.off(x, y, z))) continue;
+        Two P[6];
+        long long v[3];
         const double phi = (double)W.rho[0][i] - (double)W.rho[1][i];
+        if (node_pressure<S>(F, f, W, x, y, z, P)) {
+            // n.P.n = d.P.d / r^2 in FP32 pairs: d_i as a pair, products of pairs
+            Two e[3];
+#pragma unroll
+            for (int q3 = 0; q3 < 3; ++q3) {
+                e[q3].h = (float)d[q3];
+                e[q3].l = (float)(d[q3] - (double)e[q3].h);
+            }
+            const Two off = (norm2(mul22(P[3], norm2(mul22(e[0], e[1])))) + mul22(P[4], norm2(mul22(e[0], e[2])))) +
+                            mul22(P[5], norm2(mul22(e[1], e[2])));
+            const Two dia = (mul22(P[0], norm2(mul22(e[0], e[0]))) + mul22(P[1], norm2(mul22(e[1], e[1])))) +
+                            mul22(P[2], norm2(mul22(e[2], e[2])));
+            const double num = to_f64(dia + (off + off));
+            const double pn = num / r2;
+            const double tr = to_f64((P[0] + P[1]) + P[2]);
+            v[0] = __double2ll_rn(pn * kRadialFix);
+            v[1] = __double2ll_rn(0.5 * (tr - pn) * kRadialFix);
+        } else {
+            double D[6];
+            node_pressure_f64<S>(F, f, W, x, y, z, D);
+            const double r = sqrt(r2);
+            const double n[3] = {d[0] / r, d[1] / r, d[2] / r};
+            const double T[3][3] = {{D[0], D[3], D[4]}, {D[3], D[1], D[5]}, {D[4], D[5], D[2]}};
+            double pn = 0;
+            for (int a = 0; a < 3; ++a)
+                for (int b = 0; b < 3; ++b) pn += n[a] * T[a][b] * n[b];
+            v[0] = __double2ll_rn(pn * kRadialFix);
+            v[1] = __double2ll_rn(0.5 * (D[0] + D[1] + D[2] - pn) * kRadialFix);
+        }
+        v[2] = __double2ll_rn(phi * kRadialFix);
         const int b = (int)bf;
-        atomicAdd(&sh[b * 4 + 0], (unsigned long long)__double2ll_rn(pn * kRadialFix));
-        atomicAdd(&sh[b * 4 + 1], (unsigned long long)__double2ll_rn(pt * kRadialFix));
-        atomicAdd(&sh[b * 4 + 2], (unsigned long long)__double2ll_rn(phi * kRadialFix));
-        atomicAdd(&sh[b * 4 + 3], 1ull);
+        atomicAdd(&radial_sh[b * 7 + 6], 1u);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const long long top = v[c] >> 16;
+            if (top >= -(1ll << 16) && top < (1ll << 16)) {
+                atomicAdd(&radial_sh[b * 7 + 2 * c], (unsigned)(v[c] & 0xFFFF));
+                atomicAdd(&radial_sh[b * 7 + 2 * c + 1], (unsigned)(int)top);
+            } else {
+                atomicAdd(&out[b * 4 + c], (unsigned long long)v[c]);
+            }
+        }
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < nbins * 4; b += blockDim.x)
-        if (sh[b]) atomicAdd(&out[b], sh[b]);
+    for (int t = threadIdx.x; t < nbins * 4; t += kPressThreads) {
+        const int b = t >> 2, c = t & 3;
+        if (radial_sh[b * 7 + 6] == 0u) continue;
+        const unsigned long long s = c == 3 ? (unsigned long long)radial_sh[b * 7 + 6]
+                                            : (unsigned long long)((long long)radial_sh[b * 7 + 2 * c] +
+                                                                   ((long long)(int)radial_sh[b * 7 + 2 * c + 1] << 16));
+        if (s) atomicAdd(&out[t], s);
+    }
 }
 
 // ---------------------------------------------------------------- population copies
@@ -758,25 +1001,31 @@ template <class S>
 cudaError_t launch_pressure_field(const FieldArgs& F, const S* f, const Scratch& W, double* out, cudaStream_t st)
 {
     const long long N = (long long)F.L.nx * F.L.ny * F.L.nz;
-    pressure_field_kernel<S><<<grid_for(N, 256, 65536), 256, 0, st>>>(F, f, W, out);
+    pressure_field_kernel<S><<<grid_for(N, kPressThreads, 65536), kPressThreads, 0, st>>>(F, f, W, out);
     return cudaGetLastError();
 }
 
 template <class S>
-cudaError_t launch_pressure_planes(const FieldArgs& F, const S* f, const Scratch& W, double* out, cudaStream_t st)
+cudaError_t launch_pressure_planes(const FieldArgs& F, const S* f, const Scratch& W, int split, double* part, double* out,
+                                   cudaStream_t st)
 {
-    pressure_plane_kernel<S><<<F.L.nz, kRedThreads, 0, st>>>(F, f, W, out);
+    pressure_plane_kernel<S><<<dim3(F.L.nz, split), kPressThreads, 0, st>>>(F, f, W, split, part);
+    plane_rows_kernel<<<(F.L.nz * 8 + 127) / 128, 128, 0, st>>>(part, F.L.nz, split, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pressure_radial(const FieldArgs& F, const void* f, int prec, const Scratch& W, const double* centre,
-                                   double dr, int nbins, double zmin, unsigned long long* out, cudaStream_t st)
+template <class S>
+cudaError_t launch_pressure_radial(const FieldArgs& F, const S* f, const Scratch& W, const double* centre, double dr,
+                                   int nbins, double zmin, unsigned long long* out, cudaStream_t st)
 {
     if (nbins < 1 || nbins > kRadialBinsMax) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long) * 4 * nbins, st);
     if (e != cudaSuccess) return e;
-    pressure_radial_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(F, f, prec, W, centre[0], centre[1], centre[2], dr,
-                                                                nbins, zmin, out);
+    const long long N = (long long)F.L.nx * F.L.ny * F.L.nz;
+    long long per = (N + kRadialBlocks - 1) / kRadialBlocks;
+    per = per < kPressThreads ? kPressThreads : (per > kRadialNodes ? kRadialNodes : per);
+    pressure_radial_kernel<S><<<(unsigned)((N + per - 1) / per), kPressThreads, (size_t)nbins * 7 * sizeof(unsigned), st>>>(
+        F, f, W, centre[0], centre[1], centre[2], dr, nbins, zmin, (unsigned)per, out);
     return cudaGetLastError();
 }
 
@@ -789,7 +1038,10 @@ cudaError_t launch_pressure_radial(const FieldArgs& F, const void* f, int prec, 
     template cudaError_t launch_get_pop<S>(const FieldArgs&, const S*, double*, cudaStream_t);       \
     template cudaError_t launch_set_pop<S>(const FieldArgs&, S*, const double*, cudaStream_t);   \
     template cudaError_t launch_pressure_field<S>(const FieldArgs&, const S*, const Scratch&, double*, cudaStream_t); \
-    template cudaError_t launch_pressure_planes<S>(const FieldArgs&, const S*, const Scratch&, double*, cudaStream_t);
+    template cudaError_t launch_pressure_planes<S>(const FieldArgs&, const S*, const Scratch&, int, double*, double*, \
+                                                   cudaStream_t);                                     \
+    template cudaError_t launch_pressure_radial<S>(const FieldArgs&, const S*, const Scratch&, const double*, double, int, \
+                                                   double, unsigned long long*, cudaStream_t);
 LBSC_INST(float)
 LBSC_INST(__half)
 LBSC_INST(__nv_bfloat16)

@@ -8,7 +8,6 @@
 namespace lbsc {
 
 constexpr int kRedThreads = 256;  // threads per reduction block
-constexpr int kRedBlocks = 512;   // fixed grid of the reductions: fixed summation order
 constexpr int kConsBlocks = 2048;   // most blocks of the conservation sums (one wave of resident blocks is used)
 constexpr int kAngleBlocks = 1216;  // fixed grid of the contact-angle reduction
 constexpr int kAngleVals = 19;    // contact-angle partial sums per block
@@ -108,16 +107,20 @@ template <class S>
 cudaError_t launch_phi(const FieldArgs& F, const S* f, const Scratch& W, cudaStream_t st);
 cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, double level, double* part, double* out,
                          cudaStream_t st);
-// pressure tensor of Sec. 4.1 (after launch_fields with velocity): every node,
-// per-plane sums, and fixed-point radial bins (see fields.cu)
+// pressure tensor of Sec. 4.1 (after launch_fields): every node, per-plane
+// sums (part: 8 nz split doubles of scratch), and fixed-point radial bins (see fields.cu)
+constexpr int kPressThreads = 128;
 template <class S>
 cudaError_t launch_pressure_field(const FieldArgs& F, const S* f, const Scratch& W, double* out, cudaStream_t st);
 template <class S>
-cudaError_t launch_pressure_planes(const FieldArgs& F, const S* f, const Scratch& W, double* out, cudaStream_t st);
+cudaError_t launch_pressure_planes(const FieldArgs& F, const S* f, const Scratch& W, int split, double* part, double* out,
+                                   cudaStream_t st);
 constexpr int kRadialBinsMax = 1024;
+constexpr int kRadialBlocks = 1824;            // blocks of the radial bins (12 per SM), more where a block would take too many nodes
 constexpr double kRadialFix = 1073741824.0;  // fixed-point unit of the radial sums: 2^-30
-cudaError_t launch_pressure_radial(const FieldArgs& F, const void* f, int prec, const Scratch& W, const double* centre,
-                                   double dr, int nbins, double zmin, unsigned long long* out, cudaStream_t st);
+template <class S>
+cudaError_t launch_pressure_radial(const FieldArgs& F, const S* f, const Scratch& W, const double* centre, double dr,
+                                   int nbins, double zmin, unsigned long long* out, cudaStream_t st);
 // z-slab face messages (halo.cu): 38 entries of nx*ny values per face
 constexpr int kHaloEntries = 38;
 // face 0 = below (planes 0, 1), 1 = above (planes nz-2, nz-1); unpack 0 packs

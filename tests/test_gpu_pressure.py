@@ -193,3 +193,80 @@ def test_laplace_law_free_droplets_3d(lbsc):
     assert gamma > 0
     assert math.isclose(slope / 2, gamma, rel_tol=0.15), (slope / 2, gamma)
     assert math.isclose(g_rad, gamma, rel_tol=0.10) and abs(R_s - 1 / inv_r[-1]) < 1.0, (g_rad, gamma, R_s)
+
+
+C = np.array([(0, 0, 0), (1, 0, 0), (-1, 0, 0), (0, 1, 0), (0, -1, 0), (0, 0, 1), (0, 0, -1), (1, 1, 0), (-1, -1, 0),
+              (1, -1, 0), (-1, 1, 0), (1, 0, 1), (-1, 0, -1), (1, 0, -1), (-1, 0, 1), (0, 1, 1), (0, -1, -1),
+              (0, 1, -1), (0, -1, 1)])
+IJ = [(0, 0), (1, 1), (2, 2), (0, 1), (0, 2), (1, 2)]
+
+
+def _tensor64(lat, solid, prm):
+    """Sec. 4.1's tensor in FP64 from the lattice's own populations."""
+    n = lat.populations()
+    _, _, u, _ = lat.moments(velocity=True)
+    psi = -np.expm1(-n.sum(1))
+    psi[0][solid == 1], psi[1][solid == 1] = prm["eta_wall_r"], prm["eta_wall_b"]
+    P = np.zeros((6,) + solid.shape)
+    for k in range(19):
+        v = [C[k][d] - u[d] for d in range(3)]
+        at = [np.roll(psi[a], tuple(-C[k][::-1]), (0, 1, 2)) for a in (0, 1)]
+        G = 0.0 if k == 0 else (2.0 if k <= 6 else 1.0)
+        w = 0.5 * prm["g_br"] * prm["force_scale"] * G * (psi[0] * at[1] + psi[1] * at[0])
+        for c, (i, j) in enumerate(IJ):
+            P[c] += v[i] * v[j] * n[:, k].sum(0) + w * C[k][i] * C[k][j]
+    return P * (solid == 0)
+
+
+@pytest.mark.parametrize("precision", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("dims,periodic", [((1, 1, 10), False), ((5, 3, 6), False), ((33, 9, 7), False), ((129, 2, 5), True),
+                                           ((70, 41, 12), False), ((16, 24, 33), True)])
+def test_pressure_sums_on_ragged_lattices(lbsc, dims, periodic, precision):
+    """Tensor against FP64 sums over the same populations, at the bar of the oracle tests above (psi and u are FP32).
+    Plane means and radial bins against that tensor: pairs and FP64 sums, 1e-12; bins rounded to 2^-30 a node, 2e-9,
+    with the nodes' distances whole numbers on the bins' edges."""
+    nx, ny, nz = dims
+    solid = W.periodic_mask(*dims) if periodic else W.wall_mask(*dims)
+    rr, rb = W.droplet_fields(nx, ny, nz, 0.3 * min(nx, ny, nz) + 1.0, seed=4, centre=(nx / 2, ny / 2, nz / 2))
+    prm = dict(CONTACT, eta_wall_r=-0.04, eta_wall_b=0.04)
+    lat = lbsc.Lattice(rr, rb, precision)
+    if periodic:
+        lat.set_geometry(solid)
+    lat.set_params(**prm).step(3)
+    P = lat.pressure_tensor()
+    ref = _tensor64(lat, solid, prm)
+    assert np.abs(P - ref).max() <= 2e-6 * np.abs(ref).max()
+    r, b, _, _ = lat.moments()
+    prof, _ = lat.pressure_profile()
+    fluid = (solid == 0).astype(float)
+    cnt = fluid.sum((1, 2))
+    assert np.array_equal(prof[:, 7], cnt)
+    for v, a in enumerate(list(P) + [r - b]):
+        mean = (a * fluid).sum((1, 2)) / np.maximum(cnt, 1)
+        assert np.abs(prof[:, v] - mean).max() <= 1e-12 * max(1.0, np.abs(a).max())
+    centre = (float(nx // 2), float(ny // 2), float(nz // 2))
+    bins, _, _ = lat.pressure_radial(centre, 0.5, 40, 1.0)
+    obins, _, _ = oracle.pressure_radial(P, solid, r, b, centre, 0.5, 40, 1.0, 1e30, periodic_z=periodic)
+    assert np.array_equal(bins[:, 3], obins[:, 3])
+    assert np.abs(bins - obins).max() <= 2e-9
+
+
+def test_pressure_of_a_state_with_an_infinity(lbsc):
+    """One infinite population: the tensor is not finite at its node and as before everywhere else; the profile is not
+    finite in its plane alone."""
+    nx, ny, nz = 20, 11, 12
+    rr, rb = W.droplet_fields(nx, ny, nz, 4.0, seed=4)
+    lat = lbsc.Lattice(rr, rb).set_params(**CONTACT).step(3)
+    P0, (prof0, _) = lat.pressure_tensor(), lat.pressure_profile()
+    n = lat.populations()
+    n[0, 7, 5, 4, 3] = np.inf
+    lat.set_populations(n)
+    P, (prof, _) = lat.pressure_tensor(), lat.pressure_profile()
+    there = np.zeros((nz, ny, nx), bool)
+    there[5, 4, 3] = True
+    assert not np.isfinite(P[:, there]).any()
+    far = np.ones((nz, ny, nx), bool)
+    far[4:7, 3:6, 2:5] = False  # the neighbours see another psi
+    assert np.isfinite(P[:, ~there]).all() and np.array_equal(P[:, far], P0[:, far])
+    keep = [z for z in range(nz) if z not in (4, 5, 6)]
+    assert not np.isfinite(prof[5, :6]).any() and np.array_equal(prof[keep], prof0[keep])
