@@ -473,8 +473,7 @@ void lb_batch_free(lb_batch* b);
  *   cons         device pointer to 8 doubles, caller-owned; receives
  *                {mass_r, mass_b, Px, Py, Pz, non-finite count, fluid nodes, 0}
  *   cuda_stream  stream the two kernels are queued on; the call is asynchronous
- * At most 67,108,864 nodes (the scratch holds 1024 block rows of 65,536
- * nodes each); larger lattices return LB_ERR_ARG with a message. The first
+ * At most 67,108,864 nodes; larger lattices return LB_ERR_ARG with a message. The first
  * call on each device looks up the scratch array's device address (a
  * cudaGetSymbolAddress call), so make that first call before any stream
  * capture. Every call shares the one scratch array on a device: calls whose
