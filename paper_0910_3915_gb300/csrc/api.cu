@@ -113,7 +113,7 @@ static Plan make_plan(const Layout& L, int prec)
     p.f = align256((size_t)2 * Q * L.slot * elem_size(prec));
     p.mask = align256((size_t)L.plane * L.nz * sizeof(uint32_t));
     p.scratch = align256((size_t)10 * N * sizeof(float));
-    p.part = align256((size_t)kPartRows * kAngleVals * sizeof(double));
+    p.part = align256((size_t)kPartRows * kPartVals * sizeof(double));
     p.red = align256(64 * sizeof(double));
     p.total = 2 * p.f + p.mask + p.scratch + p.part + p.red;
     return p;
@@ -456,7 +456,8 @@ static int init_common(lb_ctx** out, int nx, int ny, int nz, int precision, cons
     if (e != cudaSuccess) return bail(LB_ERR_CUDA, std::string("lb_init: cudaMallocHost: ") + cudaGetErrorString(e));
 
     if (planar_default(c) != LB_OK) return bail(LB_ERR_CUDA, c->err);
-    // reduction area: outputs [0, 32), conservation accumulators [32, 40) and ticket [40], status word, step counter
+    // reduction area: conservation accumulators [32, 40) and ticket [40], contact-angle ticket [41], status word [48],
+    // step counter [50]
     e = cudaMemsetAsync(c->red, 0, 64 * sizeof(double), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->dev_err, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->clock, 0, 2 * sizeof(uint32_t), c->stream);
@@ -795,7 +796,7 @@ template <class S>
 static cudaError_t run_cons(lb_ctx* c, float* phi)
 {
     return launch_conservation<S>(field_args(c), (const S*)c->f[c->cur], (unsigned long long*)(c->red + 32),
-                                  (unsigned int*)(c->red + 40), c->red, c->stream, phi);
+                                  (unsigned int*)(c->red + 40), c->h_red, c->dev_err, c->stream, phi);
 }
 template <class S>
 static cudaError_t run_fields(lb_ctx* c, bool vel)
@@ -835,17 +836,24 @@ static cudaError_t dispatch_fields(lb_ctx* c, bool vel)
 
 extern "C" {
 
-// the conservation sums (and, with phi, the contact angle's phi field) of the
-// current state into cons[8]
-static int conservation_impl(lb_ctx* c, double cons[8], float* phi)
+// A measurement is queued, then (once its stream has been waited for) taken
+// from pinned host memory the kernels wrote: one wait per call, however many
+// parts or boxes it has, and no copies.
+static int wait(lb_ctx* c)
 {
-    LB_CUDA(c, dispatch_cons(c, phi));
-    LB_CUDA(c, cudaMemcpyAsync(c->h_red, c->red, 8 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     LB_CUDA(c, cudaStreamSynchronize(c->stream));
+    return LB_OK;
+}
+
+// the conservation sums queued by dispatch_cons into cons[8]
+static int take_cons(lb_ctx* c, double cons[8])
+{
     for (int i = 0; i < 7; ++i) cons[i] = c->h_red[i];
     cons[7] = (double)c->steps;
-    const int st = check_device_status(c);
-    if (st != LB_OK) return st;
+    if (c->h_red[7] != 0) {
+        const int st = check_device_status(c);
+        if (st != LB_OK) return st;
+    }
     if (cons[5] > 0) return fail(c, LB_ERR_NAN, "non-finite populations in the state");
     return LB_OK;
 }
@@ -853,7 +861,9 @@ static int conservation_impl(lb_ctx* c, double cons[8], float* phi)
 int lb_conservation(lb_ctx* c, double cons[8])
 {
     if (!c || !cons) return fail(c, LB_ERR_ARG, "lb_conservation: NULL argument");
-    return conservation_impl(c, cons, nullptr);
+    LB_CUDA(c, dispatch_cons(c));
+    const int rc = wait(c);
+    return rc == LB_OK ? take_cons(c, cons) : rc;
 }
 
 int lb_moments(lb_ctx* c, double* rho_r, double* rho_b, double* u, double cons[8])
@@ -907,9 +917,15 @@ static int solve4(double M[4][4], double v[4], double s[4])
     return 0;
 }
 
-// the droplet of the phi field in c->W (written by the phi pass or the
-// conservation pass of the current state)
-static int angle_from_phi(lb_ctx* c, double offset, double level, lb_droplet* out);
+// queue the droplet's sums of the phi field in c->W (written by the phi pass or
+// the conservation pass of the current state); take its record once waited for
+static int queue_angle(lb_ctx* c, double offset, double level)
+{
+    LB_CUDA(c, launch_angle(field_args(c), c->W, 0.5 + offset, level, c->part, (unsigned int*)(c->red + 41), c->h_red + 8,
+                            c->stream));
+    return LB_OK;
+}
+static int take_angle(lb_ctx* c, double offset, double level, lb_droplet* out);
 
 int lb_contact_angle(lb_ctx* c, double offset, lb_droplet* out) { return lb_contact_angle_at(c, offset, 0.0, out); }
 
@@ -918,26 +934,27 @@ int lb_contact_angle_at(lb_ctx* c, double offset, double level, lb_droplet* out)
     if (!c || !out || !(offset >= 0) || !std::isfinite(offset) || !std::isfinite(level))
         return fail(c, LB_ERR_ARG, "lb_contact_angle: bad argument");
     LB_CUDA(c, dispatch_phi(c));
-    return angle_from_phi(c, offset, level, out);
+    int rc = queue_angle(c, offset, level);
+    if (rc == LB_OK) rc = wait(c);
+    return rc == LB_OK ? take_angle(c, offset, level, out) : rc;
 }
 
 int lb_measure(lb_ctx* c, double cons[8], double offset, lb_droplet* out)
 {
     if (!c || !cons || !out || !(offset >= 0) || !std::isfinite(offset))
         return fail(c, LB_ERR_ARG, "lb_measure: bad argument");
-    const int rc = conservation_impl(c, cons, c->W.rho[0]);
-    if (rc != LB_OK) return rc;
-    return angle_from_phi(c, offset, 0.0, out);
+    LB_CUDA(c, dispatch_cons(c, c->W.rho[0]));
+    int rc = queue_angle(c, offset, 0.0);
+    if (rc == LB_OK) rc = wait(c);
+    if (rc == LB_OK) rc = take_cons(c, cons);
+    return rc == LB_OK ? take_angle(c, offset, 0.0, out) : rc;
 }
 
-static int angle_from_phi(lb_ctx* c, double offset, double level, lb_droplet* out)
+static int take_angle(lb_ctx* c, double offset, double level, lb_droplet* out)
 {
     memset(out, 0, sizeof(*out));
     const double zw = 0.5, zref = zw + offset;
-    LB_CUDA(c, launch_angle(field_args(c), c->W, zref, level, c->part, c->red, c->stream));
-    LB_CUDA(c, cudaMemcpyAsync(c->h_red, c->red, kAngleVals * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    LB_CUDA(c, cudaStreamSynchronize(c->stream));
-    const double* v = c->h_red;
+    const double* v = c->h_red + 8;
     const double top = v[0], area = v[1];
     const int npts = (int)v[2];
     const double h = top - zw;
@@ -945,11 +962,11 @@ static int angle_from_phi(lb_ctx* c, double offset, double level, lb_droplet* ou
     const double bref = 2.0 * std::sqrt(area / pi), hp = h - offset;
     out->h = h;
     out->base_ref = bref;
-    out->phi_max = v[17];
-    out->phi_min = -v[18];
+    out->phi_max = v[16];
+    out->phi_min = -v[17];
     const int z0 = (int)std::floor(zref);
     if (!(z0 >= 0 && z0 + 1 < c->nz)) out->status = LB_DROP_BAD_PLANE;
-    else if (!(v[17] > -1e299) || !((double)v[17] - level > 0)) out->status = LB_DROP_NO_PHASE;
+    else if (!(v[16] > -1e299) || !(v[16] - level > 0)) out->status = LB_DROP_NO_PHASE;
     else if (!(top > -1e299)) out->status = LB_DROP_NO_APEX;
     else if (!(hp > 0)) out->status = LB_DROP_LOW_APEX;
     else if (!(bref > 0)) out->status = LB_DROP_NO_BASE;
@@ -966,11 +983,15 @@ static int angle_from_phi(lb_ctx* c, double offset, double level, lb_droplet* ou
     }
     out->n_points = npts;
     if (npts >= 4) {
+        // normal equations of the sphere through the points p: rows (2 p, 1), right sides |p|^2
+        const double row[4] = {2, 2, 2, 1}, *u = v + 3;
+        const double m[4][4] = {{u[0], u[1], u[2], u[3]}, {u[1], u[4], u[5], u[6]}, {u[2], u[5], u[7], u[8]},
+                                {u[3], u[6], u[8], v[2]}};
         double M[4][4], rhs[4], s[4];
-        int m = 3;
-        for (int r = 0; r < 4; ++r)
-            for (int q = r; q < 4; ++q) M[r][q] = M[q][r] = v[m++];
-        for (int r = 0; r < 4; ++r) rhs[r] = v[13 + r];
+        for (int r = 0; r < 4; ++r) {
+            for (int q = 0; q < 4; ++q) M[r][q] = row[r] * row[q] * m[r][q];
+            rhs[r] = row[r] * v[12 + r];
+        }
         if (solve4(M, rhs, s) == 0) {
             const double R2 = s[3] + s[0] * s[0] + s[1] * s[1] + s[2] * s[2];
             if (R2 > 0) {
@@ -1409,8 +1430,10 @@ int lb_batch_box(lb_batch* b, int i, lb_ctx** out)
 int lb_batch_conservation(lb_batch* b, double* cons)
 {
     if (!b || !cons) return bfail(b, LB_ERR_ARG, "lb_batch_conservation: NULL argument");
+    for (lb_ctx* c : b->box) LB_BCUDA(b, dispatch_cons(c));
+    LB_BCUDA(b, cudaStreamSynchronize(b->stream));
     for (int i = 0; i < b->nbox; ++i) {
-        const int rc = lb_conservation(b->box[i], cons + 8 * (size_t)i);
+        const int rc = take_cons(b->box[i], cons + 8 * (size_t)i);
         if (rc != LB_OK) return bfail(b, rc, "box " + std::to_string(i) + ": " + b->box[i]->err);
     }
     return LB_OK;
@@ -1419,11 +1442,19 @@ int lb_batch_conservation(lb_batch* b, double* cons)
 int lb_batch_contact_angles(lb_batch* b, double offset, lb_droplet* out)
 {
     if (!b || !out) return bfail(b, LB_ERR_ARG, "lb_batch_contact_angles: NULL argument");
-    for (int i = 0; i < b->nbox; ++i) {
-        const int rc = lb_contact_angle(b->box[i], offset, &out[i]);
-        if (rc != LB_OK) return bfail(b, rc, "box " + std::to_string(i) + ": " + b->box[i]->err);
+    int rc = LB_OK, i = 0;
+    if (!(offset >= 0) || !std::isfinite(offset)) rc = fail(b->box[0], LB_ERR_ARG, "lb_contact_angle: bad argument");
+    for (; rc == LB_OK && i < b->nbox; ++i) {
+        LB_BCUDA(b, dispatch_phi(b->box[i]));
+        rc = queue_angle(b->box[i], offset, 0.0);
+        if (rc != LB_OK) break;
     }
-    return LB_OK;
+    if (rc == LB_OK) {
+        LB_BCUDA(b, cudaStreamSynchronize(b->stream));
+        for (i = 0; i < b->nbox; ++i) take_angle(b->box[i], offset, 0.0, &out[i]);
+        return LB_OK;
+    }
+    return bfail(b, rc, "box " + std::to_string(i) + ": " + b->box[i]->err);
 }
 
 const char* lb_batch_last_error(const lb_batch* b)
@@ -1737,7 +1768,7 @@ extern "C" int lb_pressure_profile(lb_ctx* c, double* prof, double* gamma_sum)
     const size_t need = (size_t)nz * 8 * (size_t)(split + 1);
     AdjScratch M;
     double* d = c->part;
-    if (need > (size_t)kPartRows * kAngleVals) LB_CUDA(c, M.alloc((void**)&d, need * sizeof(double)));
+    if (need > (size_t)kPartRows * kPartVals) LB_CUDA(c, M.alloc((void**)&d, need * sizeof(double)));
     double* part = d + (size_t)nz * 8;
     LB_CUDA(c, dispatch_fields(c, false));
     switch (c->prec) {
@@ -1767,7 +1798,7 @@ extern "C" int lb_pressure_radial(lb_ctx* c, const double* centre, double dr, in
     if (!c || !centre || !bins || !(dr > 0) || nbins < 1 || nbins > kRadialBinsMax || !std::isfinite(zmin) ||
         !std::isfinite(r_max) || !std::isfinite(centre[0]) || !std::isfinite(centre[1]) || !std::isfinite(centre[2]))
         return fail(c, LB_ERR_ARG, "lb_pressure_radial: bad argument (dr > 0, 1 <= nbins <= 1024, finite centre)");
-    static_assert((size_t)kRadialBinsMax * 4 <= (size_t)kPartRows * kAngleVals, "the bins fit the partials area");
+    static_assert((size_t)kRadialBinsMax * 4 <= (size_t)kPartRows * kPartVals, "the bins fit the partials area");
     unsigned long long* d = (unsigned long long*)c->part;
     LB_CUDA(c, dispatch_fields(c, false));
     switch (c->prec) {

@@ -5,6 +5,7 @@
 // warp shuffles and a final pass over the per-block partials in block order.
 #include "lb_fields.cuh"
 
+#include <cmath>
 #include <type_traits>
 
 namespace lbsc {
@@ -15,43 +16,6 @@ __device__ __forceinline__ double warp_sum(double v)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     return v;
 }
-__device__ __forceinline__ double warp_max(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-    return v;
-}
-
-// Sum (or max) nrows partial rows of NV values: block v reduces value v,
-// thread t taking rows t, t + 256, ... in order, then a fixed shuffle tree per
-// warp and the warps in order. Launched as NV blocks of 256 threads.
-template <int NV>
-__global__ void __launch_bounds__(256) finish_rows_kernel(const double* __restrict__ part, int nrows, uint32_t is_max,
-                                                          double* __restrict__ out)
-{
-    const int v = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (v >= NV) return;
-    const bool mx = (is_max >> v) & 1u;
-    double a = mx ? -1e300 : 0.0;
-    for (int r = threadIdx.x; r < nrows; r += blockDim.x) {
-        const double p = part[(long long)r * NV + v];
-        a = mx ? fmax(a, p) : a + p;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double w = __shfl_down_sync(0xffffffffu, a, o);
-        a = mx ? fmax(a, w) : a + w;
-    }
-    __shared__ double sw[8];
-    if (lane == 0) sw[warp] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = sw[0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) t = mx ? fmax(t, sw[w]) : t + sw[w];
-        out[v] = t;
-    }
-}
-
 // blocks for n items at `threads` per block, at most cap (grid-stride loops cover the rest)
 static int grid_for(long long n, int threads, int cap)
 {
@@ -93,6 +57,58 @@ __device__ __forceinline__ bool node_solid(const FieldArgs& F, int x, int y, int
     return z == 0 || z == F.L.nz - 1;
 }
 
+// ---------------------------------------------------------------- pairs of FP32 numbers
+// FP64 issues about once a clock and SM on this GPU, FP32 128 times. Sums that
+// need more than FP32 are taken in pairs (Dekker 1971, Knuth's two-sum): a
+// value is h + l with l far below h, a sum carries the rounding error of h in
+// l. That keeps about 46 bits.
+struct Two {
+    float h, l;
+};
+__device__ __forceinline__ Two two(float a) { return Two{a, 0.f}; }
+__device__ __forceinline__ Two two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return Two{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+// l may grow to a few roundings of h: normalised by norm2 before a product
+__device__ __forceinline__ Two operator+(Two a, Two b)
+{
+    const Two s = two_sum(a.h, b.h);
+    return Two{s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ Two operator-(Two a) { return Two{-a.h, -a.l}; }
+__device__ __forceinline__ Two operator-(Two a, Two b) { return a + (-b); }
+__device__ __forceinline__ Two norm2(Two a)
+{
+    const float s = __fadd_rn(a.h, a.l);
+    return Two{s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
+}
+__device__ __forceinline__ Two mul2f(Two a, float f)  // a normalised
+{
+    const float p = __fmul_rn(a.h, f);
+    return Two{p, __fmaf_rn(a.l, f, __fmaf_rn(a.h, f, -p))};
+}
+__device__ __forceinline__ Two mul22(Two a, Two b)  // both normalised
+{
+    const float p = __fmul_rn(a.h, b.h);
+    return Two{p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ double to_f64(Two a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ Two two_int(int i)  // exact below 2^47
+{
+    const float h = (float)i;
+    return Two{h, (float)((long long)i - (long long)h)};
+}
+// a / b, both normalised: one quotient and one correction
+__device__ __forceinline__ Two div22(Two a, Two b)
+{
+    const float q = __fdiv_rn(a.h, b.h);
+    const float r = __fadd_rn(__fmaf_rn(-q, b.h, a.h), __fmaf_rn(-q, b.l, a.l));
+    return norm2(Two{q, __fdiv_rn(r, b.h)});
+}
+__device__ __forceinline__ bool less2(Two a, Two b) { return a.h < b.h || (a.h == b.h && a.l < b.l); }  // normalised
+
 // ---------------------------------------------------------------- init
 // populations at rest: n_k = zeta_k rho (Eq. Equil at u = 0). err (may be
 // NULL): kErrInput is set for a density that is negative or not finite.
@@ -120,14 +136,16 @@ __global__ void init_kernel(FieldArgs F, S* __restrict__ f, const double* __rest
 }
 
 // ---------------------------------------------------------------- conservation
-// cons = {M_r, M_b, Px, Py, Pz, non-finite count, fluid nodes, -}
+// cons = {M_r, M_b, Px, Py, Pz, non-finite count, fluid nodes, the status word *err}
 // A grid-stride walk over the nodes of the fluid planes, x fastest, so that a
 // warp's load of one population slot covers consecutive addresses, with a
 // node's 38 loads independent of each other. A node's mass and momentum are
 // summed in FP32 over its 19 values per component, and each thread adds its
 // nodes in FP32. The threads' sums then go into 64-bit integers in units of
 // 2^-28 (kConsFix) and are added as integers: across warps, blocks and the
-// whole grid, by shuffles and atomics. Integer addition is exact and
+// whole grid, by shuffles and atomics. A node's values are tested one by one
+// only where its sums are not finite (testing all 38 was a quarter of the
+// instructions). Integer addition is exact and
 // associative, so the totals do not depend on the grid or on the order the
 // blocks finish, and no FP64 arithmetic (slow on this GPU) runs per node. The
 // last block to finish converts the totals to FP64 into out[0..7] and clears
@@ -141,7 +159,7 @@ template <class S>
 __global__ void __launch_bounds__(kRedThreads) cons_kernel(FieldArgs F, const S* __restrict__ f,
                                                            unsigned long long* __restrict__ acc,
                                                            unsigned int* __restrict__ ticket, double* __restrict__ out,
-                                                           float* __restrict__ phi)
+                                                           float* __restrict__ phi, const int* __restrict__ err)
 {
     float m[2] = {0.f, 0.f}, j[3] = {0.f, 0.f, 0.f};
     int bad = 0, fluid = 0;
@@ -169,7 +187,6 @@ __global__ void __launch_bounds__(kRedThreads) cons_kernel(FieldArgs F, const S*
 #pragma unroll
             for (int k = 0; k < Q; ++k) {
                 const float nk = v[a][k];
-                bad += isfinite(nk) ? 0 : 1;
                 s = __fadd_rn(s, nk);  // as the phi pass
                 if (cx(k)) jn[0] += cx(k) * nk;
                 if (cy(k)) jn[1] += cy(k) * nk;
@@ -178,6 +195,9 @@ __global__ void __launch_bounds__(kRedThreads) cons_kernel(FieldArgs F, const S*
             rho[a] = s;
         }
         if (phi) phi[i] = rho[0] - rho[1];
+        if (!isfinite(rho[0]) || !isfinite(rho[1]))  // a value that is not finite makes its component's sum so
+#pragma unroll
+            for (int k = 0; k < Q; ++k) bad += (isfinite(v[0][k]) ? 0 : 1) + (isfinite(v[1][k]) ? 0 : 1);
         m[0] += rho[0];
         m[1] += rho[1];
 #pragma unroll
@@ -213,7 +233,7 @@ __global__ void __launch_bounds__(kRedThreads) cons_kernel(FieldArgs F, const S*
         __threadfence();
         const int v = threadIdx.x;
         const long long t = v < 7 ? (long long)atomicExch(&acc[v], 0ull) : 0;
-        out[v] = v < 5 ? (double)t / kConsFix : (double)t;
+        out[v] = v < 5 ? (double)t / kConsFix : (v == 7 ? (double)*err : (double)t);
         if (v == 0) *ticket = 0u;
     }
 }
@@ -330,184 +350,280 @@ __global__ void phi_kernel(FieldArgs F, const S* __restrict__ f, Scratch W)
 }
 
 // ---------------------------------------------------------------- contact angle
-// phi - level in FP64 at a node whose phi is the FP32 value p
-__device__ __forceinline__ double phi_at(float p, double level) { return (double)p - level; }
+// phi > level for the FP32 value p, exactly: A.least is the least FP32 number above the FP64 level
+__device__ __forceinline__ bool above(float p, const AngleArgs& A) { return p >= A.least; }
 
-// p > level in FP64, out of line: the rare case the FP32 test below cannot decide
-__device__ __noinline__ bool above_fp64(float p, double level) { return (double)p > level; }
-
-// p > level, i.e. phi_at(p, level) > 0, taken in FP32 where that is exact: when
-// level is an FP32 number, or when p is far from it (the margin exceeds the
-// rounding of level to FP32 many times over); else in FP64.
-__device__ __forceinline__ bool above(float p, float lf, bool lexact, double level)
+// phi - level
+__device__ __forceinline__ Two over(float p, const AngleArgs& A)
 {
-    if (lexact || fabsf(p - lf) > 1e-6f * (fabsf(p) + fabsf(lf)) + 1e-30f) return p > lf;
-    return above_fp64(p, level);
+    const Two s = two_sum(p, -A.lh);
+    return norm2(Two{s.h, __fsub_rn(s.l, A.ll)});
 }
 
 // Positive length along x, from a node to its +x neighbour, of the linear
 // interpolant of phi - level on the reference plane z0 + fz (p: phi at the
-// node, above it, at the +x neighbour and above that). Out of line, so that
-// its FP64 work runs only on that plane's rows.
-__device__ __noinline__ double plane_length(float p0, float p0up, float p1, float p1up, double fz, double level)
+// node, above it, at the +x neighbour and above that).
+__device__ __forceinline__ Two plane_length(float p0, float p0up, float p1, float p1up, const AngleArgs& A)
 {
-    const double a0 = (1 - fz) * phi_at(p0, level) + fz * phi_at(p0up, level);
-    const double a1 = (1 - fz) * phi_at(p1, level) + fz * phi_at(p1up, level);
-    if (a0 > 0 && a1 > 0) return 1.0;
-    if (a0 <= 0 && a1 <= 0) return 0.0;
-    return a0 > 0 ? a0 / (a0 - a1) : a1 / (a1 - a0);
+    const Two f{A.fzh, A.fzl}, g = norm2(two(1.0f) - f);
+    const Two a0 = norm2(mul22(g, over(p0, A)) + mul22(f, over(p0up, A)));
+    const Two a1 = norm2(mul22(g, over(p1, A)) + mul22(f, over(p1up, A)));
+    if (a0.h > 0 && a1.h > 0) return two(1.0f);
+    if (a0.h <= 0 && a1.h <= 0) return two(0.0f);
+    return a0.h > 0 ? div22(a0, norm2(a0 - a1)) : div22(a1, norm2(a1 - a0));
 }
 
 // An interface crossing between node (x, y, z) (phi = p0) and its neighbour
 // along axis d (phi = p1): the top crossing (along z, from phi > level
 // below to phi <= level above) and the sphere-fit sums of the crossing point at
 // or above the reference plane, into the thread's accumulators acc[i * stride].
-// Kept out of line so that the FP64 work runs only in the warps that meet a
-// crossing instead of being predicated into every node's path.
-__device__ __noinline__ void add_crossing(double* acc, int stride, int x, int y, int z, int d, float p0, float p1,
-                                         double level, bool s0, double zref)
+// Out of line: it is reached from a few places and rarely, and the row loop
+// fits the instruction cache without it.
+__device__ __noinline__ void add_crossing(float2* acc, int stride, int x, int y, int z, int d, float p0, float p1,
+                                          const AngleArgs& A)
 {
-    const double q0 = phi_at(p0, level), q1 = phi_at(p1, level);
-    const double t = q0 / (q0 - q1);
-    if (d == 2 && s0) acc[0] = fmax(acc[0], z + t);  // phi > level below, <= level above
-    const double pxv = x + t * (d == 0), pyv = y + t * (d == 1), pzv = z + t * (d == 2);
-    if (pzv < zref) return;
-    const double row[4] = {2 * pxv, 2 * pyv, 2 * pzv, 1.0};
-    const double rhs = pxv * pxv + pyv * pyv + pzv * pzv;
-    acc[2 * stride] += 1.0;
-    int m = 3;
-    for (int r = 0; r < 4; ++r)
-        for (int q = r; q < 4; ++q) acc[(m++) * stride] += row[r] * row[q];
-    for (int r = 0; r < 4; ++r) acc[(13 + r) * stride] += row[r] * rhs;
+    const Two q0 = over(p0, A);
+    Two t = div22(q0, norm2(two_sum(p0, -p1)));
+    if (isinf(p1) && isfinite(p0)) t = two(0.f);  // q0 over an infinity
+    const Two c[3] = {two_int(x), two_int(y), two_int(z)};
+    Two p[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) p[q] = d == q ? norm2(c[q] + t) : c[q];
+    if (d == 2 && above(p0, A)) {  // phi > level below, <= level above
+        const float2 top = acc[0];
+        if (less2(Two{top.x, top.y}, p[2])) acc[0] = make_float2(p[2].h, p[2].l);
+    }
+    if (less2(p[2], Two{A.zh, A.zl})) return;
+    auto add = [&](int i, Two v) {
+        const float2 o = acc[i * stride];
+        const Two s = norm2(Two{o.x, o.y} + v);
+        acc[i * stride] = make_float2(s.h, s.l);
+    };
+    const Two xx = norm2(mul22(p[0], p[0])), yy = norm2(mul22(p[1], p[1])), zz = norm2(mul22(p[2], p[2]));
+    const Two rr = norm2((xx + yy) + zz);
+    add(2, two(1.0f));
+    add(3, xx);
+    add(4, mul22(p[0], p[1]));
+    add(5, mul22(p[0], p[2]));
+    add(6, p[0]);
+    add(7, yy);
+    add(8, mul22(p[1], p[2]));
+    add(9, p[1]);
+    add(10, zz);
+    add(11, p[2]);
+    add(12, mul22(p[0], rr));
+    add(13, mul22(p[1], rr));
+    add(14, mul22(p[2], rr));
+    add(15, rr);
 }
 
-// One warp per lattice row, a lane per node, reading phi at the node and at
-// its +x, +y, +z neighbours (the latter from L1/L2):
+// One warp per lattice row, a lane per node, four nodes of the row in flight a
+// lane, reading phi at the node and at its +y, +z neighbours (the latter from
+// L1/L2; +x by shuffle):
 //  [0]  (max) top phi = level crossing: z + p0/(p0 - p1) where phi > level
 //       below and <= level above (both nodes fluid);
 //  [1]  positive length along x of the reference-plane interpolant of phi
 //       (the node at z0 adds its segment to x + 1, periodic);
-//  [2..16] sphere-fit sums over crossings along +x, +y, +z at or above the
-//       reference plane: count, the 10 upper entries of M = sum row row^T and
-//       the 4 of v = sum row |p|^2, row = (2p, 1);
-//  [17] (max) max of phi over fluid nodes, [18] (max) of -phi (the contrast).
-// FP64 arithmetic (slow on this GPU) runs only at crossings and on the
-// reference plane; a thread's FP64 sums wait in shared memory, and a warp
-// reduces a value only if one of its lanes holds a contribution to it.
-__global__ void __launch_bounds__(kRedThreads) angle_kernel(FieldArgs F, Scratch W, double zref, double level,
-                                                            double* __restrict__ part)
+//  [2..15] sums over crossings along +x, +y, +z at or above the reference
+//       plane: 1, xx, xy, xz, x, yy, yz, y, zz, z, x rr, y rr, z rr, rr (rr = |p|^2);
+//  [16] (max) max of phi over fluid nodes, [17] (max) of -phi (the contrast).
+// All in pairs of FP32 numbers: with FP64 sums (a drained queue took about 70
+// FP64 operations, 2240 cycles of an SM's one FP64 lane) the kernel took 53 us
+// at 128^3, bound by the SMs that met the most crossings. A block takes rows
+// gridDim apart for the same reason: the drop's rows spread over all SMs. Now 30 us at 128^3 (9 million
+// instructions, a third of them for crossings; phi is 8 MB, in L2).
+// A thread's sums wait in shared memory, and a warp reduces a value only if one
+// of its lanes holds a contribution to it. The last block to finish adds the
+// blocks' rows, in order, and writes the 19 values lb_contact_angle works with.
+__global__ void __launch_bounds__(kAngleThreads) angle_kernel(FieldArgs F, AngleArgs A, const float* __restrict__ P,
+                                                              float2* __restrict__ part, unsigned int* __restrict__ ticket,
+                                                              double* __restrict__ out)
 {
+    constexpr int kWarps = kAngleThreads / 32, kStrips = 4;
     const int nx = F.L.nx, ny = F.L.ny, nz = F.L.nz;
-    __shared__ double sacc[kAngleVals][kRedThreads];
-    const int tid = threadIdx.x;
-#define ACC(i) sacc[i][tid]
-    for (int i = 0; i < 17; ++i) ACC(i) = 0.0;
-    ACC(0) = -1e300;
+    __shared__ float2 sacc[16][kAngleThreads];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = 0; i < 16; ++i) sacc[i][tid] = make_float2(i == 0 ? kNoTop : 0.f, 0.f);
     float pmax = -3.0e38f, pmin = 3.0e38f;
-    const int z0 = (int)floor(zref);
-    const double fz = zref - z0;
-    const float lf = (float)level;
-    const bool lexact = (double)lf == level;
-    const float* __restrict__ P = W.rho[0];
     const unsigned nxy = (unsigned)nx * (unsigned)ny;
     // Interface crossings are rare and scattered: a lane that meets one would
-    // run the FP64 work of add_crossing alone, at the cost of a whole warp's.
+    // run the arithmetic of add_crossing alone, at the cost of a whole warp's.
     // So the warp queues its crossings in shared memory, in lane order, and
     // works through them 32 at a time with every lane busy; which lane sums
     // which crossing depends only on the data, so the sums are reproducible.
-    __shared__ int4 qpos[kRedThreads / 32][64];     // (x, y, z, axis)
-    __shared__ float2 qphi[kRedThreads / 32][64];   // (phi at the node, phi at the neighbour)
-    const int lane = tid & 31, warp = tid >> 5;
+    // An entry: x and the row, each with a bit of the axis on top, and phi at
+    // the node and at its neighbour.
+    __shared__ int4 queue[kWarps][64];
     int queued = 0;
     auto drain = [&](int n) {  // lanes < n take a queued crossing each, then the queue shifts by n
         __syncwarp();
         if (lane < n) {
-            const int4 q = qpos[warp][lane];
-            const float2 f = qphi[warp][lane];
-            const bool s0 = above(f.x, lf, lexact, level);
-            add_crossing(&sacc[0][tid], kRedThreads, q.x, q.y, q.z, q.w, f.x, f.y, level, s0, zref);
+            const int4 q = queue[warp][lane];
+            const int r = q.y & 0x7FFFFFFF, z = r / ny;
+            add_crossing(&sacc[0][tid], kAngleThreads, q.x & 0x7FFFFFFF, r - z * ny, z,
+                         (int)((unsigned)q.x >> 31) | (int)((unsigned)q.y >> 31) << 1, __int_as_float(q.z), __int_as_float(q.w), A);
         }
         __syncwarp();
         if (lane + n < queued) {  // at most 31 left, read from [n, queued), written to [0, queued - n)
-            const int4 q = qpos[warp][lane + n];
-            const float2 f = qphi[warp][lane + n];
-            qpos[warp][lane] = q;
-            qphi[warp][lane] = f;
+            const int4 q = queue[warp][lane + n];
+            queue[warp][lane] = q;
         }
         __syncwarp();
         queued -= n;
     };
-    // a warp takes lattice rows (y, z) = w, w + W, ... (W warps in the grid), its lanes x = lane, lane + 32, ...
-    const int rows = ny * nz, nwarps = gridDim.x * (kRedThreads / 32);
-    for (int r = blockIdx.x * (kRedThreads / 32) + warp; r < rows; r += nwarps)
-    for (int xb = 0; xb < nx; xb += 32) {  // warp-uniform: the queue needs the whole warp
-        const int x = xb + lane;
-        const bool in = x < nx;
+    const int rows = ny * nz;
+    for (int r = blockIdx.x + warp * gridDim.x; r < rows; r += kWarps * gridDim.x) {
         const int z = r / ny, y = r - z * ny;
-        const unsigned i = (unsigned)r * (unsigned)nx + (unsigned)(in ? x : nx - 1);
-        // the node and its +x, +y, +z neighbours (the node itself past an edge), loaded together
-        const float p0 = P[i];
-        const float pn[3] = {P[in && x + 1 < nx ? i + 1 : i], P[y + 1 < ny ? i + nx : i], P[z + 1 < nz ? i + nxy : i]};
-        if (in && z == z0 && z0 + 1 < nz) {  // reference plane: every column, solid or not
-            const unsigned i1 = x + 1 < nx ? i + 1 : i - x;
-            ACC(1) += plane_length(p0, pn[2], P[i1], P[i1 + nxy], fz, level);
-        }
-        const bool fluid = in && (!F.general ? !(z == 0 || z == nz - 1) : (F.nbmask[F.L.off(x, y, z)] & kSelfSolid) == 0);
-        if (fluid) {
-            pmax = fmaxf(pmax, p0);
-            pmin = fminf(pmin, p0);
-        }
-        const bool s0 = above(p0, lf, lexact, level);
+        const float* __restrict__ R = P + (size_t)r * nx;
+        const size_t up_y = y + 1 < ny ? nx : 0, up_z = z + 1 < nz ? nxy : 0;  // past an edge: the node itself
+        // planar walls: the row is all fluid or all wall, and so is the one above it
+        const bool wall = !F.general && (z == 0 || z == nz - 1);
+        const bool wall_up = !F.general && z + 1 == nz - 1;
+        for (int xb = 0; xb < nx; xb += 32 * kStrips) {  // warp-uniform: the queue needs the whole warp
+            float p0[kStrips], py[kStrips], pz[kStrips];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const int x1 = x + (d == 0), y1 = y + (d == 1), z1 = z + (d == 2);
-            bool cross = fluid && x1 < nx && y1 < ny && z1 < nz;
-            if (cross) cross = !(F.general ? (F.nbmask[F.L.off(x1, y1, z1)] & kSelfSolid) != 0 : z1 == nz - 1);
-            if (cross) cross = s0 != above(pn[d], lf, lexact, level);
-            const unsigned m = __ballot_sync(0xffffffffu, cross);
-            if (cross) {
-                const int at = queued + __popc(m & ((1u << lane) - 1u));
-                qpos[warp][at] = make_int4(x, y, z, d);
-                qphi[warp][at] = make_float2(p0, pn[d]);
+            for (int s = 0; s < kStrips; ++s) {
+                const int x = xb + 32 * s + lane;
+                const float* q = R + (x < nx ? x : nx - 1);
+                p0[s] = q[0];
+                py[s] = q[up_y];
+                pz[s] = q[up_z];
             }
-            queued += __popc(m);
-            if (queued >= 32) drain(32);
+            const int xe = xb + 32 * kStrips;
+            const float pe = R[xe < nx ? xe : nx - 1];  // the node after the last strip
+#pragma unroll
+            for (int s = 0; s < kStrips; ++s) {
+                const int xs = xb + 32 * s, x = xs + lane;
+                if (xs >= nx) break;
+                const unsigned in = nx - xs >= 32 ? ~0u : (1u << (nx - xs)) - 1u;  // lanes on the lattice
+                if (z == A.z0 && z + 1 < nz && x < nx) {  // reference plane: every column, solid or not
+                    const int x1 = x + 1 < nx ? x + 1 : 0;
+                    const Two len = plane_length(p0[s], pz[s], R[x1], R[x1 + up_z], A);
+                    const float2 o = sacc[1][tid];
+                    const Two t = norm2(Two{o.x, o.y} + len);
+                    sacc[1][tid] = make_float2(t.h, t.l);
+                }
+                unsigned fluid = wall ? 0u : in, ok_x = in, ok_y = in, ok_z = wall_up ? 0u : in;
+                if (F.general) {
+                    auto open = [&](int xx, int yy, int zz) {
+                        return __ballot_sync(0xffffffffu, xx < nx && yy < ny && zz < nz &&
+                                                              (F.nbmask[F.L.off(xx, yy, zz)] & kSelfSolid) == 0);
+                    };
+                    fluid = open(x, y, z);
+                    ok_x = open(x + 1, y, z);
+                    ok_y = open(x, y + 1, z);
+                    ok_z = open(x, y, z + 1);
+                }
+                if ((fluid >> lane) & 1u) {
+                    pmax = fmaxf(pmax, p0[s]);
+                    pmin = fminf(pmin, p0[s]);
+                }
+                // the lanes above the level, and their +x, +y, +z neighbours above it (a neighbour past the
+                // lattice's edge is the node itself: no crossing; along x the last node's bit is cleared)
+                const unsigned b0 = __ballot_sync(0xffffffffu, above(p0[s], A));
+                const float next = s + 1 < kStrips ? __shfl_sync(0xffffffffu, p0[s + 1], 0) : pe;
+                const unsigned bx = b0 >> 1 | (above(next, A) ? 1u << 31 : 0u);
+                const unsigned by = __ballot_sync(0xffffffffu, above(py[s], A));
+                const unsigned bz = __ballot_sync(0xffffffffu, above(pz[s], A));
+                const unsigned in_x = nx - 1 - xs >= 32 ? ~0u : (1u << (nx - 1 - xs)) - 1u;
+                const unsigned m[3] = {(b0 ^ bx) & fluid & ok_x & in_x, (b0 ^ by) & fluid & ok_y, (b0 ^ bz) & fluid & ok_z};
+                if ((m[0] | m[1] | m[2]) == 0u) continue;
+                const float down = __shfl_down_sync(0xffffffffu, p0[s], 1);
+                const float px = lane == 31 ? next : down;
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    if (m[d] == 0u) continue;
+                    if ((m[d] >> lane) & 1u) {
+                        const int at = queued + __popc(m[d] & ((1u << lane) - 1u));
+                        queue[warp][at] = make_int4(x | (d & 1) << 31, r | (d >> 1) << 31, __float_as_int(p0[s]),
+                                                    __float_as_int(d == 0 ? px : (d == 1 ? py[s] : pz[s])));
+                    }
+                    queued += __popc(m[d]);
+                    if (queued >= 32) drain(32);
+                }
+            }
         }
     }
     if (queued > 0) drain(queued);
-    // block reduction: FP32 maxima by shuffles; FP64 values only in warps that hold some
-    __shared__ double sh[kRedThreads / 32][kAngleVals];
+    // block reduction: maxima by shuffles; warp w sums values w, w + kWarps, ... of all threads (each warp reducing its own
+    // lanes' sums took as many instructions as the rows)
+    __shared__ float lim[kWarps][2];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         pmax = fmaxf(pmax, __shfl_down_sync(0xffffffffu, pmax, o));
         pmin = fminf(pmin, __shfl_down_sync(0xffffffffu, pmin, o));
     }
     if (lane == 0) {
-        sh[warp][17] = pmax > -3.0e38f ? (double)pmax : -1e300;
-        sh[warp][18] = pmin < 3.0e38f ? -(double)pmin : -1e300;
+        lim[warp][0] = pmax;
+        lim[warp][1] = -pmin;
     }
-    for (int v = 0; v < 17; ++v) {
-        const bool is_max = v == 0;
-        double val = ACC(v);
-        // a contribution changed the value's bits from their start (integer test: no FP64 operation)
-        const bool held = __double_as_longlong(val) != __double_as_longlong(is_max ? -1e300 : 0.0);
-        if (__any_sync(0xffffffffu, held)) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const double w = __shfl_down_sync(0xffffffffu, val, o);
-                val = is_max ? fmax(val, w) : val + w;
-            }
-        }
-        if (lane == 0) sh[warp][v] = val;
-    }
-#undef ACC
+    auto join = [](int v, Two a, Two b) {  // the maximum (v = 0, 16, 17) or the sum
+        if (v != 0 && v < 16) return norm2(a + b);
+        return less2(a, b) ? b : a;
+    };
     __syncthreads();
-    if (tid < kAngleVals) {
-        const bool is_max = (kAngleMaxMask >> tid) & 1u;
-        double v = sh[0][tid];
-        for (int w = 1; w < kRedThreads / 32; ++w) v = is_max ? fmax(v, sh[w][tid]) : v + sh[w][tid];
-        part[(long long)blockIdx.x * kAngleVals + tid] = v;
+    for (int v = warp; v < 16; v += kWarps) {
+        Two val{sacc[v][lane].x, sacc[v][lane].y};
+#pragma unroll
+        for (int w = 1; w < kWarps; ++w) {
+            const float2 o = sacc[v][32 * w + lane];
+            val = join(v, val, Two{o.x, o.y});
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const Two w{__shfl_down_sync(0xffffffffu, val.h, o), __shfl_down_sync(0xffffffffu, val.l, o)};
+            val = join(v, val, w);
+        }
+        if (lane == 0) part[(size_t)v * gridDim.x + blockIdx.x] = make_float2(val.h, val.l);
     }
+    if (tid < 2) {
+        float v = lim[0][tid];
+        for (int w = 1; w < kWarps; ++w) v = fmaxf(v, lim[w][tid]);
+        part[(size_t)(16 + tid) * gridDim.x + blockIdx.x] = make_float2(v, 0.f);
+    }
+    __threadfence();
+    __shared__ bool last;
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // all blocks' values: warp w takes values w, w + kWarps, ... together, a lane the blocks lane, lane + 32, ... in
+    // order, eight of each in flight (one after the other this took as long as everything before it)
+    constexpr int kMine = (kAngleRow + kWarps - 1) / kWarps;
+    Two t[kMine];
+#pragma unroll
+    for (int i = 0; i < kMine; ++i) {
+        const int v = warp + i * kWarps;
+        t[i] = Two{v == 0 ? kNoTop : (v >= 16 ? -3.0e38f : 0.f), 0.f};
+    }
+    for (unsigned b0 = lane; b0 < gridDim.x; b0 += 32 * 8) {
+        float2 q[kMine][8];
+#pragma unroll
+        for (int i = 0; i < kMine; ++i)
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (warp + i * kWarps < kAngleRow && b0 + 32 * u < gridDim.x)
+                    q[i][u] = __ldcg(&part[(size_t)(warp + i * kWarps) * gridDim.x + b0 + 32 * u]);
+#pragma unroll
+        for (int i = 0; i < kMine; ++i)
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (warp + i * kWarps < kAngleRow && b0 + 32 * u < gridDim.x)
+                    t[i] = join(warp + i * kWarps, t[i], Two{q[i][u].x, q[i][u].y});
+    }
+#pragma unroll
+    for (int i = 0; i < kMine; ++i) {
+        const int v = warp + i * kWarps;
+        if (v >= kAngleRow) break;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const Two w{__shfl_down_sync(0xffffffffu, t[i].h, o), __shfl_down_sync(0xffffffffu, t[i].l, o)};
+            t[i] = join(v, t[i], w);
+        }
+        if (lane == 0) out[v] = v == 0 && t[i].h == kNoTop ? -1e300 : (v >= 16 && t[i].h == -3.0e38f ? -1e300 : to_f64(t[i]));
+    }
+    if (tid == 0) *ticket = 0u;
 }
 
 // ---------------------------------------------------------------- pressure tensor
@@ -520,50 +636,13 @@ __global__ void __launch_bounds__(kRedThreads) angle_kernel(FieldArgs F, Scratch
 // same bracket, so the interaction is 1/2 g kappa sum_k G_k [..] c_ki c_kj.
 // Components xx, yy, zz, xy, xz, yz; zero on solid nodes.
 //
-// FP64 runs at a sixtieth of the FP32 rate on this GPU, so the sums are taken
-// in pairs of FP32 numbers (Dekker 1971, Knuth's two-sum): a value is h + l
-// with l far below h, a sum carries the rounding error of h in l. That keeps
-// about 46 bits of the sums over exact FP32 inputs, 20 more than the stored
-// populations hold. With u common to both components the kinetic term is
+// The sums run in pairs of FP32 numbers: about 46 bits over exact FP32 inputs,
+// 20 more than the stored populations hold. With u common to both components the kinetic term is
 //   S_ij - u_i K_j - u_j J_i,  S = sum c c m,  J = sum c m,  K = J - u R,
 //   R = sum m,  m_k = n_k^r + n_k^b,
 // and S, J need the sums and differences of opposite velocities only. A node
 // whose result is not finite is taken again in FP64, so that infinities and
 // NaN come out as they always did.
-struct Two {
-    float h, l;
-};
-__device__ __forceinline__ Two two(float a) { return Two{a, 0.f}; }
-__device__ __forceinline__ Two two_sum(float a, float b)
-{
-    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-    return Two{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
-}
-// l may grow to a few roundings of h: normalised by norm2 before a product
-__device__ __forceinline__ Two operator+(Two a, Two b)
-{
-    const Two s = two_sum(a.h, b.h);
-    return Two{s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
-}
-__device__ __forceinline__ Two operator-(Two a) { return Two{-a.h, -a.l}; }
-__device__ __forceinline__ Two operator-(Two a, Two b) { return a + (-b); }
-__device__ __forceinline__ Two norm2(Two a)
-{
-    const float s = __fadd_rn(a.h, a.l);
-    return Two{s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
-}
-__device__ __forceinline__ Two mul2f(Two a, float f)  // a normalised
-{
-    const float p = __fmul_rn(a.h, f);
-    return Two{p, __fmaf_rn(a.l, f, __fmaf_rn(a.h, f, -p))};
-}
-__device__ __forceinline__ Two mul22(Two a, Two b)  // both normalised
-{
-    const float p = __fmul_rn(a.h, b.h);
-    return Two{p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)))};
-}
-__device__ __forceinline__ double to_f64(Two a) { return (double)a.h + (double)a.l; }
-
 // S_ij of values s[k] = v_k + v_kbar (k odd; entry (k - 1) / 2): xx, yy, zz, xy, xz, yz
 __device__ __forceinline__ void second_moment(const Two (&s)[9], Two (&S)[6], Two& XY, Two& XZ, Two& YZ)
 {
@@ -937,7 +1016,7 @@ cudaError_t launch_init(const FieldArgs& F, S* f, const double* rr, const double
 
 template <class S>
 cudaError_t launch_conservation(const FieldArgs& F, const S* f, unsigned long long* acc, unsigned int* ticket,
-                                double* out, cudaStream_t st, float* phi)
+                                double* out, const int* err, cudaStream_t st, float* phi)
 {
     // one wave of resident blocks (a grid-stride loop over the nodes): a partial
     // last wave of a fixed grid left most SMs idle at the end
@@ -952,7 +1031,7 @@ cudaError_t launch_conservation(const FieldArgs& F, const S* f, unsigned long lo
         else
             blocks = kConsBlocks;
     }
-    cons_kernel<S><<<blocks, kRedThreads, 0, st>>>(F, f, acc, ticket, out, phi);
+    cons_kernel<S><<<blocks, kRedThreads, 0, st>>>(F, f, acc, ticket, out, phi, err);
     return cudaGetLastError();
 }
 
@@ -973,11 +1052,23 @@ cudaError_t launch_phi(const FieldArgs& F, const S* f, const Scratch& W, cudaStr
     return cudaGetLastError();
 }
 
-cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, double level, double* part, double* out,
-                         cudaStream_t st)
+cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, double level, double* part,
+                         unsigned int* ticket, double* out, cudaStream_t st)
 {
-    angle_kernel<<<kAngleBlocks, kRedThreads, 0, st>>>(F, W, zref, level, part);
-    finish_rows_kernel<kAngleVals><<<kAngleVals, 256, 0, st>>>(part, kAngleBlocks, kAngleMaxMask, out);
+    AngleArgs A;
+    auto split = [](double v, float& h, float& l) {
+        h = (float)v;
+        l = (float)(v - (double)h);
+    };
+    split(level, A.lh, A.ll);
+    A.least = level < (double)A.lh ? A.lh : std::nextafterf(A.lh, INFINITY);
+    split(zref, A.zh, A.zl);
+    const double z0 = std::floor(zref);
+    split(zref - z0, A.fzh, A.fzl);
+    A.z0 = z0 < (double)F.L.nz ? (int)z0 : F.L.nz;
+    const int rows = F.L.ny * F.L.nz, warps = kAngleThreads / 32;
+    const int blocks = (rows + warps - 1) / warps < kAngleBlocks ? (rows + warps - 1) / warps : kAngleBlocks;
+    angle_kernel<<<blocks, kAngleThreads, 0, st>>>(F, A, W.rho[0], (float2*)part, ticket, out);
     return cudaGetLastError();
 }
 
@@ -1032,7 +1123,7 @@ cudaError_t launch_pressure_radial(const FieldArgs& F, const S* f, const Scratch
 #define LBSC_INST(S)                                                                                  \
     template cudaError_t launch_init<S>(const FieldArgs&, S*, const double*, const double*, cudaStream_t, int*); \
     template cudaError_t launch_conservation<S>(const FieldArgs&, const S*, unsigned long long*, unsigned int*, \
-                                                double*, cudaStream_t, float*);                                \
+                                                double*, const int*, cudaStream_t, float*);                    \
     template cudaError_t launch_fields<S>(const FieldArgs&, const S*, const Scratch&, bool, cudaStream_t); \
     template cudaError_t launch_phi<S>(const FieldArgs&, const S*, const Scratch&, cudaStream_t);      \
     template cudaError_t launch_get_pop<S>(const FieldArgs&, const S*, double*, cudaStream_t);       \

@@ -9,10 +9,20 @@ namespace lbsc {
 
 constexpr int kRedThreads = 256;  // threads per reduction block
 constexpr int kConsBlocks = 2048;   // most blocks of the conservation sums (one wave of resident blocks is used)
-constexpr int kAngleBlocks = 1216;  // fixed grid of the contact-angle reduction
-constexpr int kAngleVals = 19;    // contact-angle partial sums per block
-constexpr int kPartRows = kConsBlocks > kAngleBlocks ? kConsBlocks : kAngleBlocks;  // rows of the partials area
-constexpr uint32_t kAngleMaxMask = (1u << 0) | (1u << 17) | (1u << 18);  // max-reduced entries of the 19
+constexpr int kAngleBlocks = 456;  // most blocks of the contact-angle reduction (3 per SM)
+constexpr int kAngleThreads = 256;
+constexpr int kAngleRow = 18;     // contact-angle values per block (angle_kernel)
+constexpr float kNoTop = -3.0e38f;  // the top crossing where there is none
+constexpr int kPartRows = kConsBlocks;  // rows of the partials area
+constexpr int kPartVals = 19;           // doubles a row
+
+// The contact angle's level (lh + ll) and the least FP32 number above it, the
+// reference height zref (zh + zl), its plane z0 (nz where that lies outside)
+// and fraction there, in pairs of FP32 numbers.
+struct AngleArgs {
+    float lh, ll, least, zh, zl, fzh, fzl;
+    int z0;
+};
 
 // Geometry and parameters for the non-step kernels.
 struct FieldArgs {
@@ -93,20 +103,23 @@ cudaError_t launch_clock_set(uint32_t* clk, uint32_t v, cudaStream_t st);
 template <class S>
 cudaError_t launch_init(const FieldArgs& F, S* f, const double* rr, const double* rb, cudaStream_t st,
                         int* err = nullptr);
-// FP64 conservation sums into out[0..7] through 64-bit fixed-point accumulators
+// FP64 conservation sums into out[0..6] and the status word *err into out[7]
+// (out may be pinned host memory), through 64-bit fixed-point accumulators
 // acc[0..6] and a block ticket, both zero between calls (the kernel clears them)
 constexpr float kConsFix = 268435456.0f;  // 2^28: the accumulators' unit is 2^-28
 // phi (optional): also write phi = rho_r - rho_b of every node, as launch_phi does
 template <class S>
 cudaError_t launch_conservation(const FieldArgs& F, const S* f, unsigned long long* acc, unsigned int* ticket,
-                                double* out, cudaStream_t st, float* phi = nullptr);
+                                double* out, const int* err, cudaStream_t st, float* phi = nullptr);
 template <class S>
 cudaError_t launch_fields(const FieldArgs& F, const S* f, const Scratch& W, bool velocity, cudaStream_t st);
 // phi = rho_r - rho_b of every node into W.rho[0] (the contact angle's input)
 template <class S>
 cudaError_t launch_phi(const FieldArgs& F, const S* f, const Scratch& W, cudaStream_t st);
-cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, double level, double* part, double* out,
-                         cudaStream_t st);
+// the contact angle's 18 values of phi in W.rho[0] (angle_kernel) into out; part: kAngleRow doubles a
+// block, ticket: a counter that is 0 between calls
+cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, double level, double* part,
+                         unsigned int* ticket, double* out, cudaStream_t st);
 // pressure tensor of Sec. 4.1 (after launch_fields): every node, per-plane
 // sums (part: 8 nz split doubles of scratch), and fixed-point radial bins (see fields.cu)
 constexpr int kPressThreads = 128;

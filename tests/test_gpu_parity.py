@@ -643,3 +643,29 @@ def test_psi_series_within_one_ulp_and_packed_lanes_identical(lbsc):
     lib_err = np.abs(lib_ref.astype(np.float64) - exact) / ulp
     assert err.max() <= 1.0, (err.max(), rho[np.argmax(err)])
     assert err.max() <= lib_err.max() + 0.25, (err.max(), lib_err.max())
+
+
+@pytest.mark.parametrize("dims,offset", [((1, 1, 10), 1.0), ((31, 7, 9), 2.25), ((33, 9, 12), 0.0), ((128, 6, 11), 5.0),
+                                         ((161, 5, 14), 3.5), ((47, 40, 24), 40.0)])
+def test_contact_angle_sums_on_ragged_lattices(lbsc, dims, offset):
+    """Many crossings in every direction (a wavy phi with noise), rows shorter and longer than a warp's four strips, the
+    level on a node's own value: the oracle's construction on the same phi. Counts exactly; lengths and coordinates from
+    46-bit sums of at most 3 N points, through a 4 x 4 solve: 1e-7."""
+    nx, ny, nz = dims
+    z, y, x = np.meshgrid(np.arange(nz), np.arange(ny), np.arange(nx), indexing="ij")
+    rng = np.random.Generator(np.random.PCG64(nx))
+    s = np.sin(0.7 * x) * np.cos(0.4 * y) * np.sin(0.5 * z + 0.3) + rng.uniform(-0.2, 0.2, size=z.shape)
+    lat = lbsc.Lattice(0.4 + 0.25 * s, 0.4 - 0.25 * s)
+    r, b, _, _ = lat.moments()
+    solid = W.wall_mask(nx, ny, nz)
+    phi = (r.astype(np.float32) - b.astype(np.float32)).astype(np.float64)
+    for level in (0.0, float(phi[nz // 2, ny // 2, nx // 2]), 0.37 * float(phi.max())):
+        d = lat.contact_angle(offset, level=level)
+        o = oracle.contact_angle(phi, 0 * phi, solid, offset, level)
+        assert d["n_points"] == o["n_points"]
+        assert d["phi_max"] == phi[1:-1].max() and d["phi_min"] == phi[1:-1].min()
+        # a reference plane that touches a solid layer: the library takes phi = 0 there, the oracle phi = level
+        walled = level != 0.0 and (int(0.5 + offset) == 0 or int(0.5 + offset) + 1 == nz - 1)
+        for k in ("h", "theta_fit_deg", "xc", "yc", "zc", "r_fit") + (() if walled else ("b", "r", "base_ref", "theta_deg")):
+            if o[k] > -1e290:
+                assert abs(d[k] - o[k]) <= 1e-7 * max(1.0, abs(o[k])), (k, level, d[k], o[k])
