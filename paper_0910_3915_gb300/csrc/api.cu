@@ -18,6 +18,14 @@ int step_occupancy(int precision, int tile_y, bool general, bool tau_one);
 
 }
 
+namespace {
+// The step kernel's split of the work: tile height, even row splits, z
+// segments per tile column, and stages of the TMA kernel (0: the load-from-global one).
+struct Schedule {
+    int ty = 0, yt = 0, nseg = 0, ns = 0;
+};
+}  // namespace
+
 struct lb_ctx {
     int nx = 0, ny = 0, nz = 0, prec = LB_F32;
     Layout L{};
@@ -39,9 +47,9 @@ struct lb_ctx {
     Scratch W{};
     lb_params prm{};
     KParams kp{};
-    int tile_y = 4, nseg_req = 0;
-    int y_tiles_req = 0;  // y-tiles of the step kernel (0 = ceil(ny / tile_y))
-    int nseg_cache = 0;  // segments per tile column for the current schedule (0 = not computed)
+    // the caller's choices (0 = automatic), and the schedule the steps run with
+    int tile_y_req = 0, y_tiles_req = 0, nseg_req = 0;
+    Schedule sched;  // ty = 0: not chosen since the last change
     long long steps = 0;
     // CUDA graphs of 2^i steps (i = 0 .. kGraphLevels - 1) for each starting buffer
     static constexpr int kGraphLevels = 6;
@@ -139,7 +147,7 @@ static FieldArgs field_args(const lb_ctx* c)
 
 static void drop_graphs(lb_ctx* c)
 {
-    c->nseg_cache = 0;
+    c->sched = Schedule{};
     for (int p = 0; p < 2; ++p)
         for (int i = 0; i < lb_ctx::kGraphLevels; ++i)
             if (c->graph[p][i]) {
@@ -163,32 +171,6 @@ static void set_kparams(lb_ctx* c)
 }
 
 static bool tau_one(const lb_ctx* c) { return c->prm.tau_r == 1.0 && c->prm.tau_b == 1.0; }
-
-static int tma_stages(lb_ctx* c);
-static long long tma_call(int op, lb_ctx* c, int ty, int ns);
-
-static int y_tiles(const lb_ctx* c)
-{
-    return c->y_tiles_req > 0 ? c->y_tiles_req : (c->ny + c->tile_y - 1) / c->tile_y;
-}
-
-static int nseg_for(lb_ctx* c, int ncol)
-{
-    if (c->nseg_cache > 0) return c->nseg_cache;
-    const int nzf = c->zhi - c->zlo;
-    if (c->nseg_req > 0) return c->nseg_cache = (c->nseg_req < nzf ? c->nseg_req : nzf);
-    const int ns = tma_stages(c);
-    int occ = ns ? (int)tma_call(2, c, c->tile_y, ns) : step_occupancy(c->prec, c->tile_y, c->general, tau_one(c));
-    if (occ < 1) occ = 1;
-    const long long target = 2LL * c->nsm * occ;  // about two waves of CTAs
-    long long s = (target + ncol - 1) / ncol;
-    const long long smax = nzf / 16 > 1 ? nzf / 16 : 1;  // segments of at least 16 planes
-    if (s > smax) s = smax;
-    if (s < 1) s = 1;
-    c->nseg_cache = (int)s;
-    return (int)s;
-}
-
 
 // ---------------------------------------------------------------- TMA step support
 static const int kTmaTiles[3] = {4, 8, 16};
@@ -221,20 +203,93 @@ static cudaError_t tma_prepare(lb_ctx* c)
     return cudaSuccess;
 }
 
-// stages used by the TMA kernel for the current schedule, 0 if not available
-static int tma_stages(lb_ctx* c)
+// Estimated time in microseconds of a step of the TMA kernel on tiles of ty
+// rows and ns stages, `items` CTAs of which `occ` fit an SM, each taking p
+// planes (two of them for psi alone): a CTA's planes follow each other, one
+// taking a + b k microseconds beside k - 1 other CTAs of its SM, so a wave of
+// CTAs lasts p (a + b k); and the populations' traffic, with the planes read
+// twice, takes its time in HBM (or in L2, where both buffers fit). a, b and c
+// (the launch) are fitted to 700 schedules of 22 lattices from 24 x 24 x 100
+// to 256 x 256 x 128 (rms 7-13%): what the estimate picks is within 8% of the
+// best of those, 1.3% from it on average. A fixed 4 rows, one stage and segments
+// of at least 16 planes left 8 CTAs on 152 SMs at 32^3 (49 us a step, now 4.9),
+// 96 at 64^3 (38, now 16), and 1.5 waves at 128^3 (121, now 109).
+static double estimate(const lb_ctx* c, int ty, int ns, int occ, long long items, int p)
 {
-    // general geometry always loads from global; AUTO takes the TMA kernel
-    // with one stage (measured the faster one for both precisions)
-    if (c->general || c->variant == LB_STEP_LDG) return 0;
-    const int s0 = c->variant == LB_STEP_AUTO ? 1 : 3, s1 = c->variant == LB_STEP_AUTO ? 1 : 2;
-    const int want[2] = {c->stages ? c->stages : s0, c->stages ? c->stages : s1};
-    for (int ns : want) {
-        // occupancy 0: the pair is not built for this precision (or does not fit)
-        const long long occ = tma_call(2, c, c->tile_y, ns);
-        if (occ > 0) return ns;
+    struct Fit {
+        double a, b, c;
+    };
+    static const Fit fit[2][2][2] = {{{{2.35, 0.06, 0.2}, {1.28, 0.12, 0.2}}, {{2.45, 0.19, 0.8}, {0.77, 0.98, 0.4}}},
+                                     {{{2.12, 0.15, 2.7}, {1.45, 0.26, 3.5}}, {{2.17, 0.40, 2.0}, {2.01, 0.23, 2.4}}}};
+    static const Fit unequal = {1.3, 0.05, 3.0};  // tau != 1, two stages
+    const bool half = c->prec != LB_F32;
+    const Fit& f = tau_one(c) ? fit[half][ty > 4][ns > 1] : unequal;
+    const long long slots = (long long)c->nsm * occ, waves = items / slots, rem = items - waves * slots;
+    double t = f.c + (double)waves * p * (f.a + f.b * occ);
+    if (rem) t += p * (f.a + f.b * (double)((rem + c->nsm - 1) / c->nsm));
+    const double pops = (double)c->fluid_nodes * 2 * Q * elem_size(c->prec), rate = 2 * pops > 100e6 ? 6.2e6 : 16e6;
+    const double m = pops * (2.0 + 1.0 / (p > 3 ? p - 2 : 1)) / rate;
+    // CTAs at the edges take longer; with several waves that evens out
+    const double uneven = 1.0 + 0.1 / (double)(waves + (rem ? 1 : 0));
+    return uneven * std::sqrt(std::sqrt(t * t * t * t + m * m * m * m));
+}
+
+// The schedule of the context's steps: the caller's choices, and for what was
+// left open the least estimate among one to three waves of resident CTAs and
+// even row splits of up to a third more tiles than needed. Chosen once after
+// every change of schedule, parameters or geometry; it changes no value.
+static const Schedule& schedule(lb_ctx* c)
+{
+    if (c->sched.ty) return c->sched;
+    const int nzf = c->zhi - c->zlo, ntx = (c->nx + 31) / 32, ny = c->ny;
+    Schedule best;
+    double least = 0;
+    const int tys[2] = {c->tile_y_req ? c->tile_y_req : 4, c->tile_y_req || c->prec == LB_F32 || !tau_one(c) ? 0 : 8};
+    // a general geometry loads from global; TMA asked for by name takes three stages, else two
+    for (int ty : tys) {
+        if (!ty || c->general || c->variant == LB_STEP_LDG) continue;
+        int stages[2] = {1, 2};
+        if (c->variant == LB_STEP_TMA) stages[0] = 3;
+        if (!tau_one(c) && c->variant == LB_STEP_AUTO) stages[0] = 2;  // holds v in fewer registers than one stage does
+        if (c->stages) stages[0] = stages[1] = c->stages;
+        for (int i = 0; i < 2; ++i) {
+            const int ns = stages[i];
+            if (i && (ns == stages[0] || (best.ty == ty && c->variant == LB_STEP_TMA))) break;
+            // occupancy 0: the pair is not built for this precision (or does not fit)
+            const int occ = (int)tma_call(2, c, ty, ns);
+            if (occ < 1) continue;
+            const int base = (ny + ty - 1) / ty;
+            const int yt0 = c->y_tiles_req ? c->y_tiles_req : base;
+            const int yt1 = c->y_tiles_req ? yt0 : (base + base / 3 < ny ? base + base / 3 : ny);
+            for (int yt = yt0; yt <= yt1; ++yt) {
+                if (yt > yt0 && (ny + yt - 1) / yt < ty - 1) break;
+                for (int w = 1; w <= 3; ++w) {
+                    const long long col = (long long)ntx * yt;
+                    long long seg = c->nseg_req ? c->nseg_req : (long long)w * c->nsm * occ / col;
+                    seg = seg < 1 ? 1 : (seg > nzf ? nzf : seg);
+                    const double t = estimate(c, ty, ns, occ, col * seg, (int)((nzf + seg - 1) / seg) + 2);
+                    if (!best.ty || t < least) {
+                        best = Schedule{ty, yt, (int)seg, ns};
+                        least = t;
+                    }
+                    if (c->nseg_req) break;
+                }
+            }
+        }
     }
-    return 0;
+    if (!best.ty) {
+        // load from global: about two waves of CTAs, segments of at least 16 planes
+        best.ty = tys[0];
+        best.yt = c->y_tiles_req ? c->y_tiles_req : (ny + best.ty - 1) / best.ty;
+        int occ = step_occupancy(c->prec, best.ty, c->general, tau_one(c));
+        if (occ < 1) occ = 1;
+        const long long ncol = (long long)ntx * best.yt;
+        long long seg = (2LL * c->nsm * occ + ncol - 1) / ncol;
+        const long long smax = nzf / 16 > 1 ? nzf / 16 : 1;
+        seg = c->nseg_req ? c->nseg_req : (seg > smax ? smax : seg);
+        best.nseg = (int)(seg < 1 ? 1 : (seg > nzf ? nzf : seg));
+    }
+    return c->sched = best;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -267,7 +322,10 @@ static int encode_maps(lb_ctx* c, void* f, int ty, CUtensorMap (&maps)[4])
     if (!enc) return fail(c, LB_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
     const size_t es = elem_size(c->prec);
     const Layout& L = c->L;
-    const cuuint64_t dims[4] = {(cuuint64_t)(2 * L.px), (cuuint64_t)(L.ny + 2), (cuuint64_t)L.nz, (cuuint64_t)Q};
+    // the maps end with the lattice's last column: a box reads nothing past it (padding that no step
+    // writes would miss L2 in every step)
+    const cuuint64_t dims[4] = {(cuuint64_t)(2 * (L.gx + L.nx)), (cuuint64_t)(L.ny + 2), (cuuint64_t)L.nz,
+                                (cuuint64_t)Q};
     const cuuint64_t strides[3] = {(cuuint64_t)(2 * L.px) * es, (cuuint64_t)(2 * L.plane) * es,
                                    (cuuint64_t)(2 * L.slot) * es};
     // No L2 promotion: fetching whole 256-byte blocks around the boxes' 16-byte edges raised the
@@ -311,47 +369,38 @@ static StepArgs<S> step_args(lb_ctx* c, int src)
     A.L = c->L;
     A.P = c->kp;
     A.tiles_x = (c->nx + 31) / 32;
-    A.tiles_y = y_tiles(c);
+    A.tiles_y = schedule(c).yt;
     A.zlo = c->zlo;
     A.zhi = c->zhi;
-    A.nseg = nseg_for(c, A.tiles_x * A.tiles_y);
+    A.nseg = schedule(c).nseg;
     A.halo = c->halo;
     A.hkey = c->hkey;
     return A;
 }
 
-// one TMA-staged step
+// one step of the lattice's schedule from buffer `src`
 template <class S>
-static cudaError_t launch_tma(lb_ctx* c, int parity, int ns, cudaStream_t st)
+static cudaError_t launch_one_step(lb_ctx* c, int src, cudaStream_t st)
 {
-    const StepArgs<S> A = step_args<S>(c, parity);
-    return (cudaError_t)tma_step<S>(0, c->tile_y, ns, tau_one(c), c->tmap[parity][tile_index(c->tile_y)], &A, st);
+    const StepArgs<S> A = step_args<S>(c, src);
+    const Schedule& d = schedule(c);
+    if (d.ns) return (cudaError_t)tma_step<S>(0, d.ty, d.ns, tau_one(c), c->tmap[src][tile_index(d.ty)], &A, st);
+    return launch_step<S>(A, d.ty, c->general, tau_one(c), st);
 }
 
 static cudaError_t launch_steps(lb_ctx* c, int n, int& parity, cudaStream_t st)
 {
-    const bool t1 = tau_one(c);
-    const int ns = tma_stages(c);
-    if (ns) {
+    const Schedule& d = schedule(c);
+    if (d.ns) {
         for (int b = 0; b < 2; ++b)
-            if (tensor_map(c, b, c->tile_y) != LB_OK) return cudaErrorInvalidValue;
+            if (tensor_map(c, b, d.ty) != LB_OK) return cudaErrorInvalidValue;
     }
     for (int i = 0; i < n; ++i) {
         cudaError_t e;
-        if (ns) {
-            switch (c->prec) {
-            case LB_F32: e = launch_tma<float>(c, parity, ns, st); break;
-            case LB_F16: e = launch_tma<__half>(c, parity, ns, st); break;
-            default: e = launch_tma<__nv_bfloat16>(c, parity, ns, st); break;
-            }
-            if (e != cudaSuccess) return e;
-            parity ^= 1;
-            continue;
-        }
         switch (c->prec) {
-        case LB_F32: e = launch_step<float>(step_args<float>(c, parity), c->tile_y, c->general, t1, st); break;
-        case LB_F16: e = launch_step<__half>(step_args<__half>(c, parity), c->tile_y, c->general, t1, st); break;
-        default: e = launch_step<__nv_bfloat16>(step_args<__nv_bfloat16>(c, parity), c->tile_y, c->general, t1, st); break;
+        case LB_F32: e = launch_one_step<float>(c, parity, st); break;
+        case LB_F16: e = launch_one_step<__half>(c, parity, st); break;
+        default: e = launch_one_step<__nv_bfloat16>(c, parity, st); break;
         }
         if (e != cudaSuccess) return e;
         parity ^= 1;
@@ -722,7 +771,7 @@ int lb_set_tiling(lb_ctx* c, int tile_y, int y_tiles, int z_segments)
     if (y_tiles > 0 && (long long)((c->nx + 31) / 32) * y_tiles * (z_segments > 0 ? z_segments : 1) > (1LL << 30))
         return fail(c, LB_ERR_ARG, "lb_set_tiling: too many tiles");
     drop_graphs(c);
-    c->tile_y = tile_y;
+    c->tile_y_req = tile_y;
     c->y_tiles_req = y_tiles;
     c->nseg_req = z_segments;
     return LB_OK;
@@ -740,7 +789,7 @@ int lb_set_schedule(lb_ctx* c, int tile_y, int z_segments)
 static int capture_graphs(lb_ctx* c)
 {
     if (c->graph[0][0]) return LB_OK;
-    nseg_for(c, ((c->nx + 31) / 32) * y_tiles(c));
+    schedule(c);
     for (int p = 0; p < 2; ++p)
         for (int i = 0; i < lb_ctx::kGraphLevels; ++i) {
             cudaGraph_t g = nullptr;
@@ -761,7 +810,6 @@ int lb_step(lb_ctx* c, int nsteps)
 {
     if (!c || nsteps < 0) return fail(c, LB_ERR_ARG, "lb_step: bad argument");
     if (nsteps == 0) return LB_OK;
-    const int ns = tma_stages(c);
     // n steps as graphs of 2^i steps: one launch per set bit (and per 32 steps),
     // so that consecutive kernels follow each other without host launch gaps
     const int rc = capture_graphs(c);
@@ -1165,6 +1213,7 @@ struct lb_batch {
     int4* ditems = nullptr; // (box, tile column, first plane, end plane)
     void* dmaps = nullptr;  // TMA variant: the four tensor maps of box i, source buffer p, at 2*i + p
     int nitems = 0;
+    int tile_y_req = 0, seg_planes_req = 0;  // the caller's choices (0 = automatic)
     int tile_y = 8, seg_planes = 32, ctas_per_sm = 0, grid = 0;
     int variant = LB_STEP_AUTO;
     bool tma = false;       // the TMA-staged batch kernel runs the steps
@@ -1197,27 +1246,78 @@ static void batch_drop_graphs(lb_batch* b)
         }
 }
 
+// nseg segments of about `planes` planes of a box's fluid planes
+static int batch_segments(const lb_ctx* c, int planes)
+{
+    const int nzf = c->zhi - c->zlo, nseg = (nzf + planes / 2) / planes;
+    return nseg < 1 ? 1 : (nseg > nzf ? nzf : nseg);
+}
+
+// the work list for `planes` planes an item, and the planes (two more an item
+// than it updates) of the CTA that has most when `grid` CTAs take it in turns
+static long long batch_items(const lb_batch* b, int planes, int grid, std::vector<int4>* items)
+{
+    std::vector<long long> load((size_t)grid, 0);
+    size_t n = 0;
+    for (int i = 0; i < b->nbox; ++i) {
+        const lb_ctx* c = b->box[i];
+        const int cols = (c->nx + 31) / 32 * ((c->ny + b->tile_y - 1) / b->tile_y), nzf = c->zhi - c->zlo;
+        const int nseg = batch_segments(c, planes);
+        for (int s = 0; s < nseg; ++s) {
+            const int za = c->zlo + (int)((long long)s * nzf / nseg), zb = c->zlo + (int)((long long)(s + 1) * nzf / nseg);
+            if (za >= zb) continue;
+            for (int col = 0; col < cols; ++col, ++n) {
+                load[n % (size_t)grid] += zb - za + 2;
+                if (items) items->push_back(make_int4(i, col, za, zb));
+            }
+        }
+    }
+    long long most = 0;
+    for (long long l : load) most = l > most ? l : most;
+    return most;
+}
+
 template <class S>
 static int batch_build_typed(lb_batch* b)
 {
     std::vector<StepArgs<S>> args(2 * (size_t)b->nbox);
     std::vector<int4> items;
     b->tau1 = true;
-    for (int i = 0; i < b->nbox; ++i) {
-        lb_ctx* c = b->box[i];
-        c->tile_y = b->tile_y;
-        b->tau1 = b->tau1 && tau_one(c);
-        for (int p = 0; p < 2; ++p) args[2 * i + p] = step_args<S>(c, p);
-        const int tx = (c->nx + 31) / 32, ty = (c->ny + b->tile_y - 1) / b->tile_y;
-        const int nzf = c->zhi - c->zlo;
-        int nseg = (nzf + b->seg_planes / 2) / b->seg_planes;
-        nseg = nseg < 1 ? 1 : (nseg > nzf ? nzf : nseg);
-        for (int s = 0; s < nseg; ++s) {
-            const int za = c->zlo + (int)((long long)s * nzf / nseg), zb = c->zlo + (int)((long long)(s + 1) * nzf / nseg);
-            if (za >= zb) continue;
-            for (int col = 0; col < tx * ty; ++col) items.push_back(make_int4(i, col, za, zb));
+    for (const lb_ctx* c : b->box) b->tau1 = b->tau1 && tau_one(c);
+    // AUTO and TMA take the TMA-staged batch kernel where it is built (one
+    // stage, 4- or 8-row tiles); LDG the load-from-global one
+    // (the shared-memory attribute first: the occupancy of a kernel above 48 KB counts 0 without it)
+    const bool want_tma = b->variant != LB_STEP_LDG;
+    b->tile_y = b->tile_y_req ? b->tile_y_req : (want_tma && b->prec == LB_F32 ? 4 : 8);
+    b->tma = want_tma &&
+             tma_batch<S>(1, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr) ==
+                 (long long)cudaSuccess &&
+             tma_batch<S>(2, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr) > 0;
+    const int occ = b->ctas_per_sm > 0
+                        ? b->ctas_per_sm
+                        : (b->tma ? (int)tma_batch<S>(2, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0,
+                                                      nullptr, 0, nullptr)
+                                  : batch_occupancy<S>(b->tile_y, b->tau1));
+    b->grid = b->box[0]->nsm * (occ > 0 ? occ : 1);
+    // Planes an item, where the caller leaves them open: those that give the
+    // busiest CTA least. Long items repeat fewer planes, short ones share out
+    // better: 12 boxes of edge 48-96 took %BATCH%
+    b->seg_planes = b->seg_planes_req ? b->seg_planes_req : 32;
+    if (!b->seg_planes_req) {
+        long long least = 0;
+        for (int planes : {64, 48, 32, 24, 20, 16, 12, 10, 8, 6, 4, 3, 2, 1}) {
+            const long long most = batch_items(b, planes, b->grid, nullptr);
+            if (least && most >= least) continue;
+            least = most;
+            b->seg_planes = planes;
         }
     }
+    batch_items(b, b->seg_planes, b->grid, &items);
+    for (int i = 0; i < b->nbox; ++i)
+        for (int p = 0; p < 2; ++p) {
+            args[2 * i + p] = step_args<S>(b->box[i], p);
+            args[2 * i + p].tiles_y = (b->box[i]->ny + b->tile_y - 1) / b->tile_y;
+        }
     if (b->dargs) cudaFree(b->dargs);
     if (b->ditems) cudaFree(b->ditems);
     if (b->dmaps) cudaFree(b->dmaps);
@@ -1232,13 +1332,6 @@ static int batch_build_typed(lb_batch* b)
     LB_BCUDA(b, cudaMemcpy(b->dargs, args.data(), args.size() * sizeof(StepArgs<S>), cudaMemcpyHostToDevice));
     LB_BCUDA(b, cudaMemcpy(b->ditems, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice));
     b->nitems = (int)items.size();
-    // AUTO and TMA take the TMA-staged batch kernel where it is built (one
-    // stage, 4- or 8-row tiles); LDG the load-from-global one
-    // (the shared-memory attribute first: the occupancy of a kernel above 48 KB counts 0 without it)
-    b->tma = b->variant != LB_STEP_LDG &&
-             tma_batch<S>(1, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr) ==
-                 (long long)cudaSuccess &&
-             tma_batch<S>(2, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr) > 0;
     if (b->tma) {
         std::vector<CUtensorMap> maps(8 * (size_t)b->nbox);
         for (int i = 0; i < b->nbox; ++i) {
@@ -1252,12 +1345,6 @@ static int batch_build_typed(lb_batch* b)
         LB_BCUDA(b, cudaMalloc(&b->dmaps, maps.size() * sizeof(CUtensorMap)));  // 256-byte aligned
         LB_BCUDA(b, cudaMemcpy(b->dmaps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice));
     }
-    const int occ = b->ctas_per_sm > 0
-                        ? b->ctas_per_sm
-                        : (b->tma ? (int)tma_batch<S>(2, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0,
-                                                      nullptr, 0, nullptr)
-                                  : batch_occupancy<S>(b->tile_y, b->tau1));
-    b->grid = b->box[0]->nsm * (occ > 0 ? occ : 1);
     return LB_OK;
 }
 
@@ -1368,8 +1455,8 @@ int lb_batch_set_schedule(lb_batch* b, int tile_y, int planes_per_item, int ctas
 {
     if (!b || (tile_y != 4 && tile_y != 8 && tile_y != 16) || planes_per_item < 1 || ctas_per_sm < 0)
         return bfail(b, LB_ERR_ARG, "lb_batch_set_schedule: tile_y 4/8/16, planes_per_item >= 1, ctas_per_sm >= 0");
-    b->tile_y = tile_y;
-    b->seg_planes = planes_per_item;
+    b->tile_y_req = tile_y;
+    b->seg_planes_req = planes_per_item;
     b->ctas_per_sm = ctas_per_sm;
     return batch_build(b);
 }
@@ -1506,8 +1593,9 @@ static cudaError_t adj_step_into(lb_ctx* c, const void* src, void* dst, int ns, 
     StepArgs<S> A = step_args<S>(c, 0);
     A.src = (const S*)src;
     A.dst = (S*)dst;
-    if (ns) return (cudaError_t)tma_step<S>(0, c->tile_y, ns, tau_one(c), maps, &A, st);
-    return launch_step<S>(A, c->tile_y, c->general, tau_one(c), st);
+    const int ty = schedule(c).ty;
+    if (ns) return (cudaError_t)tma_step<S>(0, ty, ns, tau_one(c), maps, &A, st);
+    return launch_step<S>(A, ty, c->general, tau_one(c), st);
 }
 
 template <class S>
@@ -1585,11 +1673,11 @@ extern "C" int lb_step_backward(lb_ctx* c, int nsteps, int ckpt_every, int obser
         G.omega[a] = c->kp.itau[a];
         G.eta[a] = c->kp.eta[a];
     }
-    const int ns = tma_stages(c);
+    const int ns = schedule(c).ns;
     CUtensorMap maps[2][4];
     if (ns && nseg > 0)
         for (int b = 0; b < 2; ++b) {
-            const int rc = encode_maps(c, store + sb * (size_t)b, c->tile_y, maps[b]);
+            const int rc = encode_maps(c, store + sb * (size_t)b, schedule(c).ty, maps[b]);
             if (rc != LB_OK) return rc;
         }
     auto step_of = [&](int b, cudaStream_t s2) -> cudaError_t {  // store[b] -> store[1 - b]

@@ -1018,16 +1018,16 @@ template <class S>
 cudaError_t launch_conservation(const FieldArgs& F, const S* f, unsigned long long* acc, unsigned int* ticket,
                                 double* out, const int* err, cudaStream_t st, float* phi)
 {
-    // one wave of resident blocks (a grid-stride loop over the nodes): a partial
-    // last wave of a fixed grid left most SMs idle at the end
+    // one wave of resident blocks (a grid-stride loop over the nodes): a partial last wave of a fixed grid left most SMs
+    // idle at the end. A thread adds its nodes in FP32, so the grid is part of the result: four blocks an SM for FP32,
+    // five for 16-bit storage, whatever the registers of a build would admit
     static int blocks = 0;
     if (!blocks) {
-        int dev = 0, nsm = 0, occ = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) ==
-                                                      cudaSuccess &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cons_kernel<S>, kRedThreads, 0) == cudaSuccess &&
-            nsm * occ > 0)
-            blocks = nsm * occ < kConsBlocks ? nsm * occ : kConsBlocks;
+        int dev = 0, nsm = 0;
+        const int per = sizeof(S) == 4 ? 4 : 5;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && nsm > 0)
+            blocks = nsm * per < kConsBlocks ? nsm * per : kConsBlocks;
         else
             blocks = kConsBlocks;
     }

@@ -273,6 +273,30 @@ __device__ __forceinline__ void clock_tick(uint32_t* clk)
     }
 }
 
+// Programmatic dependent launch: a kernel launched by launch_after may start
+// while the kernel before it in its stream still runs, once all of that one's
+// CTAs have called grid_trigger (or ended). Everything before its grid_wait
+// must touch nothing the earlier kernels write; grid_wait returns when they
+// have ended and their writes are visible.
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+static cudaError_t launch_after(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+}
+
 // nodes in 16 bytes (a node holds two values): the ring columns a TMA box
 // carries on each side of a tile
 template <class S>

@@ -79,15 +79,23 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, u
 //   main     HY rows x BX columns: x = x0 - cofs + c (16 bytes of columns on
 //            each side of the tile; edge tiles shift the box inward, see the
 //            kernel), rows from the tile's row window;
-//   xl, xr   HY rows x SX columns (16 bytes), the same rows: the left strip
-//            holds the columns around x = nx - 1 (the images of x = -1), the
-//            right strip x = 0 .. SX - 1 (the images of x >= nx); loaded only by
-//            the tiles at the x edges;
+//   xs       HY rows x SX columns (16 bytes), the same rows, for the tiles at the
+//            x edges of a row of several: the first tile's holds the columns
+//            around x = nx - 1 (the images of x = -1), the last one's x = 0 ..
+//            SX - 1 (the images of x >= nx);
 //   ys       one row x BX columns: the row across the periodic y boundary
 //            (y = ny - 1 for the first row of tiles, y = 0 for the last);
-//   cl, cr   one row x SX columns: the x-edge pieces of that row.
-// Element offsets count values (two per node).
-template <class S, int TY>
+//   cs       one row x SX columns: the x-edge piece of that row.
+// A single tile in x holds every column from x = 0 on, and takes the images
+// from there. Element offsets count values (two per node).
+// The load is bound by the 128-byte lines its box rows touch (64^3: boxes of
+// the 36 columns, 4 lines a row, take 14.4 of the step's 16.2 us, of 2 aligned
+// lines 10.1). Tiles begun one node later, so that a row touches 3 lines, lost
+// more in their misaligned stores (128^3 FP32 116.0 against 109.4 us,
+// 256x256x128 BF16 292.7 against 282.0).
+// FP32 4-row tiles with one stage keep psi of three planes, not four (one more
+// barrier a plane): 45.5 KB, five CTAs an SM.
+template <class S, int TY, int NS>
 struct TmaGeom {
     static constexpr int TX = 32, HX = TX + 2, HY = TY + 2;
     static constexpr int GX = edge_x<S>();                    // nodes in 16 bytes
@@ -98,16 +106,19 @@ struct TmaGeom {
     static constexpr int XS_ELEMS = 2 * Q * HY * SX;
     static constexpr int YS_ELEMS = 2 * Q * BX;
     static constexpr int CS_ELEMS = 2 * Q * SX;
-    static constexpr int XL = al(MAIN_ELEMS), XR = XL + al(XS_ELEMS), YS = XR + al(XS_ELEMS);
-    static constexpr int CL = YS + al(YS_ELEMS), CR = CL + al(CS_ELEMS);
-    static constexpr int STAGE_ELEMS = CR + al(CS_ELEMS);
+    static constexpr int YS = al(MAIN_ELEMS), CS = YS + al(YS_ELEMS), XS = CS + al(CS_ELEMS);
+    static constexpr int STAGE_ELEMS = al(XS + XS_ELEMS);
     static constexpr uint32_t MAIN_BYTES = MAIN_ELEMS * sizeof(S);
     static constexpr uint32_t XS_BYTES = XS_ELEMS * sizeof(S);
     static constexpr uint32_t YS_BYTES = YS_ELEMS * sizeof(S);
     static constexpr uint32_t CS_BYTES = CS_ELEMS * sizeof(S);
     static constexpr uint32_t STAGE_BYTES = STAGE_ELEMS * sizeof(S);
-    static constexpr int PSI_FLOATS = 4 * 2 * HY * HX;
-    static constexpr size_t smem(int NS) { return 128 + (size_t)NS * STAGE_BYTES + PSI_FLOATS * 4 + NS * 8; }
+    static constexpr int PSI_PLANES = sizeof(S) == 4 && TY == 4 && NS == 1 ? 3 : 4;
+    static constexpr int PSI_FLOATS = PSI_PLANES * 2 * HY * HX;
+    // psi follows the last stage's last region without padding
+    static constexpr size_t PSI_AT = ((size_t)(NS - 1) * STAGE_ELEMS + XS + XS_ELEMS) * sizeof(S);
+    static constexpr size_t SMEM = PSI_AT + PSI_FLOATS * 4 + NS * 8;
+    static_assert(PSI_AT % 8 == 0, "psi pairs are 8-byte accesses");
 };
 
 // Resident CTAs per SM the registers are held to (tau = 1): for 8-row tiles
@@ -127,13 +138,15 @@ struct TmaMaps {
 // x tile col % tiles_x), fluid planes [za, zb), with the maps of A's source
 // buffer. `stages`, `sp` and `bar` are the CTA's shared stages, psi ring and
 // stage barriers; g counts the planes the CTA has consumed so far (the
-// barriers' phases run on across items). Returns false when a wait gave up
-// (the status word is set and the CTA's copies in flight are drained).
+// barriers' phases run on across items). The first item (started: false) waits
+// for the step before, whose end its index arithmetic overlaps, and every item
+// then reads the step counter into clk. Returns false when a wait gave up (the
+// status word is set and the CTA's copies in flight are drained).
 template <class S, int TY, int NS, bool kTauOne>
 __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>& A, int col, int za, int zb, S* stages,
-                                         float* sp, uint64_t* bar, uint32_t& g, uint32_t clk)
+                                         float* sp, uint64_t* bar, uint32_t& g, uint32_t& clk, bool& started)
 {
-    using G = TmaGeom<S, TY>;
+    using G = TmaGeom<S, TY, NS>;
     constexpr int TX = 32, NT = TX * TY, HX = G::HX, HY = G::HY, GX = G::GX, BX = G::BX, SX = G::SX;
     constexpr int RING = 2 * HX + 2 * TY;
     constexpr int NIT = (RING + NT - 1) / NT;
@@ -158,13 +171,15 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
     const bool active = ty < hgt;
     const bool valid = active && gx < nx;
     const int np = zb - za + 2;  // planes za-1 .. zb
-    // x edges: the periodic images come from the strips (column of x = nx - 1 in the left strip)
-    const bool left_edge = x0 == 0, right_edge = x0 + TX >= nx;
+    // x edges: the periodic images come from the strip (column of x = nx - 1 in the first tile's), or,
+    // with a single tile, from the box itself
+    const bool one = A.tiles_x == 1;
+    const bool left_edge = x0 == 0 && !one, right_edge = x0 + TX >= nx && !one;
     // the box's column of node x0: GX (16 bytes of ring columns on each
     // side); an edge tile takes its outer ring column from a strip, so its
     // box is shifted inward and reads no padding columns beyond the lattice
     // (0 at the left edge, 2 GX at the right edge)
-    const int cofs = left_edge ? 0 : (right_edge ? 2 * GX : GX);
+    const int cofs = x0 == 0 ? 0 : (right_edge ? 2 * GX : GX);
     const int sl = (L.gx + nx - 1) / SX * SX, ol = L.gx + nx - 1 - sl;
     // y edges: the row window of the box, given by the box row of node row
     // y0 (rofs). A middle tile's box holds rows y0 - 1 .. y0 + TY; the first
@@ -176,12 +191,12 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
     const bool first = tyi == 0 && !single, last = tyi == A.tiles_y - 1 && !single;
     const int rofs = (first || single) ? 0 : (last ? HY - hgt : 1);
     const int yrow = first ? ny - 1 : 0;  // the real row in ys (first or last row of tiles)
-    // own node: the main box; lanes past x = nx - 1 of a ragged last tile
-    // hold the periodic images x - nx from the right strip (the one at
-    // x = nx is the +x neighbour of x = nx - 1), as far as the strip reaches
-    const bool own_strip = gx >= nx;
-    const bool own_rd = active && gx - nx < SX;
-    const int own_off = own_strip ? G::XR + 2 * ((ty + rofs) * SX + gx - nx) : 2 * ((ty + rofs) * BX + tx + cofs);
+    // own node: the main box; the lane past x = nx - 1 of a ragged last tile
+    // holds the periodic image x = 0, the +x neighbour of x = nx - 1
+    const bool own_strip = right_edge && gx >= nx;
+    const bool own_rd = active && gx <= nx;
+    const int own_off = own_strip ? G::XS + 2 * ((ty + rofs) * SX + gx - nx)
+                                  : 2 * ((ty + rofs) * BX + (one && gx == nx ? 0 : tx + cofs));
     // the copies' coordinates: x of the main box and of the left strip in
     // values (two per node; 16-byte aligned, as the copy requires), storage
     // row (real row + 1) of the box's first row and of the y-edge row (-1: none)
@@ -207,20 +222,20 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
             else if (r < 2 * HX) { ix = r - HX; iy = hgt + 1; }
             else if (r < 2 * HX + TY) { ix = 0; iy = r - 2 * HX + 1; }
             else { ix = HX - 1; iy = r - 2 * HX - TY + 1; }
-            const bool on = r < 2 * HX || iy <= hgt;  // side columns: the tile's own rows only
             it_sm = iy * HX + ix;
             const int xr = x0 - 1 + ix, yr = y0 - 1 + iy;  // the ring node (unwrapped)
+            // side columns: the tile's own rows only; nothing past x = nx
+            const bool on = (r < 2 * HX || iy <= hgt) && xr <= nx;
             const bool across = (first && yr < 0) || (last && yr >= ny);  // in the y-edge row
             const int row = wrapi(yr, ny) - y0 + rofs;                   // box row otherwise
-            if (xr < 0) {  // x = -1: the image of x = nx - 1
+            if ((xr < 0 || xr >= nx) && !one) {
+                const int c = xr < 0 ? ol : xr - nx;  // the image's column in the strip
                 it_cls = across ? 3 : 1;
-                it_base = across ? G::CL + 2 * ol : G::XL + 2 * (row * SX + ol);
-            } else if (xr >= nx && xr - nx < SX) {  // x >= nx: the images of x - nx
-                it_cls = across ? 3 : 1;
-                it_base = across ? G::CR + 2 * (xr - nx) : G::XR + 2 * (row * SX + xr - nx);
+                it_base = across ? G::CS + 2 * c : G::XS + 2 * (row * SX + c);
             } else {
+                const int c = one ? wrapi(xr, nx) : ix - 1 + cofs;
                 it_cls = across ? 2 : 0;
-                it_base = across ? G::YS + 2 * (ix - 1 + cofs) : 2 * (row * BX + ix - 1 + cofs);
+                it_base = across ? G::YS + 2 * c : 2 * (row * BX + c);
             }
             if (on) it_code[i] = it_base | (it_sm << 17) | (it_cls << 27);
         }
@@ -234,19 +249,20 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
             S* stg = stages + (size_t)(gi % NS) * G::STAGE_ELEMS;
             const bool ye = ysr >= 0;
             fence_proxy_async();
-            mbar_expect_tx(b, G::MAIN_BYTES + (left_edge ? G::XS_BYTES : 0u) + (right_edge ? G::XS_BYTES : 0u) +
-                                  (ye ? G::YS_BYTES + (left_edge ? G::CS_BYTES : 0u) +
-                                            (right_edge ? G::CS_BYTES : 0u)
-                                      : 0u));
+            const bool xe = left_edge || right_edge;
+            const int xc = left_edge ? xs : 2 * L.gx;
+            mbar_expect_tx(b, G::MAIN_BYTES + (xe ? G::XS_BYTES : 0u) + (ye ? G::YS_BYTES + (xe ? G::CS_BYTES : 0u) : 0u));
             tma_load_4d(stg, &maps.m[0], b, xb, yb, zp, 0);
-            if (left_edge) tma_load_4d(stg + G::XL, &maps.m[1], b, xs, yb, zp, 0);
-            if (right_edge) tma_load_4d(stg + G::XR, &maps.m[1], b, 2 * L.gx, yb, zp, 0);
+            if (xe) tma_load_4d(stg + G::XS, &maps.m[1], b, xc, yb, zp, 0);
             if (ye) {
                 tma_load_4d(stg + G::YS, &maps.m[2], b, xb, ysr, zp, 0);
-                if (left_edge) tma_load_4d(stg + G::CL, &maps.m[3], b, xs, ysr, zp, 0);
-                if (right_edge) tma_load_4d(stg + G::CR, &maps.m[3], b, 2 * L.gx, ysr, zp, 0);
+                if (xe) tma_load_4d(stg + G::CS, &maps.m[3], b, xc, ysr, zp, 0);
             }
         }
+    };
+    // the psi ring's plane of lattice plane z
+    auto psi_plane = [&](int z) {
+        return (float2*)sp + (G::PSI_PLANES == 4 ? (z & 3) : z % 3) * (HY * HX);
     };
 
     // wait for plane i of the item, reduce it to psi (tile + ring) and own
@@ -255,7 +271,9 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
         const int zp = za - 1 + i;
         const uint32_t gi = g + i;
         const bool ok = mbar_wait(&bar[gi % NS], (gi / NS) & 1u);
-        float2* spl = (float2*)sp + (zp & 3) * (HY * HX);
+        float2* spl = psi_plane(zp);
+        // with three planes, this one takes the place of the lowest that the collision before read
+        if constexpr (G::PSI_PLANES == 3) __syncthreads();
         const bool solid = (zp == 0 && !(A.halo & 1)) || (zp == nz - 1 && !(A.halo & 2));
         if (ok) {
             const S* st = stages + (size_t)(gi % NS) * G::STAGE_ELEMS;
@@ -340,6 +358,11 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
 
     float rc[2], jc[2][3], vc[2][Q], mc[2];
     float rn[2], jn[2][3], vn[2][Q], mn[2];
+    if (!started) {
+        grid_wait();
+        started = true;
+    }
+    if constexpr (Codec<S>::kDeviation) clk = clock_read(A.clock);
     __syncthreads();  // the previous item's collide is done with the psi ring
     if (tid == 0)
         for (int i = 0; i < NS && i < np; ++i) issue(za - 1 + i, g + i);
@@ -354,9 +377,7 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
         if (!consume(z - za + 2, rn, jn, vn, mn)) return false;
         if (valid) {
             float F[2][3];
-            const float2* ring = (const float2*)sp;
-            sc_force<HX, HY>(ring + ((z - 1) & 3) * (HY * HX), ring + (z & 3) * (HY * HX),
-                             ring + ((z + 1) & 3) * (HY * HX), ty, tx, gk, Gax, Gdi, F);
+            sc_force<HX, HY>(psi_plane(z - 1), psi_plane(z), psi_plane(z + 1), ty, tx, gk, Gax, Gdi, F);
             D.zo[0] = (int)((z - 1) * plane);
             D.zo[1] = (int)(z * plane);
             D.zo[2] = (int)((z + 1) * plane);
@@ -391,25 +412,25 @@ template <class S, int TY, int NS, bool kTauOne>
 __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
     step_tma_kernel(const __grid_constant__ TmaMaps maps, const StepArgs<S> A)
 {
-    using G = TmaGeom<S, TY>;
-    static_assert(G::STAGE_BYTES % 128 == 0 && (G::XL * sizeof(S)) % 128 == 0 && (G::YS * sizeof(S)) % 128 == 0 &&
-                      (G::CL * sizeof(S)) % 128 == 0 && (G::CR * sizeof(S)) % 128 == 0,
+    using G = TmaGeom<S, TY, NS>;
+    static_assert(G::STAGE_BYTES % 128 == 0 && (G::XS * sizeof(S)) % 128 == 0 && (G::YS * sizeof(S)) % 128 == 0 &&
+                      (G::CS * sizeof(S)) % 128 == 0,
                   "stages and their regions stay 128-byte aligned");
     static_assert((2 * G::BX * sizeof(S)) % 16 == 0 && (2 * G::SX * sizeof(S)) % 16 == 0,
                   "box rows are whole 16-byte units");
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-    S* stages = (S*)base;
-    float* sp = (float*)(base + (size_t)NS * G::STAGE_BYTES);  // psi ring [4][HY][HX] of pairs (psi^b, psi^r)
+    extern __shared__ __align__(128) unsigned char smem[];
+    S* stages = (S*)smem;
+    float* sp = (float*)(smem + G::PSI_AT);  // psi ring [PSI_PLANES][HY][HX] of pairs (psi^b, psi^r)
     uint64_t* bar = (uint64_t*)(sp + G::PSI_FLOATS);
     if (threadIdx.x == 0) {
         for (int s = 0; s < NS; ++s) mbar_init(&bar[s], 1);
         mbar_fence_init();
     }
     __syncthreads();
+    grid_trigger();  // the next step's CTAs may take the slots that free up, up to their own wait
     uint32_t g = 0;  // planes this CTA has issued and consumed so far
     uint32_t clk = 0;
-    if constexpr (Codec<S>::kDeviation) clk = clock_read(A.clock);
+    bool started = false;
     const int ncol = A.tiles_x * A.tiles_y;
     const int nzf = A.zhi - A.zlo;
     for (int item = blockIdx.x; item < ncol * A.nseg; item += gridDim.x) {
@@ -417,8 +438,9 @@ __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
         const int za = A.zlo + (int)((long long)seg * nzf / A.nseg);
         const int zb = A.zlo + (int)((long long)(seg + 1) * nzf / A.nseg);
         if (za >= zb) continue;
-        if (!tma_item<S, TY, NS, kTauOne>(maps, A, col, za, zb, stages, sp, bar, g, clk)) break;
+        if (!tma_item<S, TY, NS, kTauOne>(maps, A, col, za, zb, stages, sp, bar, g, clk, started)) break;
     }
+    if (!started) grid_wait();
     if constexpr (Codec<S>::kDeviation) clock_tick(A.clock);
 }
 
@@ -432,18 +454,19 @@ __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
     batch_tma_kernel(const TmaMaps* __restrict__ maps, const StepArgs<S>* __restrict__ args,
                      const int4* __restrict__ items, int nitems, int parity, int nbox, uint32_t* done)
 {
-    using G = TmaGeom<S, TY>;
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-    S* stages = (S*)base;
-    float* sp = (float*)(base + (size_t)NS * G::STAGE_BYTES);
+    using G = TmaGeom<S, TY, NS>;
+    extern __shared__ __align__(128) unsigned char smem[];
+    S* stages = (S*)smem;
+    float* sp = (float*)(smem + G::PSI_AT);
     uint64_t* bar = (uint64_t*)(sp + G::PSI_FLOATS);
     if (threadIdx.x == 0) {
         for (int s = 0; s < NS; ++s) mbar_init(&bar[s], 1);
         mbar_fence_init();
     }
     __syncthreads();
+    grid_trigger();
     uint32_t g = 0;
+    bool started = false;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int4 w = items[it];
         const StepArgs<S>& A = args[2 * w.x + parity];
@@ -452,9 +475,9 @@ __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
             for (int i = 0; i < 4; ++i)  // the maps were written through the generic proxy
                 asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&M.m[i]) : "memory");
         uint32_t clk = 0;
-        if constexpr (Codec<S>::kDeviation) clk = clock_read(A.clock);
-        if (!tma_item<S, TY, NS, kTauOne>(M, A, w.y, w.z, w.w, stages, sp, bar, g, clk)) break;
+        if (!tma_item<S, TY, NS, kTauOne>(M, A, w.y, w.z, w.w, stages, sp, bar, g, clk, started)) break;
     }
+    if (!started) grid_wait();
     if constexpr (Codec<S>::kDeviation) {
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -470,19 +493,18 @@ __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
 template <class S, int TY, int NS, bool T1>
 static cudaError_t tma_launch_one(const CUtensorMap* m, const StepArgs<S>& A, cudaStream_t st)
 {
-    const size_t smem = TmaGeom<S, TY>::smem(NS);
+    const size_t smem = TmaGeom<S, TY, NS>::SMEM;
     const int items = A.tiles_x * A.tiles_y * A.nseg;
     TmaMaps maps;
     for (int i = 0; i < 4; ++i) maps.m[i] = m[i];
-    step_tma_kernel<S, TY, NS, T1><<<items, 32 * TY, smem, st>>>(maps, A);
-    return cudaGetLastError();
+    return launch_after(step_tma_kernel<S, TY, NS, T1>, dim3(items), 32 * TY, smem, st, maps, A);
 }
 
 template <class S, int TY, int NS, bool T1>
 static cudaError_t tma_prepare_one()
 {
     return cudaFuncSetAttribute(step_tma_kernel<S, TY, NS, T1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)TmaGeom<S, TY>::smem(NS));
+                                (int)TmaGeom<S, TY, NS>::SMEM);
 }
 
 template <class S, int TY, int NS, bool T1>
@@ -490,7 +512,7 @@ static int tma_occ_one()
 {
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_tma_kernel<S, TY, NS, T1>, 32 * TY,
-                                                      TmaGeom<S, TY>::smem(NS)) != cudaSuccess)
+                                                      TmaGeom<S, TY, NS>::SMEM) != cudaSuccess)
         return 1;
     return n;
 }
@@ -532,10 +554,10 @@ template <class S, int TY, bool T1>
 static long long tma_batch_one(int op, const TmaMaps* maps, const StepArgs<S>* args, const int4* items, int nitems,
                                int parity, int nbox, uint32_t* done, int grid, cudaStream_t st)
 {
-    const size_t smem = TmaGeom<S, TY>::smem(1);
+    const size_t smem = TmaGeom<S, TY, 1>::SMEM;
     if (op == 0) {
-        batch_tma_kernel<S, TY, 1, T1><<<grid, 32 * TY, smem, st>>>(maps, args, items, nitems, parity, nbox, done);
-        return cudaGetLastError();
+        return launch_after(batch_tma_kernel<S, TY, 1, T1>, dim3(grid), 32 * TY, smem, st, maps, args, items, nitems, parity,
+                            nbox, done);
     }
     if (op == 1)
         return cudaFuncSetAttribute(batch_tma_kernel<S, TY, 1, T1>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -669,3 +669,20 @@ def test_contact_angle_sums_on_ragged_lattices(lbsc, dims, offset):
         for k in ("h", "theta_fit_deg", "xc", "yc", "zc", "r_fit") + (() if walled else ("b", "r", "base_ref", "theta_deg")):
             if o[k] > -1e290:
                 assert abs(d[k] - o[k]) <= 1e-7 * max(1.0, abs(o[k])), (k, level, d[k], o[k])
+
+
+@pytest.mark.parametrize("precision", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("dims", [(1, 1, 3), (2, 1, 4), (3, 5, 3), (31, 4, 5), (32, 9, 8), (33, 3, 21), (34, 16, 7), (63, 5, 6),
+                                  (64, 6, 40), (65, 33, 9), (96, 2, 11), (97, 13, 130)])
+def test_automatic_schedule_at_tile_edges(lbsc, dims, precision):
+    """The chosen split and the TMA kernel at the edges of its tiles and boxes (one tile in x holding its own images, the
+    first and last tile's strips, one and several rows of tiles, segments of one plane): bit for bit the
+    load-from-global kernel, for equal and unequal relaxation times."""
+    nx, ny, nz = dims
+    rng = np.random.Generator(np.random.PCG64(nx * ny * nz))
+    rr, rb = rng.uniform(0.05, 0.7, size=(2, nz, ny, nx))
+    for tau in ((1.0, 1.0), (0.9, 1.2)):
+        prm = dict(CONTACT, tau_r=tau[0], tau_b=tau[1], eta_wall_r=-0.04, eta_wall_b=0.04)
+        auto = lbsc.Lattice(rr, rb, precision).set_params(**prm).step(7)
+        ldg = lbsc.Lattice(rr, rb, precision).set_params(**prm).set_step_variant("ldg").step(7)
+        assert np.array_equal(auto.populations(), ldg.populations())
