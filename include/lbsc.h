@@ -52,9 +52,9 @@ extern "C" {
 #define LB_BF16 2  /* BF16 deviations, as above */
 
 /* step kernel variants (lb_set_step_variant) */
-#define LB_STEP_AUTO 0  /* the TMA kernel with one stage where it applies, else load-from-global */
+#define LB_STEP_AUTO 0  /* the TMA kernel where it is built, else load-from-global */
 #define LB_STEP_LDG 1   /* every plane loaded from global memory by the compute threads */
-#define LB_STEP_TMA 2   /* planes staged into shared memory by TMA (planar walls only) */
+#define LB_STEP_TMA 2   /* planes staged into shared memory by TMA */
 
 /* neighbour weights G_k of the Shan-Chen force sum */
 #define LB_WEIGHTS_UNIT 0  /* G_k = 1 for the 18 neighbours, as Eq. SCforce is printed */
@@ -360,7 +360,9 @@ int lb_set_populations(lb_ctx* ctx, const double* n);
 int lb_build_flags(int* flags);
 
 /* Choose the step kernel's tile height (4, 8 or 16 rows of 32 nodes) and the
- * number of z segments per tile column (0 = automatic). */
+ * number of z segments per tile column (0 = automatic). Without this call the
+ * height, the row split, the segments and the TMA stages are all chosen by the
+ * estimated time of a step. */
 int lb_set_schedule(lb_ctx* ctx, int tile_y, int z_segments);
 
 /* The same, with the ny rows split evenly into y_tiles tiles of at most
@@ -372,11 +374,12 @@ int lb_set_tiling(lb_ctx* ctx, int tile_y, int y_tiles, int z_segments);
 
 /* Choose the step kernel: LB_STEP_AUTO, LB_STEP_LDG or LB_STEP_TMA, and for
  * the TMA kernel the number of shared-memory stages, i.e. planes in flight
- * (1, 2 or 3; 0 = automatic: 1 for LB_STEP_AUTO, else 3, else 2). One stage
- * leaves room for more resident CTAs per SM (measured the fastest on GB300).
+ * (1, 2 or 3; 0 = automatic: for LB_STEP_AUTO one or two by the estimated
+ * time of a step, else 3, else 2). One stage leaves room for more resident
+ * CTAs per SM, two keep a small lattice's few CTAs supplied.
  * Every variant computes bit-identical results. LB_STEP_AUTO and LB_STEP_TMA
- * with a non-planar geometry, or a (tile height, stages) pair that
- * is not built for the precision, fall back to LB_STEP_LDG. */
+ * with a (tile height, stages) pair that is not built for the precision and
+ * geometry fall back to LB_STEP_LDG. */
 int lb_set_step_variant(lb_ctx* ctx, int variant, int stages);
 
 /* ------------------------------------------------------------ adjoint

@@ -176,30 +176,32 @@ static bool tau_one(const lb_ctx* c) { return c->prm.tau_r == 1.0 && c->prm.tau_
 static const int kTmaTiles[3] = {4, 8, 16};
 static int tile_index(int ty) { return ty == 4 ? 0 : (ty == 8 ? 1 : 2); }
 
+// ops of tma_step for the context's geometry
 template <class S>
-static long long tma_op(int op, lb_ctx* c, int ty, int ns, const CUtensorMap* m, const StepArgs<S>* A,
+static long long tma_op(int op, lb_ctx* c, bool general, int ty, int ns, const CUtensorMap* m, const StepArgs<S>* A,
                         cudaStream_t st)
 {
-    return tma_step<S>(op, ty, ns, tau_one(c), m, A, st);
+    return general ? tma_step_general<S>(op, ty, ns, tau_one(c), m, A, st) : tma_step<S>(op, ty, ns, tau_one(c), m, A, st);
 }
 
-static long long tma_call(int op, lb_ctx* c, int ty, int ns)
+static long long tma_call(int op, lb_ctx* c, bool general, int ty, int ns)
 {
     switch (c->prec) {
-    case LB_F32: return tma_op<float>(op, c, ty, ns, nullptr, nullptr, nullptr);
-    case LB_F16: return tma_op<__half>(op, c, ty, ns, nullptr, nullptr, nullptr);
-    default: return tma_op<__nv_bfloat16>(op, c, ty, ns, nullptr, nullptr, nullptr);
+    case LB_F32: return tma_op<float>(op, c, general, ty, ns, nullptr, nullptr, nullptr);
+    case LB_F16: return tma_op<__half>(op, c, general, ty, ns, nullptr, nullptr, nullptr);
+    default: return tma_op<__nv_bfloat16>(op, c, general, ty, ns, nullptr, nullptr, nullptr);
     }
 }
 
 // raise the shared-memory limit of every TMA kernel built for this precision
 static cudaError_t tma_prepare(lb_ctx* c)
 {
-    for (int ty : kTmaTiles)
-        for (int ns = 1; ns <= 3; ++ns) {
-            const long long e = tma_call(1, c, ty, ns);  // cudaErrorInvalidValue: pair not built
-            if (e != (long long)cudaSuccess && e != (long long)cudaErrorInvalidValue) return (cudaError_t)e;
-        }
+    for (int general = 0; general < 2; ++general)
+        for (int ty : kTmaTiles)
+            for (int ns = 1; ns <= 3; ++ns) {
+                const long long e = tma_call(1, c, general != 0, ty, ns);  // cudaErrorInvalidValue: pair not built
+                if (e != (long long)cudaSuccess && e != (long long)cudaErrorInvalidValue) return (cudaError_t)e;
+            }
     return cudaSuccess;
 }
 
@@ -245,9 +247,9 @@ static const Schedule& schedule(lb_ctx* c)
     Schedule best;
     double least = 0;
     const int tys[2] = {c->tile_y_req ? c->tile_y_req : 4, c->tile_y_req || c->prec == LB_F32 || !tau_one(c) ? 0 : 8};
-    // a general geometry loads from global; TMA asked for by name takes three stages, else two
+    // TMA asked for by name takes three stages, else two
     for (int ty : tys) {
-        if (!ty || c->general || c->variant == LB_STEP_LDG) continue;
+        if (!ty || c->variant == LB_STEP_LDG) continue;
         int stages[2] = {1, 2};
         if (c->variant == LB_STEP_TMA) stages[0] = 3;
         if (!tau_one(c) && c->variant == LB_STEP_AUTO) stages[0] = 2;  // holds v in fewer registers than one stage does
@@ -256,11 +258,12 @@ static const Schedule& schedule(lb_ctx* c)
             const int ns = stages[i];
             if (i && (ns == stages[0] || (best.ty == ty && c->variant == LB_STEP_TMA))) break;
             // occupancy 0: the pair is not built for this precision (or does not fit)
-            const int occ = (int)tma_call(2, c, ty, ns);
+            const int occ = (int)tma_call(2, c, c->general, ty, ns);
             if (occ < 1) continue;
             const int base = (ny + ty - 1) / ty;
+            // a height asked for without a split takes as few tiles as it needs
             const int yt0 = c->y_tiles_req ? c->y_tiles_req : base;
-            const int yt1 = c->y_tiles_req ? yt0 : (base + base / 3 < ny ? base + base / 3 : ny);
+            const int yt1 = c->tile_y_req ? yt0 : (base + base / 3 < ny ? base + base / 3 : ny);
             for (int yt = yt0; yt <= yt1; ++yt) {
                 if (yt > yt0 && (ny + yt - 1) / yt < ty - 1) break;
                 for (int w = 1; w <= 3; ++w) {
@@ -384,7 +387,7 @@ static cudaError_t launch_one_step(lb_ctx* c, int src, cudaStream_t st)
 {
     const StepArgs<S> A = step_args<S>(c, src);
     const Schedule& d = schedule(c);
-    if (d.ns) return (cudaError_t)tma_step<S>(0, d.ty, d.ns, tau_one(c), c->tmap[src][tile_index(d.ty)], &A, st);
+    if (d.ns) return (cudaError_t)tma_op<S>(0, c, c->general, d.ty, d.ns, c->tmap[src][tile_index(d.ty)], &A, st);
     return launch_step<S>(A, d.ty, c->general, tau_one(c), st);
 }
 

@@ -80,6 +80,10 @@ cudaError_t launch_step(const StepArgs<S>& A, int tile_y, bool general, bool tau
 template <class S>
 long long tma_step(int op, int tile_y, int stages, bool tau_one, const CUtensorMap* map, const StepArgs<S>* args,
                    cudaStream_t stream);
+// the same for a general geometry (4-row tiles, and 8-row ones for 16-bit storage, with one or two stages)
+template <class S>
+long long tma_step_general(int op, int tile_y, int stages, bool tau_one, const CUtensorMap* map, const StepArgs<S>* args,
+                           cudaStream_t stream);
 template <class S>
 cudaError_t launch_batch_step(const StepArgs<S>* args, const int4* items, int nitems, int parity, int tile_y,
                               bool tau_one, int grid, int nbox, uint32_t* done, cudaStream_t st);

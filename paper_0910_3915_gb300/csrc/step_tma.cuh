@@ -1,5 +1,5 @@
-// Fused time step (Sec. 2) for the planar-wall geometry, with the next
-// planes' populations staged into shared memory by TMA.
+// Fused time step (Sec. 2) with the next planes' populations staged into
+// shared memory by TMA: planar walls, and (kGeneral) any solid mask.
 //
 // A CTA owns a 32 x TY tile of columns and a z segment, as in the
 // load-from-global kernel, but one thread streams whole planes of the tile
@@ -13,7 +13,9 @@
 // across the periodic boundary) and 16-byte corner pieces of that row, so no
 // image of any node is ever stored. Every wait is bounded: a wait that gives
 // up writes an error status, drains the CTA's copies in flight and leaves the
-// kernel.
+// kernel. In a general geometry the planes wrap along z, and a node's mask word
+// (its own and its links' solid bits) is loaded while its plane's copy is
+// awaited: 4 bytes beside the 304 of an update.
 #pragma once
 
 #include <cuda.h>
@@ -142,7 +144,7 @@ struct TmaMaps {
 // for the step before, whose end its index arithmetic overlaps, and every item
 // then reads the step counter into clk. Returns false when a wait gave up (the
 // status word is set and the CTA's copies in flight are drained).
-template <class S, int TY, int NS, bool kTauOne>
+template <class S, int TY, int NS, bool kTauOne, bool kGeneral = false>
 __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>& A, int col, int za, int zb, S* stages,
                                          float* sp, uint64_t* bar, uint32_t& g, uint32_t& clk, bool& started)
 {
@@ -197,6 +199,7 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
     const bool own_rd = active && gx <= nx;
     const int own_off = own_strip ? G::XS + 2 * ((ty + rofs) * SX + gx - nx)
                                   : 2 * ((ty + rofs) * BX + (one && gx == nx ? 0 : tx + cofs));
+    const int own_node = (gy + 1) * L.px + L.gx + (gx < nx ? gx : 0);  // its offset in its plane (general geometry)
     // the copies' coordinates: x of the main box and of the left strip in
     // values (two per node; 16-byte aligned, as the copy requires), storage
     // row (real row + 1) of the box's first row and of the y-edge row (-1: none)
@@ -210,11 +213,12 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
     // (packed in one word: stage position in bits 0-16, shared-memory position in
     // bits 17-26, stride class in bits 27-28; -1 for no item)
     static_assert(G::STAGE_ELEMS <= (1 << 17) && HY * HX <= (1 << 10), "ring item fields fit their bits");
-    int it_code[NIT];
+    int it_code[NIT], it_node[NIT];  // it_node (general geometry): the node's offset in its plane
 #pragma unroll
     for (int i = 0; i < NIT; ++i) {
         const int r = tid + i * NT;
         it_code[i] = -1;
+        it_node[i] = 0;
         if (r < RING) {
             int it_sm, it_base, it_cls;
             int ix, iy;
@@ -238,13 +242,20 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
                 it_base = across ? G::YS + 2 * c : 2 * (row * BX + c);
             }
             if (on) it_code[i] = it_base | (it_sm << 17) | (it_cls << 27);
+            if constexpr (kGeneral)
+                if (on) it_node[i] = (wrapi(yr, ny) + 1) * L.px + L.gx + (xr < 0 ? xr + nx : xr % nx);
         }
     }
 
-    auto issue = [&](int zp, uint32_t gi) {
+    // a wall plane of the planar geometry (a z slab's halo plane is loaded like fluid)
+    auto wall_plane = [&](int zp) {
+        return !kGeneral && ((zp == 0 && !(A.halo & 1)) || (zp == nz - 1 && !(A.halo & 2)));
+    };
+    auto issue = [&](int zu, uint32_t gi) {
         uint64_t* b = &bar[gi % NS];
-        if ((zp == 0 && !(A.halo & 1)) || (zp == nz - 1 && !(A.halo & 2))) {
-            mbar_arrive(b);  // a wall plane: nothing to load (a z slab's halo plane is loaded like fluid)
+        const int zp = kGeneral ? wrapi(zu, nz) : zu;
+        if (wall_plane(zp)) {
+            mbar_arrive(b);  // nothing to load
         } else {
             S* stg = stages + (size_t)(gi % NS) * G::STAGE_ELEMS;
             const bool ye = ysr >= 0;
@@ -262,26 +273,36 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
     };
     // the psi ring's plane of lattice plane z
     auto psi_plane = [&](int z) {
-        return (float2*)sp + (G::PSI_PLANES == 4 ? (z & 3) : z % 3) * (HY * HX);
+        return (float2*)sp + (G::PSI_PLANES == 4 ? (z & 3) : (z + 3) % 3) * (HY * HX);
     };
 
     // wait for plane i of the item, reduce it to psi (tile + ring) and own
     // moments, then refill its stage with plane i + NS
-    auto consume = [&](int i, float (&rho)[2], float (&j)[2][3], float (&v)[2][Q], float (&m)[2]) -> bool {
+    auto consume = [&](int i, float (&rho)[2], float (&j)[2][3], float (&v)[2][Q], float (&m)[2], uint32_t& nb) -> bool {
         const int zp = za - 1 + i;
         const uint32_t gi = g + i;
+        bool solid_own = wall_plane(zp), solid_it[NIT];
+#pragma unroll
+        for (int q = 0; q < NIT; ++q) solid_it[q] = solid_own;
+        if constexpr (kGeneral) {
+            const uint32_t* mask = A.nbmask + (long long)wrapi(zp, nz) * plane;
+            nb = own_rd ? __ldg(mask + own_node) : kSelfSolid;
+            solid_own = (nb & kSelfSolid) != 0;
+#pragma unroll
+            for (int q = 0; q < NIT; ++q)
+                if (it_code[q] >= 0) solid_it[q] = (__ldg(mask + it_node[q]) & kSelfSolid) != 0;
+        }
         const bool ok = mbar_wait(&bar[gi % NS], (gi / NS) & 1u);
         float2* spl = psi_plane(zp);
         // with three planes, this one takes the place of the lowest that the collision before read
         if constexpr (G::PSI_PLANES == 3) __syncthreads();
-        const bool solid = (zp == 0 && !(A.halo & 1)) || (zp == nz - 1 && !(A.halo & 2));
         if (ok) {
             const S* st = stages + (size_t)(gi % NS) * G::STAGE_ELEMS;
             float ps[2] = {eta[0], eta[1]};
             rho[0] = rho[1] = m[0] = m[1] = 0.f;
 #pragma unroll
             for (int a = 0; a < 2; ++a) j[a][0] = j[a][1] = j[a][2] = 0.f;
-            if (!solid && own_rd) {
+            if (!solid_own && own_rd) {
                 float w[2][Q];
                 // both components of velocity k in one shared-memory load
                 const P2* so = (const P2*)(st + own_off);
@@ -320,7 +341,7 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
                 if (code < 0) continue;
                 const int it_sm = (code >> 17) & 0x3FF;
                 float2 pr = f2(eta[0], eta[1]);
-                if (!solid) {
+                if (!solid_it[q]) {
                     // both components of velocity k in one shared-memory load
                     float2 w[Q];
                     const P2* si = (const P2*)(st + (code & 0x1FFFF));
@@ -358,6 +379,7 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
 
     float rc[2], jc[2][3], vc[2][Q], mc[2];
     float rn[2], jn[2][3], vn[2][Q], mn[2];
+    uint32_t nbc = 0, nbn = 0;  // general geometry: mask words of the current and the next plane's own node
     if (!started) {
         grid_wait();
         started = true;
@@ -366,7 +388,7 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
     __syncthreads();  // the previous item's collide is done with the psi ring
     if (tid == 0)
         for (int i = 0; i < NS && i < np; ++i) issue(za - 1 + i, g + i);
-    if (!consume(0, rn, jn, vn, mn) || !consume(1, rc, jc, vc, mc)) return false;
+    if (!consume(0, rn, jn, vn, mn, nbn) || !consume(1, rc, jc, vc, mc, nbc)) return false;
 
     Dest D;
     D.set_column(L, valid ? gx : 0, valid ? gy : 0);
@@ -374,24 +396,26 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
     D.hoff = A.hkey;
 
     for (int z = za; z < zb; ++z) {
-        if (!consume(z - za + 2, rn, jn, vn, mn)) return false;
-        if (valid) {
+        if (!consume(z - za + 2, rn, jn, vn, mn, nbn)) return false;
+        if (valid && !(kGeneral && (nbc & kSelfSolid))) {
             float F[2][3];
             sc_force<HX, HY>(psi_plane(z - 1), psi_plane(z), psi_plane(z + 1), ty, tx, gk, Gax, Gdi, F);
-            D.zo[0] = (int)((z - 1) * plane);
+            D.zo[0] = (int)((kGeneral ? wrapi(z - 1, nz) : z - 1) * plane);
             D.zo[1] = (int)(z * plane);
-            D.zo[2] = (int)((z + 1) * plane);
-            D.bot = z - 1 == 0 && !(A.halo & 1);  // a halo plane takes pushes like fluid
-            D.top = z + 1 == nz - 1 && !(A.halo & 2);
+            D.zo[2] = (int)((kGeneral ? wrapi(z + 1, nz) : z + 1) * plane);
+            D.bot = !kGeneral && z - 1 == 0 && !(A.halo & 1);  // a halo plane takes pushes like fluid
+            D.top = !kGeneral && z + 1 == nz - 1 && !(A.halo & 2);
+            D.nb = nbc;
             if constexpr (Codec<S>::kDeviation) {
                 // rho = rho_ref + m36 / 36, as moments2 forms it: not held across the plane
                 const float2 r = fma2(f2(mc[0], mc[1]), sp2(1.0f / 36.0f), f2(ref[0], ref[1]));
                 const float rr[2] = {r.x, r.y};
-                collide_store<S, false, kTauOne>(rr, jc, vc, F, tau, itau, ref, dst, L, gx, gy, D, mc, clk);
+                collide_store<S, kGeneral, kTauOne>(rr, jc, vc, F, tau, itau, ref, dst, L, gx, gy, D, mc, clk);
             } else {
-                collide_store<S, false, kTauOne>(rc, jc, vc, F, tau, itau, ref, dst, L, gx, gy, D, mc, clk);
+                collide_store<S, kGeneral, kTauOne>(rc, jc, vc, F, tau, itau, ref, dst, L, gx, gy, D, mc, clk);
             }
         }
+        nbc = nbn;
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
             if constexpr (!Codec<S>::kDeviation) rc[a] = rn[a];
@@ -408,7 +432,7 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
     return true;
 }
 
-template <class S, int TY, int NS, bool kTauOne>
+template <class S, int TY, int NS, bool kTauOne, bool kGeneral>
 __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
     step_tma_kernel(const __grid_constant__ TmaMaps maps, const StepArgs<S> A)
 {
@@ -438,7 +462,7 @@ __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
         const int za = A.zlo + (int)((long long)seg * nzf / A.nseg);
         const int zb = A.zlo + (int)((long long)(seg + 1) * nzf / A.nseg);
         if (za >= zb) continue;
-        if (!tma_item<S, TY, NS, kTauOne>(maps, A, col, za, zb, stages, sp, bar, g, clk, started)) break;
+        if (!tma_item<S, TY, NS, kTauOne, kGeneral>(maps, A, col, za, zb, stages, sp, bar, g, clk, started)) break;
     }
     if (!started) grid_wait();
     if constexpr (Codec<S>::kDeviation) clock_tick(A.clock);
@@ -490,56 +514,48 @@ __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
     }
 }
 
-template <class S, int TY, int NS, bool T1>
-static cudaError_t tma_launch_one(const CUtensorMap* m, const StepArgs<S>& A, cudaStream_t st)
+template <class S, int TY, int NS, bool T1, bool GEN>
+static long long tma_one(int op, const CUtensorMap* m, const StepArgs<S>* A, cudaStream_t st)
 {
-    const size_t smem = TmaGeom<S, TY, NS>::SMEM;
-    const int items = A.tiles_x * A.tiles_y * A.nseg;
-    TmaMaps maps;
-    for (int i = 0; i < 4; ++i) maps.m[i] = m[i];
-    return launch_after(step_tma_kernel<S, TY, NS, T1>, dim3(items), 32 * TY, smem, st, maps, A);
-}
-
-template <class S, int TY, int NS, bool T1>
-static cudaError_t tma_prepare_one()
-{
-    return cudaFuncSetAttribute(step_tma_kernel<S, TY, NS, T1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)TmaGeom<S, TY, NS>::SMEM);
-}
-
-template <class S, int TY, int NS, bool T1>
-static int tma_occ_one()
-{
+    const auto kernel = step_tma_kernel<S, TY, NS, T1, GEN>;
+    constexpr size_t smem = TmaGeom<S, TY, NS>::SMEM;
+    if (op == 0) {
+        TmaMaps maps;
+        for (int i = 0; i < 4; ++i) maps.m[i] = m[i];
+        return launch_after(kernel, dim3(A->tiles_x * A->tiles_y * A->nseg), 32 * TY, smem, st, maps, *A);
+    }
+    if (op == 1) return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_tma_kernel<S, TY, NS, T1>, 32 * TY,
-                                                      TmaGeom<S, TY, NS>::SMEM) != cudaSuccess)
-        return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, 32 * TY, smem) != cudaSuccess) return 1;
     return n;
 }
 
 // Dispatch over the built (tile height, stages, tau == 1) combinations.
 // op 0: launch; op 1: set the shared-memory attribute; op 2: occupancy.
-template <class S>
+template <class S, bool GEN>
 static long long tma_dispatch(int op, int ty, int ns, bool t1, const CUtensorMap* m, const StepArgs<S>* A,
                               cudaStream_t st)
 {
-#define LBSC_TMA_CASE(TY_, NS_)                                                                       \
-    if (ty == TY_ && ns == NS_) {                                                                     \
-        if (op == 0) return t1 ? tma_launch_one<S, TY_, NS_, true>(m, *A, st)                         \
-                               : tma_launch_one<S, TY_, NS_, false>(m, *A, st);                       \
-        if (op == 1) {                                                                                \
-            cudaError_t e = tma_prepare_one<S, TY_, NS_, true>();                                     \
-            return e != cudaSuccess ? e : tma_prepare_one<S, TY_, NS_, false>();                      \
-        }                                                                                             \
-        return t1 ? tma_occ_one<S, TY_, NS_, true>() : tma_occ_one<S, TY_, NS_, false>();             \
+#define LBSC_TMA_CASE(TY_, NS_)                                                           \
+    if (ty == TY_ && ns == NS_) {                                                         \
+        if (op == 1) {                                                                    \
+            const long long e = tma_one<S, TY_, NS_, true, GEN>(op, m, A, st);            \
+            return e != cudaSuccess ? e : tma_one<S, TY_, NS_, false, GEN>(op, m, A, st); \
+        }                                                                                 \
+        return t1 ? tma_one<S, TY_, NS_, true, GEN>(op, m, A, st)                         \
+                  : tma_one<S, TY_, NS_, false, GEN>(op, m, A, st);                       \
     }
     LBSC_TMA_CASE(4, 1)
     LBSC_TMA_CASE(4, 2)
-    LBSC_TMA_CASE(4, 3)
-    LBSC_TMA_CASE(8, 1)
-    LBSC_TMA_CASE(8, 2)
-    LBSC_TMA_CASE(8, 3)
-    if constexpr (sizeof(S) == 2) {
+    if constexpr (!GEN || sizeof(S) == 2) {
+        LBSC_TMA_CASE(8, 1)
+        LBSC_TMA_CASE(8, 2)
+    }
+    if constexpr (!GEN) {
+        LBSC_TMA_CASE(4, 3)
+        LBSC_TMA_CASE(8, 3)
+    }
+    if constexpr (!GEN && sizeof(S) == 2) {
         LBSC_TMA_CASE(16, 1)
         LBSC_TMA_CASE(16, 2)
     }

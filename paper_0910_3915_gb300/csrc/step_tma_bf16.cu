@@ -7,7 +7,7 @@ template <>
 long long tma_step<__nv_bfloat16>(int op, int tile_y, int stages, bool tau_one, const CUtensorMap* map,
                         const StepArgs<__nv_bfloat16>* args, cudaStream_t stream)
 {
-    return tma_dispatch<__nv_bfloat16>(op, tile_y, stages, tau_one, map, args, stream);
+    return tma_dispatch<__nv_bfloat16, false>(op, tile_y, stages, tau_one, map, args, stream);
 }
 
 template <>

@@ -7,7 +7,7 @@ template <>
 long long tma_step<__half>(int op, int tile_y, int stages, bool tau_one, const CUtensorMap* map,
                         const StepArgs<__half>* args, cudaStream_t stream)
 {
-    return tma_dispatch<__half>(op, tile_y, stages, tau_one, map, args, stream);
+    return tma_dispatch<__half, false>(op, tile_y, stages, tau_one, map, args, stream);
 }
 
 template <>

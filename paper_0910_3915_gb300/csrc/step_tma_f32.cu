@@ -7,7 +7,7 @@ template <>
 long long tma_step<float>(int op, int tile_y, int stages, bool tau_one, const CUtensorMap* map,
                         const StepArgs<float>* args, cudaStream_t stream)
 {
-    return tma_dispatch<float>(op, tile_y, stages, tau_one, map, args, stream);
+    return tma_dispatch<float, false>(op, tile_y, stages, tau_one, map, args, stream);
 }
 
 template <>
