@@ -249,7 +249,8 @@ static const Schedule& schedule(lb_ctx* c)
     const int tys[2] = {c->tile_y_req ? c->tile_y_req : 4, c->tile_y_req || c->prec == LB_F32 || !tau_one(c) ? 0 : 8};
     // TMA asked for by name takes three stages, else two
     for (int ty : tys) {
-        if (!ty || c->variant == LB_STEP_LDG) continue;
+        // (the TMA kernels address a plane with 32-bit byte offsets)
+        if (!ty || c->variant == LB_STEP_LDG || c->L.plane * 2 * (long long)elem_size(c->prec) >= (1LL << 32)) continue;
         int stages[2] = {1, 2};
         if (c->variant == LB_STEP_TMA) stages[0] = 3;
         if (!tau_one(c) && c->variant == LB_STEP_AUTO) stages[0] = 2;  // holds v in fewer registers than one stage does

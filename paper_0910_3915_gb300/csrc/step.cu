@@ -37,7 +37,7 @@ __device__ __forceinline__ void step_item(const StepArgs<S>& A, int col, int za,
     const float ref[2] = {A.P.ref[0], A.P.ref[1]};
     const float tau[2] = {A.P.tau[0], A.P.tau[1]};
     const float itau[2] = {A.P.itau[0], A.P.itau[1]};
-    const float gk = A.P.gk, Gax = A.P.Gax, Gdi = A.P.Gdi;
+    const float gk = A.P.gk, Gax = A.P.Gax;
     const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
 
     // tile rows [y0, y0 + hgt): the tiles_y tiles split the ny rows evenly
@@ -151,7 +151,7 @@ __device__ __forceinline__ void step_item(const StepArgs<S>& A, int col, int za,
     reduce(za, rc, jc, vc, mc);
     issue(za + 1);
 
-    Dest D;
+    Dest<S, false> D;
     D.set_column(L, valid ? gx : 0, valid ? gy : 0);
     D.err = A.err;
     D.hoff = A.hkey;
@@ -171,7 +171,7 @@ __device__ __forceinline__ void step_item(const StepArgs<S>& A, int col, int za,
         if (valid && !self_solid) {
             float F[2][3];
             sc_force<HX, HY>(&sp[(z - 1) & 3][0][0], &sp[z & 3][0][0], &sp[(z + 1) & 3][0][0], ty, tx,
-                             gk, Gax, Gdi, F);
+                             gk, Gax, F);
             if constexpr (kGeneral) {
                 D.zo[0] = wrapi(z - 1, nz) * plane;
                 D.zo[2] = wrapi(z + 1, nz) * plane;
@@ -182,7 +182,7 @@ __device__ __forceinline__ void step_item(const StepArgs<S>& A, int col, int za,
             D.zo[1] = z * plane;
             D.bot = !kGeneral && z - 1 == 0 && !(A.halo & 1);  // a halo plane takes pushes like fluid
             D.top = !kGeneral && z + 1 == nz - 1 && !(A.halo & 2);
-            collide_store<S, kGeneral, kTauOne>(rc, jc, vc, F, tau, itau, ref, dst, L, gx, gy, D, mc, clk);
+            collide_store<S, kGeneral, kTauOne>(rc, jc, vc, F, tau, itau, ref, dst, L, D, mc, clk);
         }
         // rotate: next plane becomes current
 #pragma unroll

@@ -156,13 +156,13 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
 
     const Layout L = A.L;
     const int nx = L.nx, ny = L.ny, nz = L.nz;
-    const long long plane = L.plane;
+    const int plane = (int)L.plane;
     S* __restrict__ dst = A.dst;
     const float eta[2] = {A.P.eta[0], A.P.eta[1]};
     const float ref[2] = {A.P.ref[0], A.P.ref[1]};
     const float tau[2] = {A.P.tau[0], A.P.tau[1]};
     const float itau[2] = {A.P.itau[0], A.P.itau[1]};
-    const float gk = A.P.gk, Gax = A.P.Gax, Gdi = A.P.Gdi;
+    const float gk = A.P.gk, Gax = A.P.Gax;
     const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
 
     // rows [y0, y0 + hgt) of an even split of ny (hgt <= TY); a row past hgt is an idle warp
@@ -285,7 +285,7 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
 #pragma unroll
         for (int q = 0; q < NIT; ++q) solid_it[q] = solid_own;
         if constexpr (kGeneral) {
-            const uint32_t* mask = A.nbmask + (long long)wrapi(zp, nz) * plane;
+            const uint32_t* mask = A.nbmask + wrapi(zp, nz) * plane;
             nb = own_rd ? __ldg(mask + own_node) : kSelfSolid;
             solid_own = (nb & kSelfSolid) != 0;
 #pragma unroll
@@ -390,7 +390,7 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
         for (int i = 0; i < NS && i < np; ++i) issue(za - 1 + i, g + i);
     if (!consume(0, rn, jn, vn, mn, nbn) || !consume(1, rc, jc, vc, mc, nbc)) return false;
 
-    Dest D;
+    Dest<S, sizeof(S) == 4> D;
     D.set_column(L, valid ? gx : 0, valid ? gy : 0);
     D.err = A.err;
     D.hoff = A.hkey;
@@ -399,10 +399,10 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
         if (!consume(z - za + 2, rn, jn, vn, mn, nbn)) return false;
         if (valid && !(kGeneral && (nbc & kSelfSolid))) {
             float F[2][3];
-            sc_force<HX, HY>(psi_plane(z - 1), psi_plane(z), psi_plane(z + 1), ty, tx, gk, Gax, Gdi, F);
-            D.zo[0] = (int)((kGeneral ? wrapi(z - 1, nz) : z - 1) * plane);
-            D.zo[1] = (int)(z * plane);
-            D.zo[2] = (int)((kGeneral ? wrapi(z + 1, nz) : z + 1) * plane);
+            sc_force<HX, HY>(psi_plane(z - 1), psi_plane(z), psi_plane(z + 1), ty, tx, gk, Gax, F);
+            D.zo[0] = (kGeneral ? wrapi(z - 1, nz) : z - 1) * plane;
+            D.zo[1] = z * plane;
+            D.zo[2] = (kGeneral ? wrapi(z + 1, nz) : z + 1) * plane;
             D.bot = !kGeneral && z - 1 == 0 && !(A.halo & 1);  // a halo plane takes pushes like fluid
             D.top = !kGeneral && z + 1 == nz - 1 && !(A.halo & 2);
             D.nb = nbc;
@@ -410,9 +410,9 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
                 // rho = rho_ref + m36 / 36, as moments2 forms it: not held across the plane
                 const float2 r = fma2(f2(mc[0], mc[1]), sp2(1.0f / 36.0f), f2(ref[0], ref[1]));
                 const float rr[2] = {r.x, r.y};
-                collide_store<S, kGeneral, kTauOne>(rr, jc, vc, F, tau, itau, ref, dst, L, gx, gy, D, mc, clk);
+                collide_store<S, kGeneral, kTauOne>(rr, jc, vc, F, tau, itau, ref, dst, L, D, mc, clk);
             } else {
-                collide_store<S, kGeneral, kTauOne>(rc, jc, vc, F, tau, itau, ref, dst, L, gx, gy, D, mc, clk);
+                collide_store<S, kGeneral, kTauOne>(rc, jc, vc, F, tau, itau, ref, dst, L, D, mc, clk);
             }
         }
         nbc = nbn;
