@@ -4,11 +4,14 @@
 #include "../../include/lbsc.h"
 #include "lb_fields.cuh"
 
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
+#include <thread>
 #include <vector>
 
 using namespace lbsc;
@@ -52,7 +55,7 @@ struct lb_ctx {
     Schedule sched;  // ty = 0: not chosen since the last change
     long long steps = 0;
     // CUDA graphs of 2^i steps (i = 0 .. kGraphLevels - 1) for each starting buffer
-    static constexpr int kGraphLevels = 6;
+    static constexpr int kGraphLevels = 5;  // (a sixth, of 32 steps, took half of the 0.44 ms that capturing them takes)
     cudaGraphExec_t graph[2][kGraphLevels] = {};
     int variant = LB_STEP_AUTO, stages = 0;  // step kernel selection
     CUtensorMap tmap[2][3][4];               // per buffer, per tile height 4/8/16: main box, x strip, y row, corner
@@ -440,6 +443,8 @@ extern "C" {
 static int check_device_status(lb_ctx* c);
 }
 
+static void context_added();  // the readback's staging blocks live as long as there are contexts
+
 static int init_common(lb_ctx** out, int nx, int ny, int nz, int precision, const double* rho_r,
                        const double* rho_b, void* stream, void* ext, size_t ext_bytes, int halo = 0, int zbase = 0,
                        const double* ref = nullptr)
@@ -457,6 +462,7 @@ static int init_common(lb_ctx** out, int nx, int ny, int nz, int precision, cons
 
     lb_ctx* c = new (std::nothrow) lb_ctx();
     if (!c) return fail(nullptr, LB_ERR_CUDA, "lb_init: out of host memory");
+    context_added();
     c->nx = nx;
     c->ny = ny;
     c->nz = nz;
@@ -814,7 +820,7 @@ int lb_step(lb_ctx* c, int nsteps)
 {
     if (!c || nsteps < 0) return fail(c, LB_ERR_ARG, "lb_step: bad argument");
     if (nsteps == 0) return LB_OK;
-    // n steps as graphs of 2^i steps: one launch per set bit (and per 32 steps),
+    // n steps as graphs of 2^i steps: one launch per set bit (and per 16 steps),
     // so that consecutive kernels follow each other without host launch gaps
     const int rc = capture_graphs(c);
     if (rc != LB_OK) return rc;
@@ -843,6 +849,154 @@ int lb_sync(lb_ctx* c)
 }
 
 }  // extern "C"
+
+// ---------------------------------------------------------------- readback of FP32 fields into FP64 host arrays
+// A field's chunks are copied into one half of a pinned staging block while the
+// other half is converted into the caller's array, by several threads for
+// large fields: a large caller array is fresh memory, whose first touch
+// (3.5 ms for the 67 MB of a 256x256x128 field) is most of the time, and a
+// pageable copy into a temporary vector, cleared first, most of the rest. Two
+// fields of 256x256x128: 10.5 ms, now 3.2; of 128^3 with the velocity 4.7, now 1.7; of 64^3 0.23 both ways.
+namespace {
+constexpr size_t kStageValues = 1 << 20;  // FP32 values of a half
+
+// Staging blocks (two halves of 4 MB) are kept between calls, at most four,
+// and released with the last context.
+struct Staging {
+    std::mutex mu;
+    std::vector<float*> free;
+    int contexts = 0;
+    float* take()
+    {
+        {
+            std::lock_guard<std::mutex> lock(mu);
+            if (!free.empty()) {
+                float* p = free.back();
+                free.pop_back();
+                return p;
+            }
+        }
+        float* p = nullptr;
+        return cudaMallocHost((void**)&p, 2 * kStageValues * sizeof(float)) == cudaSuccess ? p : nullptr;
+    }
+    void give(float* p)
+    {
+        {
+            std::lock_guard<std::mutex> lock(mu);
+            if (free.size() < 4 && contexts > 0) {
+                free.push_back(p);
+                return;
+            }
+        }
+        cudaFreeHost(p);
+    }
+    void add_context()
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        ++contexts;
+    }
+    void drop_context()
+    {
+        std::vector<float*> old;
+        {
+            std::lock_guard<std::mutex> lock(mu);
+            if (--contexts == 0) old.swap(free);
+        }
+        for (float* p : old) cudaFreeHost(p);
+    }
+};
+Staging& staging()
+{
+    static Staging* s = new Staging;  // outlives the contexts a program frees at its exit
+    return *s;
+}
+
+struct Readback {
+    const float* src;  // device
+    double* dst;       // host
+};
+
+// Wait for stream st and fill the host arrays of n fields of N values each.
+cudaError_t read_back(const Readback* f, int n, long long N, cudaStream_t st)
+{
+    struct Chunk {
+        const float* src;
+        double* dst;
+        size_t values;
+    };
+    std::vector<Chunk> chunks;
+    for (int i = 0; i < n; ++i)
+        for (long long o = 0; o < N; o += kStageValues)
+            chunks.push_back({f[i].src + o, f[i].dst + o, (size_t)(N - o < (long long)kStageValues ? N - o : kStageValues)});
+    float* stage = staging().take();
+    if (!stage) return cudaErrorMemoryAllocation;
+    cudaEvent_t ev = nullptr;
+    cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e != cudaSuccess) {
+        staging().give(stage);
+        return e;
+    }
+    const int total = (int)chunks.size();
+    const unsigned hw = std::thread::hardware_concurrency();
+    // a thread for every 2^18 values of a field, up to 8 and half the cores; below two this one does it (8 threads for the
+    // 2^18 values of 64^3 took longer to start than the conversion: 0.58 against 0.2 ms)
+    int workers = (int)(N >> 18 < 8 ? N >> 18 : 8);
+    workers = workers > (int)(hw / 2) ? (int)(hw / 2) : workers;
+    if (workers < 2) workers = 0;
+    std::atomic<int> ready{0};  // chunks that have landed
+    std::atomic<int> done{0};   // shares of chunks converted
+    auto share = [&](int i, int w, int of) {
+        const size_t lo = chunks[i].values * (size_t)w / of, hi = chunks[i].values * (size_t)(w + 1) / of;
+        const float* src = stage + (size_t)(i & 1) * kStageValues;
+        double* dst = chunks[i].dst;
+        for (size_t v = lo; v < hi; ++v) dst[v] = src[v];
+    };
+    std::vector<std::thread> pool;
+    auto work = [&](int w, int of) {
+        for (int i = 0; i < total; ++i) {
+            int r;
+            while ((r = ready.load(std::memory_order_acquire)) <= i) {
+                if (r < 0) return;  // given up
+                std::this_thread::yield();
+            }
+            share(i, w, of);
+            done.fetch_add(1, std::memory_order_release);
+        }
+    };
+    // the threads' number is needed by each: created one after the other, they start on the first chunk only when it is ready
+    try {
+        for (int w = 0; w < workers; ++w) pool.emplace_back(work, w, workers);
+    } catch (...) {  // no more threads: the ones created stop, this thread converts alone
+        ready.store(-1, std::memory_order_release);
+        for (std::thread& t : pool) t.join();
+        pool.clear();
+        ready.store(0, std::memory_order_relaxed);
+        workers = 0;
+    }
+    auto copy = [&](int i) {
+        return cudaMemcpyAsync(stage + (size_t)(i & 1) * kStageValues, chunks[i].src, chunks[i].values * sizeof(float),
+                               cudaMemcpyDeviceToHost, st);
+    };
+    e = copy(0);
+    for (int i = 0; i < total && e == cudaSuccess; ++i) {
+        e = cudaEventRecord(ev, st);
+        if (e == cudaSuccess) e = cudaEventSynchronize(ev);
+        if (e != cudaSuccess) break;
+        // chunk i + 1 goes where chunk i - 1 was, once that is converted
+        while (workers && done.load(std::memory_order_acquire) < i * workers) std::this_thread::yield();
+        if (i + 1 < total) e = copy(i + 1);
+        if (workers) ready.store(i + 1, std::memory_order_release);
+        else share(i, 0, 1);
+    }
+    if (e != cudaSuccess && workers) ready.store(-1, std::memory_order_release);
+    for (std::thread& t : pool) t.join();
+    if (e != cudaSuccess) cudaStreamSynchronize(st);  // no copy into the block is left in flight
+    cudaEventDestroy(ev);
+    staging().give(stage);
+    return e;
+}
+}  // namespace
+static void context_added() { staging().add_context(); }
 
 template <class S>
 static cudaError_t run_cons(lb_ctx* c, float* phi)
@@ -922,25 +1076,18 @@ int lb_moments(lb_ctx* c, double* rho_r, double* rho_b, double* u, double cons[8
 {
     if (!c) return fail(c, LB_ERR_ARG, "lb_moments: NULL context");
     const long long N = (long long)c->nx * c->ny * c->nz;
-    if (rho_r || rho_b || u) {
-        LB_CUDA(c, dispatch_fields(c, u != nullptr));
-        std::vector<float> tmp((size_t)N);
-        auto pull = [&](const float* src, double* dst) -> int {
-            LB_CUDA(c, cudaMemcpyAsync(tmp.data(), src, N * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
-            LB_CUDA(c, cudaStreamSynchronize(c->stream));
-            for (long long i = 0; i < N; ++i) dst[i] = tmp[i];
-            return LB_OK;
-        };
-        int rc;
-        if (rho_r && (rc = pull(c->W.rho[0], rho_r)) != LB_OK) return rc;
-        if (rho_b && (rc = pull(c->W.rho[1], rho_b)) != LB_OK) return rc;
-        if (u)
-            for (int d = 0; d < 3; ++d)
-                if ((rc = pull(c->W.u[d], u + d * N)) != LB_OK) return rc;
-    }
+    Readback fields[5];
+    int n = 0;
+    if (rho_r) fields[n++] = {c->W.rho[0], rho_r};
+    if (rho_b) fields[n++] = {c->W.rho[1], rho_b};
+    for (int d = 0; u && d < 3; ++d) fields[n++] = {c->W.u[d], u + d * N};
+    if (n) LB_CUDA(c, dispatch_fields(c, u != nullptr));
+    LB_CUDA(c, dispatch_cons(c));
+    if (n) LB_CUDA(c, read_back(fields, n, N, c->stream));
     double tmp[8];
-    int rc = lb_conservation(c, tmp);
-    if (cons) memcpy(cons, tmp, sizeof(tmp));
+    int rc = wait(c);
+    if (rc == LB_OK) rc = take_cons(c, tmp);
+    if (cons && (rc == LB_OK || rc == LB_ERR_NAN)) memcpy(cons, tmp, sizeof(tmp));
     return rc;
 }
 
@@ -1197,6 +1344,7 @@ void lb_free(lb_ctx* c)
     if (c->h_red) cudaFreeHost(c->h_red);
     if (c->cap) cudaStreamDestroy(c->cap);
     delete c;
+    staging().drop_context();
 }
 
 }  // extern "C"

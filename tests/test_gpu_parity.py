@@ -705,3 +705,25 @@ def test_general_geometry_kernels_agree_at_tile_edges(lbsc, dims, precision):
                  for v in ("auto", "ldg")]
             fluid = np.broadcast_to(solid == 0, n[0].shape)
             assert np.array_equal(n[0][fluid], n[1][fluid])
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 3), (100, 70, 75), (127, 129, 64), (1024, 513, 4)])
+def test_readback_in_chunks_equals_the_populations(lbsc, dims):
+    """Fields below, at and above a staging half (2^20 values), converted by this thread alone and by several: densities
+    are the FP32 sums of the populations in their order, the velocity of a uniform moving state is that state's."""
+    nx, ny, nz = dims
+    rng = np.random.Generator(np.random.PCG64(nx))
+    rr, rb = rng.uniform(0.05, 0.7, size=(2, nz, ny, nx))
+    lat = lbsc.Lattice(rr, rb)
+    for _ in range(2):  # the second call takes the staging block of the first
+        r, b, u, cons = lat.moments(velocity=True)
+        n = lat.populations().astype(np.float32)
+        s = [np.zeros((nz, ny, nx), np.float32) for _ in range(2)]
+        for k in range(19):
+            for a in range(2):
+                s[a] = s[a] + n[a, k]
+        fluid = slice(1, nz - 1)
+        assert np.array_equal(r[fluid], s[0][fluid].astype(np.float64)) and np.array_equal(b[fluid], s[1][fluid].astype(np.float64))
+        assert np.all(r[[0, -1]] == 0) and np.all(np.abs(u) < 1e-6) and cons[6] == nx * ny * (nz - 2)
+        r1, b1, none, _ = lat.moments()
+        assert none is None and np.array_equal(r1, r) and np.array_equal(b1, b)
