@@ -51,8 +51,10 @@ __device__ __forceinline__ float add_c(float s, int c, float v) { return c == 0 
 template <class S>
 __global__ void __launch_bounds__(kAdjThreads) adj_forward_kernel(Layout L, KParams P, const S* __restrict__ f, AdjState A)
 {
+    grid_trigger();
     const int N = L.nx * L.ny * L.nz;
     const int i = blockIdx.x * kAdjThreads + threadIdx.x;
+    grid_wait();  // every thread of a dependent launch waits, so that the launch's end implies the earlier kernels'
     if (i >= N) return;
     int x, y, z;
     node_xyz(i, L.nx, L.ny, x, y, z);
@@ -95,9 +97,11 @@ __global__ void __launch_bounds__(kAdjThreads) adj_forward_kernel(Layout L, KPar
 // (before the psi term) rhobar into E(t), M(t) where tau != 1, and V and psibar
 // for pass B. The wall gradient of the block is added to its own row of
 // part[block][2] (FP64), which one pass sums after the last step.
-// Issue-bound (about 1500 FP32 operations a node, 25 of them divisions): the
-// neighbours' E and psi are L1/L2 hits, 8-byte loads of both components.
-// 25 us at 64^3; 75 when it read and wrote lambda's 38 values. One thread summed
+// Bound by the latency of its 68 loads of neighbours' E and psi (8 bytes, both components; L1/L2 hits) and about 1400
+// instructions, 25 of them divisions: packed lanes for the two components were slower (20.6 against 20.3 ms for the
+// gradient below), and so were 6 to 8 blocks an SM instead of 5.
+// 25 us at 64^3; 75 when it read and wrote lambda's 38 values. The passes are launched dependently: a gradient over 300
+// steps at 64^3 21.8 -> 20.3 ms. One thread summed
 // the blocks' rows after every step before (32 us).
 template <bool kTauOne>
 __global__ void __launch_bounds__(kAdjThreads)
@@ -107,10 +111,12 @@ __global__ void __launch_bounds__(kAdjThreads)
     const int nx = G.nx, ny = G.ny, nz = G.nz;
     const int N = nx * ny * nz;
     const int i = blockIdx.x * kAdjThreads + threadIdx.x;
+    grid_trigger();
     double geta[2] = {0.0, 0.0};
     bool at_wall = false;
     int x = 0, y = 0, z = 0;
     if (i < N) node_xyz(i, nx, ny, x, y, z);
+    grid_wait();
     if (i < N && !wall_z(z, nz)) {
         const int xo[3] = {wrapi(x - 1, nx), x, wrapi(x + 1, nx)};
         const int yo[3] = {wrapi(y - 1, ny), y, wrapi(y + 1, ny)};
@@ -281,9 +287,11 @@ __global__ void __launch_bounds__(kAdjThreads) adj_gather_kernel(AdjArgs G, AdjS
     const int nx = G.nx, ny = G.ny, nz = G.nz;
     const int N = nx * ny * nz;
     const int i = blockIdx.x * kAdjThreads + threadIdx.x;
-    if (i >= N) return;
+    grid_trigger();
     int x, y, z;
-    node_xyz(i, nx, ny, x, y, z);
+    node_xyz(i < N ? i : 0, nx, ny, x, y, z);
+    grid_wait();
+    if (i >= N) return;
     if (wall_z(z, nz)) return;
     const int xo[3] = {wrapi(x - 1, nx), x, wrapi(x + 1, nx)};
     const int yo[3] = {wrapi(y - 1, ny), y, wrapi(y + 1, ny)};
@@ -416,18 +424,17 @@ static int adj_blocks(long long n) { return (int)((n + kAdjThreads - 1) / kAdjTh
 template <class S>
 cudaError_t launch_adj_forward(const Layout& L, const KParams& P, const S* f, const AdjState& A, cudaStream_t st)
 {
-    adj_forward_kernel<S><<<adj_blocks((long long)L.nx * L.ny * L.nz), kAdjThreads, 0, st>>>(L, P, f, A);
-    return cudaGetLastError();
+    return launch_after(adj_forward_kernel<S>, dim3(adj_blocks((long long)L.nx * L.ny * L.nz)), kAdjThreads, 0, st, L, P, f, A);
 }
 
 cudaError_t launch_adj_backstep(const AdjArgs& G, const AdjState& A, bool tau_one, const AdjE& En, const float* Mn,
                                 const AdjE& Ec, float* Mc, const AdjV& W, double* part, cudaStream_t st)
 {
     const int blocks = adj_blocks((long long)G.nx * G.ny * G.nz);
-    if (tau_one) adj_local_kernel<true><<<blocks, kAdjThreads, 0, st>>>(G, A, En, Mn, Ec, Mc, W, part);
-    else adj_local_kernel<false><<<blocks, kAdjThreads, 0, st>>>(G, A, En, Mn, Ec, Mc, W, part);
-    adj_gather_kernel<<<blocks, kAdjThreads, 0, st>>>(G, A, W, Ec);
-    return cudaGetLastError();
+    const cudaError_t e = launch_after(tau_one ? adj_local_kernel<true> : adj_local_kernel<false>, dim3(blocks), kAdjThreads, 0,
+                                       st, G, A, En, Mn, Ec, Mc, W, part);
+    if (e != cudaSuccess) return e;
+    return launch_after(adj_gather_kernel, dim3(blocks), kAdjThreads, 0, st, G, A, W, Ec);
 }
 
 cudaError_t launch_rows_sum(const double* part, int nblocks, double* out, cudaStream_t st)
