@@ -430,12 +430,12 @@ __device__ __noinline__ void add_crossing(float2* acc, int stride, int x, int y,
 // All in pairs of FP32 numbers: with FP64 sums (a drained queue took about 70
 // FP64 operations, 2240 cycles of an SM's one FP64 lane) the kernel took 53 us
 // at 128^3, bound by the SMs that met the most crossings. A block takes rows
-// gridDim apart for the same reason: the drop's rows spread over all SMs. Now 30 us at 128^3 (9 million
+// gridDim apart for the same reason: the drop's rows spread over all SMs. Now 27 us at 128^3 (9 million
 // instructions, a third of them for crossings; phi is 8 MB, in L2).
 // A thread's sums wait in shared memory, and a warp reduces a value only if one
 // of its lanes holds a contribution to it. The last block to finish adds the
 // blocks' rows, in order, and writes the 19 values lb_contact_angle works with.
-__global__ void __launch_bounds__(kAngleThreads) angle_kernel(FieldArgs F, AngleArgs A, const float* __restrict__ P,
+__global__ void __launch_bounds__(kAngleThreads, 3) angle_kernel(FieldArgs F, AngleArgs A, const float* __restrict__ P,
                                                               float2* __restrict__ part, unsigned int* __restrict__ ticket,
                                                               double* __restrict__ out)
 {
@@ -444,6 +444,7 @@ __global__ void __launch_bounds__(kAngleThreads) angle_kernel(FieldArgs F, Angle
     __shared__ float2 sacc[16][kAngleThreads];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int i = 0; i < 16; ++i) sacc[i][tid] = make_float2(i == 0 ? kNoTop : 0.f, 0.f);
+    grid_wait();  // for the pass that wrote phi
     float pmax = -3.0e38f, pmin = 3.0e38f;
     const unsigned nxy = (unsigned)nx * (unsigned)ny;
     // Interface crossings are rare and scattered: a lane that meets one would
@@ -1068,8 +1069,7 @@ cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, doub
     A.z0 = z0 < (double)F.L.nz ? (int)z0 : F.L.nz;
     const int rows = F.L.ny * F.L.nz, warps = kAngleThreads / 32;
     const int blocks = (rows + warps - 1) / warps < kAngleBlocks ? (rows + warps - 1) / warps : kAngleBlocks;
-    angle_kernel<<<blocks, kAngleThreads, 0, st>>>(F, A, W.rho[0], (float2*)part, ticket, out);
-    return cudaGetLastError();
+    return launch_after(angle_kernel, dim3(blocks), kAngleThreads, 0, st, F, A, W.rho[0], (float2*)part, ticket, out);
 }
 
 template <class S>

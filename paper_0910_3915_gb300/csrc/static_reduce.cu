@@ -67,12 +67,13 @@ __device__ __forceinline__ void add_eight(const double (&v)[kStaticUnroll], doub
 // sum with its test for finite values 2), and a block's threads are summed by
 // one warp. The moments are formed from the 38 totals in static_finish_kernel.
 // 64^3: 147 us with whole nodes in 128 blocks, 39 with a plain sum, about 15
-// now (both kernels in a stream 26.7 a call; 128^3 116, 0.83 of the measured bandwidth).
+// now (both kernels, the second launched dependently, 24.6 a call; 128^3 116, 0.83 of the measured bandwidth).
 __global__ void __launch_bounds__(kStaticThreads)
     static_sum_kernel(const double* __restrict__ n, const uint8_t* __restrict__ solid, long long N, int chunks,
                       double* __restrict__ part)
 {
     const int c = blockIdx.x, ak = blockIdx.y;
+    grid_trigger();
     const long long lo = c * N / chunks, hi = (c + 1) * N / chunks;
     const double* __restrict__ p = n + (long long)ak * N;
     double s = 0;
@@ -150,6 +151,7 @@ __global__ void __launch_bounds__(1024) static_finish_kernel(const double* __res
     __shared__ int num[2 * Q + 1];
     const int* count = (const int*)(part + 2 * Q * chunks);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    grid_wait();
     for (int r = warp; r <= 2 * Q; r += 32) {
         double t = 0;
         int b = 0;
@@ -246,8 +248,8 @@ extern "C" int lb_conservation_static(const double* populations, const uint8_t* 
     const long long want = (N + kStaticMinNodes - 1) / kStaticMinNodes;
     const int chunks = (int)(want < kStaticChunks ? want : kStaticChunks);
     static_sum_kernel<<<dim3(chunks, 2 * Q), kStaticThreads, 0, st>>>(populations, solid, N, chunks, part);
-    static_finish_kernel<<<1, 1024, 0, st>>>(part, chunks, cons);
-    const cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_after(static_finish_kernel, dim3(1), 1024, 0, st, part, chunks, cons);
     if (e != cudaSuccess) {
         lbsc_set_global_error(std::string("lb_conservation_static: launch: ") + cudaGetErrorString(e));
         return LB_ERR_CUDA;
