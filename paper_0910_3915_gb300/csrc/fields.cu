@@ -796,7 +796,7 @@ __global__ void __launch_bounds__(kPressThreads) pressure_field_kernel(FieldArgs
 // Sums over the fluid nodes of a plane (blockIdx.x) and a range of its nodes
 // (one of `split` equal ones, blockIdx.y) of the six components, phi = rho_r -
 // rho_b and the count -> out[(z * split + range) * 8 + v]. A thread sums its
-// nodes in FP32 pairs (as node_pressure), then FP64 across threads.
+// nodes in FP32 pairs (as node_pressure), as do the threads of a warp; then FP64 across warps.
 // Bound by the pairs' arithmetic (2180 instructions a node at half the issue rate, five blocks an SM): 110 us at 96^3; the
 // sums in FP64, one block a plane, took 1480.
 template <class S>
@@ -809,6 +809,7 @@ __global__ void __launch_bounds__(kPressThreads, 5) pressure_plane_kernel(FieldA
     for (int v = 0; v < 7; ++v) sum[v] = two(0.f);
     double odd[6] = {0, 0, 0, 0, 0, 0};  // nodes taken in FP64
     int count = 0;
+    bool odd_nodes = false;
     for (int c = lo + threadIdx.x; c < hi; c += kPressThreads) {
         const int y = c / nx, x = c - y * nx;
         if (node_solid(F, x, y, z, F.L.off(x, y, z))) continue;
@@ -821,26 +822,44 @@ __global__ void __launch_bounds__(kPressThreads, 5) pressure_plane_kernel(FieldA
             double D[6];
             node_pressure_f64<S>(F, f, W, x, y, z, D);
             for (int v = 0; v < 6; ++v) odd[v] += D[v];
+            odd_nodes = true;
         }
         sum[6] = norm2(sum[6] + two_sum(W.rho[0][i], -W.rho[1][i]));
         ++count;
     }
-    double acc[8];
-#pragma unroll
-    for (int v = 0; v < 7; ++v) acc[v] = to_f64(sum[v]) + (v < 6 ? odd[v] : 0.0);
-    acc[7] = (double)count;
-    __shared__ double sh[kPressThreads / 32][8];
+    __shared__ float2 sh[kPressThreads / 32][7];
+    __shared__ double sodd[kPressThreads / 32][6];
+    __shared__ int sn[kPressThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int v = 0; v < 8; ++v) {
-        const double t = warp_sum(acc[v]);
-        if (lane == 0) sh[warp][v] = t;
+    for (int v = 0; v < 7; ++v) {
+        Two t = sum[v];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const Two w{__shfl_down_sync(0xffffffffu, t.h, o), __shfl_down_sync(0xffffffffu, t.l, o)};
+            t = norm2(t + w);
+        }
+        if (lane == 0) sh[warp][v] = make_float2(t.h, t.l);
     }
-    __syncthreads();
+    count = __reduce_add_sync(0xffffffffu, count);
+    if (lane == 0) sn[warp] = count;
+    const bool any_odd = __syncthreads_or(odd_nodes);
+    if (any_odd) {  // uniform
+        for (int v = 0; v < 6; ++v) {
+            const double t = warp_sum(odd[v]);
+            if (lane == 0) sodd[warp][v] = t;
+        }
+        __syncthreads();
+    }
     if (threadIdx.x < 8) {
+        const int v = threadIdx.x;
         double t = 0;
-        for (int w = 0; w < kPressThreads / 32; ++w) t += sh[w][threadIdx.x];
-        out[((size_t)z * split + blockIdx.y) * 8 + threadIdx.x] = t;
+        for (int w = 0; w < kPressThreads / 32; ++w) {
+            if (v < 7) t += (double)sh[w][v].x + (double)sh[w][v].y;
+            else t += (double)sn[w];
+            if (any_odd && v < 6) t += sodd[w][v];
+        }
+        out[((size_t)z * split + blockIdx.y) * 8 + v] = t;
     }
 }
 
@@ -860,85 +879,109 @@ __global__ void plane_rows_kernel(const double* __restrict__ part, int nz, int s
 // P_T = (tr P - P_N)/2, phi and 1. Sums are kept in 64-bit fixed point
 // (units of 2^-30) so that the atomic accumulation is exact and the result
 // does not depend on the order the nodes are added in.
-// The bin comes from an FP32 root of the FP64 r^2; only where that lies within
-// its rounding of a bin's edge is it taken from the FP64 root and quotient. A
+// Offsets, r^2, P_N and the fixed-point values are formed in FP32 pairs too (65
+// FP64 operations a node were what bounded the pass), the bin from an FP32 root;
+// only where that lies within its rounding of a bin's edge, a periodic offset near
+// half the box, a value out of range or not finite, is the node taken in FP64. A
 // block gathers its nodes' sums in shared memory as 32-bit words (the low 16
 // and the high bits of a value apart: 64-bit adds in shared memory are loops)
 // and adds them to the global bins at its end; a value too large for that
 // goes to the global bins at once.
-// As the plane sums, plus about 30 FP64 operations a node for the radius and the split into words: 155 us at 96^3, 1230 with
-// the tensor, three divisions and 64-bit shared-memory adds in FP64.
+// 96^3 (the call with the moment fields and the readback): 1.3 ms with the tensor, three divisions and 64-bit shared-memory
+// adds in FP64, 214 us with the tensor in pairs alone, 153 now; six blocks an SM (with five 7% longer).
+// round(v 2^30) of a pair below 2^20
+__device__ __forceinline__ long long to_fix30(Two v)
+{
+    const float h = __fmul_rn(v.h, (float)kRadialFix), a = rintf(h);
+    return __float2ll_rn(a) + (long long)__float2int_rn(__fmaf_rn(v.l, (float)kRadialFix, __fsub_rn(h, a)));
+}
+
+// The FP64 form of a node's values v[3] (P_N, P_T, phi in units of 2^-30) and
+// bin: false where it falls in none.
+template <class S>
+__device__ __noinline__ bool radial_node_f64(const FieldArgs& F, const S* __restrict__ f, const Scratch& W,
+                                             const RadialArgs& R, int x, int y, int z, long long* v, int* bin)
+{
+    double d[3] = {x - R.c[0], y - R.c[1], z - R.c[2]};
+    d[0] -= F.L.nx * rint(d[0] / F.L.nx);
+    d[1] -= F.L.ny * rint(d[1] / F.L.ny);
+    if (F.general) d[2] -= F.L.nz * rint(d[2] / F.L.nz);
+    const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+    if (!(r > 0)) return false;
+    const double bf = floor(r / R.dr);
+    if (!(bf < R.nbins)) return false;
+    double D[6];
+    node_pressure_f64<S>(F, f, W, x, y, z, D);
+    const double n[3] = {d[0] / r, d[1] / r, d[2] / r};
+    const double T[3][3] = {{D[0], D[3], D[4]}, {D[3], D[1], D[5]}, {D[4], D[5], D[2]}};
+    double pn = 0;
+    for (int a = 0; a < 3; ++a)
+        for (int b = 0; b < 3; ++b) pn += n[a] * T[a][b] * n[b];
+    const size_t i = (size_t)x + (size_t)F.L.nx * (y + (size_t)F.L.ny * z);
+    v[0] = __double2ll_rn(pn * kRadialFix);
+    v[1] = __double2ll_rn(0.5 * (D[0] + D[1] + D[2] - pn) * kRadialFix);
+    v[2] = __double2ll_rn(((double)W.rho[0][i] - (double)W.rho[1][i]) * kRadialFix);
+    *bin = (int)bf;
+    return true;
+}
+
 constexpr int kRadialNodes = 32000;  // most nodes a block takes: its 32-bit sums cannot overflow (below 2^15 nodes of 2^16)
 
 template <class S>
-__global__ void __launch_bounds__(kPressThreads, 5) pressure_radial_kernel(FieldArgs F, const S* __restrict__ f, Scratch W,
-                                                                        double cxx, double cyy, double czz, double dr,
-                                                                        int nbins, double zmin, unsigned per,
-                                                                        unsigned long long* __restrict__ out)
+__global__ void __launch_bounds__(kPressThreads, 6) pressure_radial_kernel(FieldArgs F, const S* __restrict__ f, Scratch W,
+                                                                           RadialArgs R, unsigned per,
+                                                                           unsigned long long* __restrict__ out)
 {
     extern __shared__ unsigned radial_sh[];  // [nbins][7]: low and high words of the three sums, count
+    const int nbins = R.nbins;
     for (int b = threadIdx.x; b < nbins * 7; b += kPressThreads) radial_sh[b] = 0u;
     __syncthreads();
     const int nx = F.L.nx, ny = F.L.ny, nz = F.L.nz;
     const unsigned nxy = (unsigned)nx * (unsigned)ny, N = nxy * (unsigned)nz;
     const unsigned lo = blockIdx.x * per, hi = N - lo < per ? N : lo + per;
-    const float idr = (float)(1.0 / dr);
-    const bool plain_dr = dr > 1e-6 && dr < 1e6;
     for (unsigned i = lo + threadIdx.x; i < hi; i += kPressThreads) {
         const int z = (int)(i / nxy), y = (int)((i - z * nxy) / (unsigned)nx), x = (int)(i - z * nxy - y * nx);
-        if (z < zmin) continue;
-        double d[3] = {x - cxx, y - cyy, z - czz};
-        // v - n rint(v / n): rint is 0 up to |v| = n / 2 (a tie goes to even), where no quotient is needed
-        auto image = [](double v, int n) { return 2 * fabs(v) <= (double)n ? v : v - n * rint(v / n); };
-        d[0] = image(d[0], nx);
-        d[1] = image(d[1], ny);
-        if (F.general) d[2] = image(d[2], nz);
-        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-        if (!(r2 > 0)) continue;
-        const float q = sqrtf((float)r2) * idr;  // r / dr within 3e-7 of itself for the moderate r2 and dr that `fast` asks for
-        const bool fast = plain_dr && r2 > 1e-12 && r2 < 1e12;
-        float bf = floorf(q);
-        if (!fast || fabsf(q - rintf(q)) <= 1e-6f * q) {
-            const double be = floor(sqrt(r2) / dr);
-            if (be >= nbins) continue;
-            bf = (float)be;
-        }
-        if (!(bf < (float)nbins)) continue;
-        if (node_solid(F, x, y, z, F.L.off(x, y, z))) continue;
-        Two P[6];
-        long long v[3];
-        const double phi = (double)W.rho[0][i] - (double)W.rho[1][i];
-        if (node_pressure<S>(F, f, W, x, y, z, P)) {
-            // n.P.n = d.P.d / r^2 in FP32 pairs: d_i as a pair, products of pairs
-            Two e[3];
-#pragma unroll
-            for (int q3 = 0; q3 < 3; ++q3) {
-                e[q3].h = (float)d[q3];
-                e[q3].l = (float)(d[q3] - (double)e[q3].h);
+        if (z < R.z0) continue;
+        // offset from the centre, the nearest image along a periodic axis
+        bool plain = R.plain;
+        auto offset = [&](int at, int q, int n, bool periodic) {
+            Two d = two_sum((float)at, -R.ch[q]);
+            d.l = __fsub_rn(d.l, R.cl[q]);
+            if (periodic) {
+                // near half the box FP64 decides which image it is, but for the plain tie, which keeps its side
+                const float half = 0.5f * (float)n;
+                if (fabsf(d.h) == half && d.l == 0.f) return d;
+                const float m = rintf(d.h / (float)n), rest = fabsf(d.h - m * (float)n);
+                if (fabsf(rest - half) <= 1e-5f * half) plain = false;
+                d = d + two(-m * (float)n);
             }
-            const Two off = (norm2(mul22(P[3], norm2(mul22(e[0], e[1])))) + mul22(P[4], norm2(mul22(e[0], e[2])))) +
-                            mul22(P[5], norm2(mul22(e[1], e[2])));
-            const Two dia = (mul22(P[0], norm2(mul22(e[0], e[0]))) + mul22(P[1], norm2(mul22(e[1], e[1])))) +
-                            mul22(P[2], norm2(mul22(e[2], e[2])));
-            const double num = to_f64(dia + (off + off));
-            const double pn = num / r2;
-            const double tr = to_f64((P[0] + P[1]) + P[2]);
-            v[0] = __double2ll_rn(pn * kRadialFix);
-            v[1] = __double2ll_rn(0.5 * (tr - pn) * kRadialFix);
-        } else {
-            double D[6];
-            node_pressure_f64<S>(F, f, W, x, y, z, D);
-            const double r = sqrt(r2);
-            const double n[3] = {d[0] / r, d[1] / r, d[2] / r};
-            const double T[3][3] = {{D[0], D[3], D[4]}, {D[3], D[1], D[5]}, {D[4], D[5], D[2]}};
-            double pn = 0;
-            for (int a = 0; a < 3; ++a)
-                for (int b = 0; b < 3; ++b) pn += n[a] * T[a][b] * n[b];
-            v[0] = __double2ll_rn(pn * kRadialFix);
-            v[1] = __double2ll_rn(0.5 * (D[0] + D[1] + D[2] - pn) * kRadialFix);
+            return norm2(d);
+        };
+        const Two d[3] = {offset(x, 0, nx, true), offset(y, 1, ny, true), offset(z, 2, nz, F.general != 0)};
+        const Two xx = norm2(mul22(d[0], d[0])), yy = norm2(mul22(d[1], d[1])), zz = norm2(mul22(d[2], d[2]));
+        const Two r2 = norm2((xx + yy) + zz);
+        const float q = sqrtf(r2.h) * R.idr;  // r / dr within 3e-7 of itself
+        plain = plain && r2.h > 1e-6f && r2.h < 1e12f && fabsf(q - rintf(q)) > 1e-6f * q;
+        if (plain && q >= (float)nbins) continue;
+        if (node_solid(F, x, y, z, F.L.off(x, y, z))) continue;
+        int b = (int)q;
+        long long v[3];
+        Two P[6];
+        plain = plain && node_pressure<S>(F, f, W, x, y, z, P);
+        if (plain) {
+            // n.P.n = d.P.d / r^2
+            const Two off = (norm2(mul22(P[3], norm2(mul22(d[0], d[1])))) + mul22(P[4], norm2(mul22(d[0], d[2])))) +
+                            mul22(P[5], norm2(mul22(d[1], d[2])));
+            const Two dia = (mul22(P[0], xx) + mul22(P[1], yy)) + mul22(P[2], zz);
+            const Two pn = div22(norm2(dia + (off + off)), r2);
+            const Two pt = norm2(((P[0] + P[1]) + P[2]) - pn);
+            const Two phi = two_sum(W.rho[0][i], -W.rho[1][i]);
+            plain = fabsf(pn.h) < 1e6f && fabsf(pt.h) < 1e6f && fabsf(phi.h) < 1e6f;
+            v[0] = to_fix30(pn);
+            v[1] = to_fix30(Two{0.5f * pt.h, 0.5f * pt.l});
+            v[2] = to_fix30(phi);
         }
-        v[2] = __double2ll_rn(phi * kRadialFix);
-        const int b = (int)bf;
+        if (!plain && !radial_node_f64<S>(F, f, W, R, x, y, z, v, &b)) continue;
         atomicAdd(&radial_sh[b * 7 + 6], 1u);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -1112,11 +1155,26 @@ cudaError_t launch_pressure_radial(const FieldArgs& F, const S* f, const Scratch
     if (nbins < 1 || nbins > kRadialBinsMax) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long) * 4 * nbins, st);
     if (e != cudaSuccess) return e;
+    RadialArgs R;
+    bool near = true;
+    for (int q = 0; q < 3; ++q) {
+        R.c[q] = centre[q];
+        R.ch[q] = (float)centre[q];
+        R.cl[q] = (float)(centre[q] - (double)R.ch[q]);
+        near = near && std::fabs(centre[q]) < 1e6;
+    }
+    R.dr = dr;
+    R.idr = (float)(1.0 / dr);
+    R.nbins = nbins;
+    const double z0 = std::ceil(zmin);  // z < zmin is z < z0 for whole z
+    R.z0 = z0 < 0 ? 0 : (z0 > F.L.nz ? F.L.nz : (int)z0);
+    // the FP32 pairs hold whole coordinates below 2^24 exactly
+    R.plain = near && dr > 1e-3 && dr < 1e6 && F.L.nx < (1 << 23) && F.L.ny < (1 << 23) && F.L.nz < (1 << 23);
     const long long N = (long long)F.L.nx * F.L.ny * F.L.nz;
     long long per = (N + kRadialBlocks - 1) / kRadialBlocks;
     per = per < kPressThreads ? kPressThreads : (per > kRadialNodes ? kRadialNodes : per);
     pressure_radial_kernel<S><<<(unsigned)((N + per - 1) / per), kPressThreads, (size_t)nbins * 7 * sizeof(unsigned), st>>>(
-        F, f, W, centre[0], centre[1], centre[2], dr, nbins, zmin, (unsigned)per, out);
+        F, f, W, R, (unsigned)per, out);
     return cudaGetLastError();
 }
 

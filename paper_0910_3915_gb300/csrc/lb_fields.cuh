@@ -32,6 +32,15 @@ struct FieldArgs {
     const uint32_t* nbmask;
 };
 
+// Radial bins of the pressure tensor: centre (also as pairs ch + cl), bin
+// width and its inverse, first plane, and whether FP32 pairs serve at all.
+struct RadialArgs {
+    double c[3], dr;
+    float ch[3], cl[3], idr;
+    int nbins, z0;
+    bool plain;
+};
+
 // Unpadded float fields (index x + nx*(y + ny*z)) used by readback kernels.
 struct Scratch {
     float* rho[2];
