@@ -176,7 +176,6 @@ static void set_kparams(lb_ctx* c)
 static bool tau_one(const lb_ctx* c) { return c->prm.tau_r == 1.0 && c->prm.tau_b == 1.0; }
 
 // ---------------------------------------------------------------- TMA step support
-static const int kTmaTiles[3] = {4, 8, 16};
 static int tile_index(int ty) { return ty == 4 ? 0 : (ty == 8 ? 1 : 2); }
 
 // ops of tma_step for the context's geometry
@@ -194,18 +193,6 @@ static long long tma_call(int op, lb_ctx* c, bool general, int ty, int ns)
     case LB_F16: return tma_op<__half>(op, c, general, ty, ns, nullptr, nullptr, nullptr);
     default: return tma_op<__nv_bfloat16>(op, c, general, ty, ns, nullptr, nullptr, nullptr);
     }
-}
-
-// raise the shared-memory limit of every TMA kernel built for this precision
-static cudaError_t tma_prepare(lb_ctx* c)
-{
-    for (int general = 0; general < 2; ++general)
-        for (int ty : kTmaTiles)
-            for (int ns = 1; ns <= 3; ++ns) {
-                const long long e = tma_call(1, c, general != 0, ty, ns);  // cudaErrorInvalidValue: pair not built
-                if (e != (long long)cudaSuccess && e != (long long)cudaErrorInvalidValue) return (cudaError_t)e;
-            }
-    return cudaSuccess;
 }
 
 // Estimated time in microseconds of a step of the TMA kernel on tiles of ty
@@ -261,7 +248,9 @@ static const Schedule& schedule(lb_ctx* c)
         for (int i = 0; i < 2; ++i) {
             const int ns = stages[i];
             if (i && (ns == stages[0] || (best.ty == ty && c->variant == LB_STEP_TMA))) break;
-            // occupancy 0: the pair is not built for this precision (or does not fit)
+            // the shared-memory limit first: the occupancy of a kernel above 48 KB counts 0 without it (only the kernels
+            // asked about are set: raising all of them took 0.3 ms of every lb_init). 0: not built, or does not fit
+            if (tma_call(1, c, c->general, ty, ns) != (long long)cudaSuccess) continue;
             const int occ = (int)tma_call(2, c, c->general, ty, ns);
             if (occ < 1) continue;
             const int base = (ny + ty - 1) / ty;
@@ -520,7 +509,6 @@ static int init_common(lb_ctx** out, int nx, int ny, int nz, int precision, cons
     e = cudaMemsetAsync(c->red, 0, 64 * sizeof(double), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->dev_err, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->clock, 0, 2 * sizeof(uint32_t), c->stream);
-    if (e == cudaSuccess) e = tma_prepare(c);
     if (e != cudaSuccess) return bail(LB_ERR_CUDA, std::string("lb_init: ") + cudaGetErrorString(e));
     // 16-bit deviation references: mean initial density over fluid nodes
     double sum[2] = {0, 0};
@@ -1453,7 +1441,8 @@ static int batch_build_typed(lb_batch* b)
     b->grid = b->box[0]->nsm * (occ > 0 ? occ : 1);
     // Planes an item, where the caller leaves them open: those that give the
     // busiest CTA least. Long items repeat fewer planes, short ones share out
-    // better: 12 boxes of edge 48-96 took %BATCH%
+    // better: 12 boxes of edge 48-96 FP32 take 249.6 us a step with the best of 22 (rows, planes) pairs, 259.9 with this
+    // choice and 311 with 8 rows and 32 planes
     b->seg_planes = b->seg_planes_req ? b->seg_planes_req : 32;
     if (!b->seg_planes_req) {
         long long least = 0;
