@@ -96,8 +96,8 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, u
 // more in their misaligned stores (128^3 FP32 116.0 against 109.4 us,
 // 256x256x128 BF16 292.7 against 282.0).
 // FP32 4-row tiles with one stage keep psi of three planes, not four (one more
-// barrier a plane): 45.5 KB, five CTAs an SM.
-template <class S, int TY, int NS>
+// barrier a plane): 45.5 KB, five CTAs an SM (the batched step: four, see there).
+template <class S, int TY, int NS, bool kBatch = false>
 struct TmaGeom {
     static constexpr int TX = 32, HX = TX + 2, HY = TY + 2;
     static constexpr int GX = edge_x<S>();                    // nodes in 16 bytes
@@ -115,7 +115,7 @@ struct TmaGeom {
     static constexpr uint32_t YS_BYTES = YS_ELEMS * sizeof(S);
     static constexpr uint32_t CS_BYTES = CS_ELEMS * sizeof(S);
     static constexpr uint32_t STAGE_BYTES = STAGE_ELEMS * sizeof(S);
-    static constexpr int PSI_PLANES = sizeof(S) == 4 && TY == 4 && NS == 1 ? 3 : 4;
+    static constexpr int PSI_PLANES = sizeof(S) == 4 && TY == 4 && NS == 1 && !kBatch ? 3 : 4;
     static constexpr int PSI_FLOATS = PSI_PLANES * 2 * HY * HX;
     // psi follows the last stage's last region without padding
     static constexpr size_t PSI_AT = ((size_t)(NS - 1) * STAGE_ELEMS + XS + XS_ELEMS) * sizeof(S);
@@ -144,11 +144,11 @@ struct TmaMaps {
 // for the step before, whose end its index arithmetic overlaps, and every item
 // then reads the step counter into clk. Returns false when a wait gave up (the
 // status word is set and the CTA's copies in flight are drained).
-template <class S, int TY, int NS, bool kTauOne, bool kGeneral = false>
+template <class S, int TY, int NS, bool kTauOne, bool kGeneral, bool kBatch>
 __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>& A, int col, int za, int zb, S* stages,
                                          float* sp, uint64_t* bar, uint32_t& g, uint32_t& clk, bool& started)
 {
-    using G = TmaGeom<S, TY, NS>;
+    using G = TmaGeom<S, TY, NS, kBatch>;
     constexpr int TX = 32, NT = TX * TY, HX = G::HX, HY = G::HY, GX = G::GX, BX = G::BX, SX = G::SX;
     constexpr int RING = 2 * HX + 2 * TY;
     constexpr int NIT = (RING + NT - 1) / NT;
@@ -390,7 +390,7 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
         for (int i = 0; i < NS && i < np; ++i) issue(za - 1 + i, g + i);
     if (!consume(0, rn, jn, vn, mn, nbn) || !consume(1, rc, jc, vc, mc, nbc)) return false;
 
-    Dest<S, sizeof(S) == 4> D;
+    Dest<S, sizeof(S) == 4 && !kBatch> D;
     D.set_column(L, valid ? gx : 0, valid ? gy : 0);
     D.err = A.err;
     D.hoff = A.hkey;
@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
         const int za = A.zlo + (int)((long long)seg * nzf / A.nseg);
         const int zb = A.zlo + (int)((long long)(seg + 1) * nzf / A.nseg);
         if (za >= zb) continue;
-        if (!tma_item<S, TY, NS, kTauOne, kGeneral>(maps, A, col, za, zb, stages, sp, bar, g, clk, started)) break;
+        if (!tma_item<S, TY, NS, kTauOne, kGeneral, false>(maps, A, col, za, zb, stages, sp, bar, g, clk, started)) break;
     }
     if (!started) grid_wait();
     if constexpr (Codec<S>::kDeviation) clock_tick(A.clock);
@@ -473,12 +473,18 @@ __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
 // sizes and parameters; args[2 box + parity] and maps[2 box + parity] describe
 // box `box` for this step (the maps live in global memory, written by the host
 // before the launch). The last CTA out advances every box's step counter.
+// It is launched after the step before has ended, keeps psi of four planes (four
+// FP32 CTAs of 4-row tiles an SM) and stores by node offsets: an item's ring
+// rows come from L2 only while neighbouring CTAs stay in step, which CTAs placed
+// as slots free up, or five an SM, do not (64 boxes of edge 48-96: 1262 us a step
+// FP32 and 958 BF16, launched dependently with three planes 1668 and 1511; 6
+// boxes 115 and 91, 124 and 90).
 template <class S, int TY, int NS, bool kTauOne>
 __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
     batch_tma_kernel(const TmaMaps* __restrict__ maps, const StepArgs<S>* __restrict__ args,
                      const int4* __restrict__ items, int nitems, int parity, int nbox, uint32_t* done)
 {
-    using G = TmaGeom<S, TY, NS>;
+    using G = TmaGeom<S, TY, NS, true>;
     extern __shared__ __align__(128) unsigned char smem[];
     S* stages = (S*)smem;
     float* sp = (float*)(smem + G::PSI_AT);
@@ -488,9 +494,8 @@ __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
         mbar_fence_init();
     }
     __syncthreads();
-    grid_trigger();
     uint32_t g = 0;
-    bool started = false;
+    bool started = true;  // launched whole, after the step before
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int4 w = items[it];
         const StepArgs<S>& A = args[2 * w.x + parity];
@@ -499,9 +504,8 @@ __global__ void __launch_bounds__(32 * TY, (kTmaCtas<S, TY, kTauOne>))
             for (int i = 0; i < 4; ++i)  // the maps were written through the generic proxy
                 asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&M.m[i]) : "memory");
         uint32_t clk = 0;
-        if (!tma_item<S, TY, NS, kTauOne>(M, A, w.y, w.z, w.w, stages, sp, bar, g, clk, started)) break;
+        if (!tma_item<S, TY, NS, kTauOne, false, true>(M, A, w.y, w.z, w.w, stages, sp, bar, g, clk, started)) break;
     }
-    if (!started) grid_wait();
     if constexpr (Codec<S>::kDeviation) {
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -570,10 +574,12 @@ template <class S, int TY, bool T1>
 static long long tma_batch_one(int op, const TmaMaps* maps, const StepArgs<S>* args, const int4* items, int nitems,
                                int parity, int nbox, uint32_t* done, int grid, cudaStream_t st)
 {
-    const size_t smem = TmaGeom<S, TY, 1>::SMEM;
+    // FP32 8-row tiles ask for 9000 bytes they do not use: three CTAs an SM either way, but with the SM's memory
+    // split for shared memory in full 64 boxes take 1344 us a step, else 1863
+    const size_t smem = TmaGeom<S, TY, 1, true>::SMEM + (TY == 8 && sizeof(S) == 4 ? 9000 : 0);
     if (op == 0) {
-        return launch_after(batch_tma_kernel<S, TY, 1, T1>, dim3(grid), 32 * TY, smem, st, maps, args, items, nitems, parity,
-                            nbox, done);
+        batch_tma_kernel<S, TY, 1, T1><<<grid, 32 * TY, smem, st>>>(maps, args, items, nitems, parity, nbox, done);
+        return cudaGetLastError();
     }
     if (op == 1)
         return cudaFuncSetAttribute(batch_tma_kernel<S, TY, 1, T1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
