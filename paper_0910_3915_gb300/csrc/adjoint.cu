@@ -44,12 +44,13 @@ __device__ __forceinline__ float lane(const float2& v, int a) { return a ? v.y :
 __device__ __forceinline__ float add_c(float s, int c, float v) { return c == 0 ? s : (c > 0 ? s + v : s - v); }
 
 // Forward rho, j, psi of the stored state (lattice layout L), one thread per
-// node, both components of a velocity in one load. Bound by the read of the
+// node, both components of a velocity in one load: a plain one, since the step
+// that writes f may still run when this kernel starts. Bound by the read of the
 // populations (152 bytes a node, from L2 when it follows the step that wrote
 // them): 8.5 us at 64^3 FP32 (cold caches), 11.4 with a grid-stride grid of 512
 // blocks and one component at a time.
 template <class S>
-__global__ void __launch_bounds__(kAdjThreads) adj_forward_kernel(Layout L, KParams P, const S* __restrict__ f, AdjState A)
+__global__ void __launch_bounds__(kAdjThreads) adj_forward_kernel(Layout L, KParams P, const S* f, AdjState A)
 {
     grid_trigger();
     const int N = L.nx * L.ny * L.nz;
@@ -63,7 +64,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_forward_kernel(Layout L, KPar
     if (!solid) {
         const long long off = L.off(x, y, z);
 #pragma unroll
-        for (int k = 0; k < Q; ++k) w[k] = Codec<S>::load2(f + L.at(0, k, off));
+        for (int k = 0; k < Q; ++k) w[k] = Codec<S>::val2(*(const typename Codec<S>::Pair*)(f + L.at(0, k, off)));
     }
     float r[2], j[2][3], psi[2];
 #pragma unroll
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_forward_kernel(Layout L, KPar
 // the blocks' rows after every step before (32 us).
 template <bool kTauOne>
 __global__ void __launch_bounds__(kAdjThreads)
-    adj_local_kernel(AdjArgs G, AdjState A, AdjE En, const float* __restrict__ Mn, AdjE Ec, float* __restrict__ Mc,
+    adj_local_kernel(AdjArgs G, AdjState A, AdjE En, const float* Mn, AdjE Ec, float* Mc,
                      AdjV W, double* __restrict__ part)
 {
     const int nx = G.nx, ny = G.ny, nz = G.nz;

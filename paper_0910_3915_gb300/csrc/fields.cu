@@ -435,7 +435,7 @@ __device__ __noinline__ void add_crossing(float2* acc, int stride, int x, int y,
 // A thread's sums wait in shared memory, and a warp reduces a value only if one
 // of its lanes holds a contribution to it. The last block to finish adds the
 // blocks' rows, in order, and writes the 19 values lb_contact_angle works with.
-__global__ void __launch_bounds__(kAngleThreads, 3) angle_kernel(FieldArgs F, AngleArgs A, const float* __restrict__ P,
+__global__ void __launch_bounds__(kAngleThreads, 3) angle_kernel(FieldArgs F, AngleArgs A, const float* P,
                                                               float2* __restrict__ part, unsigned int* __restrict__ ticket,
                                                               double* __restrict__ out)
 {
@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(kAngleThreads, 3) angle_kernel(FieldArgs F, An
     const int rows = ny * nz;
     for (int r = blockIdx.x + warp * gridDim.x; r < rows; r += kWarps * gridDim.x) {
         const int z = r / ny, y = r - z * ny;
-        const float* __restrict__ R = P + (size_t)r * nx;
+        const float* R = P + (size_t)r * nx;
         const size_t up_y = y + 1 < ny ? nx : 0, up_z = z + 1 < nz ? nxy : 0;  // past an edge: the node itself
         // planar walls: the row is all fluid or all wall, and so is the one above it
         const bool wall = !F.general && (z == 0 || z == nz - 1);

@@ -277,7 +277,9 @@ __device__ __forceinline__ void clock_tick(uint32_t* clk)
 // while the kernel before it in its stream still runs, once all of that one's
 // CTAs have called grid_trigger (or ended). Everything before its grid_wait
 // must touch nothing the earlier kernels write; grid_wait returns when they
-// have ended and their writes are visible.
+// have ended and their writes are visible. Memory that they write changes while
+// the dependent kernel is resident, so it reads it by plain loads: no __ldg, and
+// no const __restrict__ pointer, which lets the compiler load it as read-only data.
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

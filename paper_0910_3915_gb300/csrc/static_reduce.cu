@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kStaticThreads)
 // The 38 arrays' totals (warp w takes arrays w and w + 32, the ranges in a
 // fixed tree), then {M_r, M_b, Px, Py, Pz, non-finite count, fluid nodes, 0},
 // a warp each (a chain of FP64 additions in one thread took 12 us)
-__global__ void __launch_bounds__(1024) static_finish_kernel(const double* __restrict__ part, int chunks,
+__global__ void __launch_bounds__(1024) static_finish_kernel(const double* part, int chunks,
                                                              double* __restrict__ out)
 {
     __shared__ double tot[2 * Q];
