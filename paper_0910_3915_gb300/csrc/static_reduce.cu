@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(1024) static_finish_kernel(const double* part,
     __syncthreads();
     if (warp >= 8) return;
     double x = 0;
-    int b = 0;
+    long long b = 0;  // 38 counts of up to 67,108,864
     for (int r = lane; r < 2 * Q; r += 32) {
         const int k = r % Q;
         if (warp < 2) x += r / Q == warp ? tot[r] : 0.0;
@@ -177,9 +177,10 @@ __global__ void __launch_bounds__(1024) static_finish_kernel(const double* part,
         else if (warp < 5) x += (warp == 2 ? cx(k) : (warp == 3 ? cy(k) : cz(k))) * tot[r];
         else if (warp == 5) b += num[r];
     }
-    if (warp < 5)
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    b = __reduce_add_sync(0xffffffffu, b);
+    for (int o = 16; o > 0; o >>= 1) {
+        if (warp < 5) x += __shfl_down_sync(0xffffffffu, x, o);
+        else b += __shfl_down_sync(0xffffffffu, b, o);
+    }
     if (lane == 0) out[warp] = warp < 5 ? x : (warp == 5 ? (double)b : (warp == 6 ? (double)num[2 * Q] : 0.0));
 }
 

@@ -72,3 +72,27 @@ def test_sums_of_values_far_apart():
         for g, w in zip(got[:5], want):
             assert abs(Fraction(float(g)) - w) <= n.size * Fraction(2) ** -53 * size + Fraction(2) ** -1070
         assert got[5] == 0 and got[6] == nx * ny * nz
+
+
+@pytest.mark.parametrize("masked", [False, True])
+def test_a_large_field_without_finite_values_is_counted(masked):
+    """The largest field there may be, every value NaN (a run that blew up): 38 values a fluid node, above 2^31 of them."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0910_3915_gb300 import lbsc
+    nx, ny, nz = 512, 512, 256
+    if torch.cuda.mem_get_info()[0] < 24e9:
+        pytest.skip("the field takes 20.4 GB")
+    n = torch.full((2, 19, nz, ny, nx), float("nan"), dtype=torch.float64, device="cuda")
+    solid = torch.zeros((nz, ny, nx), dtype=torch.uint8, device="cuda")
+    if masked:
+        solid[0] = solid[-1] = 1
+    out = torch.zeros(8, dtype=torch.float64, device="cuda")
+    lbsc.conservation_static(n.data_ptr(), solid.data_ptr() if masked else None, nx, ny, nz, out.data_ptr())
+    got = out.cpu().numpy()
+    fluid = nx * ny * (nz - 2 * masked)
+    assert got[5] == 38 * fluid and got[6] == fluid
+    assert np.isnan(got[:5]).all()
+    del n, solid
+    torch.cuda.empty_cache()
