@@ -1772,9 +1772,9 @@ extern "C" int lb_step_backward(lb_ctx* c, int nsteps, int ckpt_every, int obser
     const int slen = nsteps < ckpt_every ? nsteps : ckpt_every;  // steps of the longest segment
     const int blocks = (int)((N + kAdjThreads - 1) / kAdjThreads);
     // Device memory of the call: the states at the starts of all segments but
-    // the last, two states the recompute steps between, the forward fields
-    // (10 values a node) of one segment's states and of the final one, and
-    // the adjoint's fields
+    // the last and two states their recompute steps between (the last segment
+    // steps in the lattice's own buffers), the forward fields (10 values a
+    // node) of one segment's states and of the final one, and the adjoint's fields
     AdjScratch M;
     char* ck = nullptr;
     char* store = nullptr;
@@ -1783,7 +1783,7 @@ extern "C" int lb_step_backward(lb_ctx* c, int nsteps, int ckpt_every, int obser
     float* mom = nullptr;
     double* dsc = nullptr;
     if (nseg > 1) LB_CUDA(c, M.alloc((void**)&ck, sb * (size_t)(nseg - 1)));
-    if (nseg > 0) LB_CUDA(c, M.alloc((void**)&store, 2 * sb));
+    if (nseg > 1) LB_CUDA(c, M.alloc((void**)&store, 2 * sb));
     LB_CUDA(c, M.alloc((void**)&fields, sizeof(float) * kAdjStateVals * N * (size_t)(slen + 1)));
     LB_CUDA(c, M.alloc((void**)&adj, sizeof(float) * (2 * kAdjEVals + kAdjVVals) * N));
     if (!t1) LB_CUDA(c, M.alloc((void**)&mom, sizeof(float) * 2 * 2 * Q * N));
@@ -1816,7 +1816,7 @@ extern "C" int lb_step_backward(lb_ctx* c, int nsteps, int ckpt_every, int obser
     }
     const int ns = schedule(c).ns;
     CUtensorMap maps[2][4];
-    if (ns && nseg > 0)
+    if (ns && nseg > 1)
         for (int b = 0; b < 2; ++b) {
             const int rc = encode_maps(c, store + sb * (size_t)b, schedule(c).ty, maps[b]);
             if (rc != LB_OK) return rc;
@@ -1831,13 +1831,12 @@ extern "C" int lb_step_backward(lb_ctx* c, int nsteps, int ckpt_every, int obser
     };
     auto fields_of = [&](int i) { return adj_state(fields + kAdjStateVals * N * (size_t)i, N); };
     // the forward fields of a segment's `len` states, stepping on from store[0]
-    // (the fields pass reads the state while it is in L2); with `end` also the
-    // step that ends the segment
-    auto recompute = [&](int len, bool end, cudaStream_t s2) -> cudaError_t {
+    // (the fields pass reads the state while it is in L2)
+    auto recompute = [&](int len, cudaStream_t s2) -> cudaError_t {
         cudaError_t e = cudaSuccess;
         for (int i = 0; i < len && e == cudaSuccess; ++i) {
             e = adj_forward(c, store + sb * (size_t)(i & 1), fields_of(i), s2);
-            if (e == cudaSuccess && (end || i + 1 < len)) e = step_of(i & 1, s2);
+            if (e == cudaSuccess && i + 1 < len) e = step_of(i & 1, s2);
         }
         return e;
     };
@@ -1862,14 +1861,14 @@ extern "C" int lb_step_backward(lb_ctx* c, int nsteps, int ckpt_every, int obser
     // about as much as launching it twice).
     auto segment = [&](int len, int en) -> cudaError_t {
         if (nseg < 5) {
-            cudaError_t e = recompute(len, false, st);
+            cudaError_t e = recompute(len, st);
             return e == cudaSuccess ? reverse(len, en, st) : e;
         }
         if (!graphs.g[en]) {
             cudaGraph_t gr = nullptr;
             cudaError_t e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
             if (e != cudaSuccess) return e;
-            cudaError_t e1 = recompute(len, false, c->cap);
+            cudaError_t e1 = recompute(len, c->cap);
             if (e1 == cudaSuccess) e1 = reverse(len, en, c->cap);
             e = cudaStreamEndCapture(c->cap, &gr);
             if (e1 != cudaSuccess) e = e1;
@@ -1889,14 +1888,14 @@ extern "C" int lb_step_backward(lb_ctx* c, int nsteps, int ckpt_every, int obser
         const int rc = lb_step(c, ckpt_every);
         if (rc != LB_OK) return rc;
     }
-    // the last segment steps with its forward fields kept, so it needs no recompute
+    // the last segment steps on in the lattice's own buffers (which keep what no
+    // step writes, as lb_step leaves them) with its forward fields kept, so it
+    // needs no recompute
     const int llen = nseg > 0 ? nsteps - (nseg - 1) * ckpt_every : 0;
-    if (nseg > 0) {
-        LB_CUDA(c, cudaMemcpyAsync(store, c->f[c->cur], sb, cudaMemcpyDeviceToDevice, st));
-        LB_CUDA(c, recompute(llen, true, st));
-        c->cur ^= llen & 1;  // as lb_step leaves it
-        c->steps += llen;
-        LB_CUDA(c, cudaMemcpyAsync(c->f[c->cur], store + sb * (size_t)(llen & 1), sb, cudaMemcpyDeviceToDevice, st));
+    for (int i = 0; i < llen; ++i) {
+        LB_CUDA(c, adj_forward(c, c->f[c->cur], fields_of(i), st));
+        LB_CUDA(c, launch_steps(c, 1, c->cur, st));
+        c->steps += 1;
     }
     // observable of the final state and lambda(T) = dJ/dn(T)
     const double eps = 0.05;
