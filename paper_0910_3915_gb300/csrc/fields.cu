@@ -360,6 +360,27 @@ __device__ __forceinline__ Two over(float p, const AngleArgs& A)
     return norm2(Two{s.h, __fsub_rn(s.l, A.ll)});
 }
 
+// Pairs serve where a difference of phi lies well inside FP32's range: not for
+// infinities, NaN or values whose differences overflow, nor where the low part
+// of a product would fall below the least FP32 number. Those nodes, rare, are
+// taken in FP64 out of line.
+__device__ __forceinline__ bool pairs_serve(float size) { return size > 1e-20f && size < 1e37f; }
+__device__ __forceinline__ Two two_f64(double v)
+{
+    const float h = (float)v;
+    return Two{h, isfinite(h) ? (float)(v - (double)h) : 0.f};
+}
+
+// plane_length in FP64
+__device__ __noinline__ Two plane_length_f64(float p0, float p0up, float p1, float p1up, const AngleArgs& A)
+{
+    const double a0 = (1 - A.fz) * ((double)p0 - A.level) + A.fz * ((double)p0up - A.level);
+    const double a1 = (1 - A.fz) * ((double)p1 - A.level) + A.fz * ((double)p1up - A.level);
+    if (a0 > 0 && a1 > 0) return two(1.0f);
+    if (a0 <= 0 && a1 <= 0) return two(0.0f);
+    return two_f64(a0 > 0 ? a0 / (a0 - a1) : a1 / (a1 - a0));
+}
+
 // Positive length along x, from a node to its +x neighbour, of the linear
 // interpolant of phi - level on the reference plane z0 + fz (p: phi at the
 // node, above it, at the +x neighbour and above that).
@@ -368,9 +389,35 @@ __device__ __forceinline__ Two plane_length(float p0, float p0up, float p1, floa
     const Two f{A.fzh, A.fzl}, g = norm2(two(1.0f) - f);
     const Two a0 = norm2(mul22(g, over(p0, A)) + mul22(f, over(p0up, A)));
     const Two a1 = norm2(mul22(g, over(p1, A)) + mul22(f, over(p1up, A)));
+    if (!pairs_serve(fabsf(a0.h) + fabsf(a1.h))) return plane_length_f64(p0, p0up, p1, p1up, A);
     if (a0.h > 0 && a1.h > 0) return two(1.0f);
     if (a0.h <= 0 && a1.h <= 0) return two(0.0f);
     return a0.h > 0 ? div22(a0, norm2(a0 - a1)) : div22(a1, norm2(a1 - a0));
+}
+
+__device__ __forceinline__ void add_to(float2* acc, Two v)
+{
+    const float2 o = *acc;
+    const Two s = norm2(Two{o.x, o.y} + v);
+    *acc = make_float2(s.h, s.l);
+}
+
+// add_crossing in FP64; a crossing that is not a number goes into the sums
+__device__ __noinline__ void add_crossing_f64(float2* acc, int stride, int x, int y, int z, int d, float p0, float p1,
+                                              const AngleArgs& A)
+{
+    const double q0 = (double)p0 - A.level, q1 = (double)p1 - A.level, t = q0 / (q0 - q1);
+    const double p[3] = {x + t * (d == 0), y + t * (d == 1), z + t * (d == 2)};
+    if (d == 2 && q0 > 0) {
+        const float2 top = acc[0];
+        const Two v = two_f64(z + t);
+        if (less2(Two{top.x, top.y}, v)) acc[0] = make_float2(v.h, v.l);
+    }
+    if (p[2] < A.zref) return;
+    const double rr = p[0] * p[0] + p[1] * p[1] + p[2] * p[2];
+    const double v[14] = {1.0,         p[0] * p[0], p[0] * p[1], p[0] * p[2], p[0],      p[1] * p[1], p[1] * p[2],
+                          p[1],        p[2] * p[2], p[2],        p[0] * rr,   p[1] * rr, p[2] * rr,   rr};
+    for (int i = 0; i < 14; ++i) add_to(&acc[(i + 2) * stride], two_f64(v[i]));
 }
 
 // An interface crossing between node (x, y, z) (phi = p0) and its neighbour
@@ -382,9 +429,9 @@ __device__ __forceinline__ Two plane_length(float p0, float p0up, float p1, floa
 __device__ __noinline__ void add_crossing(float2* acc, int stride, int x, int y, int z, int d, float p0, float p1,
                                           const AngleArgs& A)
 {
-    const Two q0 = over(p0, A);
-    Two t = div22(q0, norm2(two_sum(p0, -p1)));
-    if (isinf(p1) && isfinite(p0)) t = two(0.f);  // q0 over an infinity
+    const Two gap = norm2(two_sum(p0, -p1));
+    if (!pairs_serve(fabsf(gap.h))) return add_crossing_f64(acc, stride, x, y, z, d, p0, p1, A);
+    const Two t = div22(over(p0, A), gap);
     const Two c[3] = {two_int(x), two_int(y), two_int(z)};
     Two p[3];
 #pragma unroll
@@ -394,11 +441,7 @@ __device__ __noinline__ void add_crossing(float2* acc, int stride, int x, int y,
         if (less2(Two{top.x, top.y}, p[2])) acc[0] = make_float2(p[2].h, p[2].l);
     }
     if (less2(p[2], Two{A.zh, A.zl})) return;
-    auto add = [&](int i, Two v) {
-        const float2 o = acc[i * stride];
-        const Two s = norm2(Two{o.x, o.y} + v);
-        acc[i * stride] = make_float2(s.h, s.l);
-    };
+    auto add = [&](int i, Two v) { add_to(&acc[i * stride], v); };
     const Two xx = norm2(mul22(p[0], p[0])), yy = norm2(mul22(p[1], p[1])), zz = norm2(mul22(p[2], p[2]));
     const Two rr = norm2((xx + yy) + zz);
     add(2, two(1.0f));
@@ -1109,6 +1152,9 @@ cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, doub
     split(zref, A.zh, A.zl);
     const double z0 = std::floor(zref);
     split(zref - z0, A.fzh, A.fzl);
+    A.level = level;
+    A.zref = zref;
+    A.fz = zref - z0;
     A.z0 = z0 < (double)F.L.nz ? (int)z0 : F.L.nz;
     const int rows = F.L.ny * F.L.nz, warps = kAngleThreads / 32;
     const int blocks = (rows + warps - 1) / warps < kAngleBlocks ? (rows + warps - 1) / warps : kAngleBlocks;

@@ -18,10 +18,12 @@ constexpr int kPartVals = 19;           // doubles a row
 
 // The contact angle's level (lh + ll) and the least FP32 number above it, the
 // reference height zref (zh + zl), its plane z0 (nz where that lies outside)
-// and fraction there, in pairs of FP32 numbers.
+// and fraction there, in pairs of FP32 numbers, and level, zref and the
+// fraction in FP64 for the nodes that pairs do not serve.
 struct AngleArgs {
     float lh, ll, least, zh, zl, fzh, fzl;
     int z0;
+    double level, zref, fz;
 };
 
 // Geometry and parameters for the non-step kernels.

@@ -727,3 +727,39 @@ def test_readback_in_chunks_equals_the_populations(lbsc, dims):
         assert np.all(r[[0, -1]] == 0) and np.all(np.abs(u) < 1e-6) and cons[6] == nx * ny * (nz - 2)
         r1, b1, none, _ = lat.moments()
         assert none is None and np.array_equal(r1, r) and np.array_equal(b1, b)
+
+
+@pytest.mark.parametrize("offset", [1.0, 2.25])
+@pytest.mark.parametrize("what", ["inf", "-inf", "nan", "huge", "tiny", "level above", "level below"])
+def test_contact_angle_sums_outside_fp32_pairs(lbsc, what, offset):
+    """Infinities and NaN at the reference plane, the apex and between, values whose differences overflow FP32 or whose
+    products fall below its least number, levels beyond its range: the oracle's construction on the same phi in FP64.
+    Lengths from sums of at most nx ny terms of 44 bits, the sphere's values through a 4 x 4 solve: 1e-11 and 1e-7."""
+    nx, ny, nz = 37, 9, 12
+    z, y, x = np.meshgrid(np.arange(nz), np.arange(ny), np.arange(nx), indexing="ij")
+    phi = np.sin(0.7 * x) * np.cos(0.4 * y) * np.sin(0.5 * z + 0.3)
+    rng = np.random.Generator(np.random.PCG64(3))
+    phi = (phi + rng.uniform(-0.2, 0.2, size=phi.shape)).astype(np.float32).astype(np.float64)
+    level = 0.0
+    spots = [(int(0.5 + offset), 4, 5), (int(0.5 + offset), 4, 6), (int(0.5 + offset) + 1, 2, 20), (8, 3, 36), (5, 8, 0)]
+    if what in ("inf", "-inf", "nan"):
+        for s in spots:
+            phi[s] = float(what)
+    elif what == "huge":
+        phi = (phi * 2.5e38).astype(np.float32).astype(np.float64)
+    elif what == "tiny":
+        phi = (phi * 1e-36).astype(np.float32).astype(np.float64)
+    else:
+        level = 1e300 if what == "level above" else -1e300
+    solid = W.wall_mask(nx, ny, nz)
+    phi[solid != 0] = 0.0
+    n = np.zeros((2, 19, nz, ny, nx))
+    n[0, 0] = phi
+    lat = lbsc.Lattice(np.full(phi.shape, 0.4), np.full(phi.shape, 0.3)).set_populations(n)
+    d = lat.contact_angle(offset, level=level)
+    with np.errstate(all="ignore"):
+        o = oracle.contact_angle(phi, 0 * n[1, 0], solid, offset, level)
+    assert d["n_points"] == o["n_points"] and d["ok"] == o["ok"]
+    for k, tol in (("h", 1e-11), ("base_ref", 1e-11), ("theta_fit_deg", 1e-7), ("xc", 1e-7), ("yc", 1e-7), ("zc", 1e-7), ("r_fit", 1e-7)):
+        assert np.isnan(d[k]) == np.isnan(o[k]), (k, d[k], o[k])
+        assert np.isnan(o[k]) or abs(d[k] - o[k]) <= tol * max(1.0, abs(o[k])), (k, d[k], o[k])
