@@ -742,8 +742,11 @@ __device__ __noinline__ void node_pressure_f64(const FieldArgs& F, const S* __re
     for (int c = 0; c < 6; ++c) P[c] += h * I[c];
 }
 
+// values that a plane's sums may hold as FP32 pairs: sums of fewer than 2^31 stay below FP32's largest number
+constexpr float kSumLimit = 1e28f;
+
 // the tensor at the fluid node (x, y, z), normalised; false where a component
-// is not finite (the caller then takes node_pressure_f64)
+// is not finite or too large for the sums (the caller then takes node_pressure_f64)
 template <class S>
 __device__ __forceinline__ bool node_pressure(const FieldArgs& F, const S* __restrict__ f, const Scratch& W, int x, int y,
                                               int z, Two (&P)[6])
@@ -810,7 +813,7 @@ __device__ __forceinline__ bool node_pressure(const FieldArgs& F, const S* __res
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
         P[c] = norm2(P[c] + mul2f(norm2(I[c]), h));
-        finite = finite && isfinite(P[c].h) && isfinite(P[c].l);
+        finite = finite && fabsf(P[c].h) < kSumLimit;
     }
     return finite;
 }
@@ -850,7 +853,7 @@ __global__ void __launch_bounds__(kPressThreads, 5) pressure_plane_kernel(FieldA
     const int lo = (int)((long long)blockIdx.y * nxy / split), hi = (int)((long long)(blockIdx.y + 1) * nxy / split);
     Two sum[7];
     for (int v = 0; v < 7; ++v) sum[v] = two(0.f);
-    double odd[6] = {0, 0, 0, 0, 0, 0};  // nodes taken in FP64
+    double odd[7] = {0, 0, 0, 0, 0, 0, 0};  // nodes taken in FP64
     int count = 0;
     bool odd_nodes = false;
     for (int c = lo + threadIdx.x; c < hi; c += kPressThreads) {
@@ -867,11 +870,17 @@ __global__ void __launch_bounds__(kPressThreads, 5) pressure_plane_kernel(FieldA
             for (int v = 0; v < 6; ++v) odd[v] += D[v];
             odd_nodes = true;
         }
-        sum[6] = norm2(sum[6] + two_sum(W.rho[0][i], -W.rho[1][i]));
+        const Two phi = two_sum(W.rho[0][i], -W.rho[1][i]);
+        if (fabsf(phi.h) < kSumLimit) {
+            sum[6] = norm2(sum[6] + phi);
+        } else {
+            odd[6] += (double)W.rho[0][i] - (double)W.rho[1][i];
+            odd_nodes = true;
+        }
         ++count;
     }
     __shared__ float2 sh[kPressThreads / 32][7];
-    __shared__ double sodd[kPressThreads / 32][6];
+    __shared__ double sodd[kPressThreads / 32][7];
     __shared__ int sn[kPressThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -888,7 +897,7 @@ __global__ void __launch_bounds__(kPressThreads, 5) pressure_plane_kernel(FieldA
     if (lane == 0) sn[warp] = count;
     const bool any_odd = __syncthreads_or(odd_nodes);
     if (any_odd) {  // uniform
-        for (int v = 0; v < 6; ++v) {
+        for (int v = 0; v < 7; ++v) {
             const double t = warp_sum(odd[v]);
             if (lane == 0) sodd[warp][v] = t;
         }
@@ -900,7 +909,7 @@ __global__ void __launch_bounds__(kPressThreads, 5) pressure_plane_kernel(FieldA
         for (int w = 0; w < kPressThreads / 32; ++w) {
             if (v < 7) t += (double)sh[w][v].x + (double)sh[w][v].y;
             else t += (double)sn[w];
-            if (any_odd && v < 6) t += sodd[w][v];
+            if (any_odd && v < 7) t += sodd[w][v];
         }
         out[((size_t)z * split + blockIdx.y) * 8 + v] = t;
     }

@@ -270,3 +270,26 @@ def test_pressure_of_a_state_with_an_infinity(lbsc):
     assert np.isfinite(P[:, ~there]).all() and np.array_equal(P[:, far], P0[:, far])
     keep = [z for z in range(nz) if z not in (4, 5, 6)]
     assert not np.isfinite(prof[5, :6]).any() and np.array_equal(prof[keep], prof0[keep])
+
+
+def test_profile_of_infinite_and_huge_densities(lbsc):
+    """Plane means of phi where a density is infinite, or where two sum past FP32's range: what FP64 sums of the same FP32
+    densities give."""
+    nx, ny, nz = 33, 5, 6
+    n = np.zeros((2, 19, nz, ny, nx))
+    n[:, 0] = 0.25
+    n[0, 0, 2, 1, 3] = np.inf
+    n[1, 0, 3, 4, 32] = np.inf
+    n[0, 0, 4, 0, :20] = 2.0 ** 127  # 20 of them: above FP32's largest number, far below FP64's
+    lat = lbsc.Lattice(np.full((nz, ny, nx), 0.4), np.full((nz, ny, nx), 0.3)).set_populations(n)
+    prof, _ = lat.pressure_profile()
+    phi = n[0, 0] - n[1, 0]
+    with np.errstate(invalid="ignore"):
+        want = phi.reshape(nz, -1).sum(1) / (nx * ny)
+    assert want[2] == np.inf and want[3] == -np.inf and np.isfinite(want[4])
+    assert np.array_equal(prof[1:-1, 7], np.full(nz - 2, nx * ny))
+    assert np.array_equal(np.isfinite(prof[1:-1, 6]), np.isfinite(want[1:-1]))
+    assert prof[2, 6] == np.inf and prof[3, 6] == -np.inf
+    assert abs(prof[4, 6] - want[4]) <= 1e-12 * want[4] and prof[1, 6] == want[1]
+    # xx of the nodes at rest: n c c vanishes, the interaction of finite psi is finite
+    assert np.isfinite(prof[4, :6]).all()
