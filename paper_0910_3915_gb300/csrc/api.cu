@@ -507,6 +507,8 @@ static int init_common(lb_ctx** out, int nx, int ny, int nz, int precision, cons
     // reduction area: conservation accumulators [32, 40) and ticket [40], contact-angle ticket [41], status word [48],
     // step counter [50]
     e = cudaMemsetAsync(c->red, 0, 64 * sizeof(double), c->stream);
+    // the buffer the first step writes: no step writes its solid nodes, which lb_get_populations and lb_save read
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->f[1], 0, p.f, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->dev_err, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->clock, 0, 2 * sizeof(uint32_t), c->stream);
     if (e != cudaSuccess) return bail(LB_ERR_CUDA, std::string("lb_init: ") + cudaGetErrorString(e));

@@ -4,6 +4,7 @@ Bar: per-node relative density error <= 1e-5 after 100 FP32 steps; contact
 angle within 0.5 deg at steady state. Inputs are seeded droplet-on-wall
 lattices from paper_0910_3915_gb300.workloads, identical on both sides.
 """
+import ctypes
 import math
 
 import numpy as np
@@ -763,3 +764,27 @@ def test_contact_angle_sums_outside_fp32_pairs(lbsc, what, offset):
     for k, tol in (("h", 1e-11), ("base_ref", 1e-11), ("theta_fit_deg", 1e-7), ("xc", 1e-7), ("yc", 1e-7), ("zc", 1e-7), ("r_fit", 1e-7)):
         assert np.isnan(d[k]) == np.isnan(o[k]), (k, d[k], o[k])
         assert np.isnan(o[k]) or abs(d[k] - o[k]) <= tol * max(1.0, abs(o[k])), (k, d[k], o[k])
+
+
+@pytest.mark.parametrize("precision", ["f32", "bf16"])
+def test_solid_nodes_of_both_buffers_are_defined(lbsc, precision):
+    """A lattice in memory that held something else: after an odd number of steps (the second buffer) the solid nodes'
+    populations do not depend on what that was."""
+    torch = pytest.importorskip("torch")
+    nx, ny, nz = 35, 9, 7
+    rr, rb = W.droplet_fields(nx, ny, nz, 4.0, seed=2)
+    need = ctypes.c_size_t()
+    assert lbsc.load().lb_required_bytes(nx, ny, nz, lbsc.PRECISIONS[precision], ctypes.byref(need)) == 0
+    out = []
+    for fill in (0x00, 0x3C):
+        torch.cuda.empty_cache()
+        t = torch.full((need.value + 256,), fill, dtype=torch.uint8, device="cuda")
+        at = t.data_ptr()
+        del t
+        lat = lbsc.Lattice(rr, rb, precision, torch_memory=True)
+        assert lat._buf.data_ptr() == at  # the caching allocator hands the same block out again
+        lat.set_params(**CONTACT)
+        out.append([lat.step(1).populations() for _ in range(2)])
+        lat.close()
+        lat._buf = None
+    assert np.array_equal(out[0], out[1])
