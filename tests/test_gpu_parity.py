@@ -788,3 +788,20 @@ def test_solid_nodes_of_both_buffers_are_defined(lbsc, precision):
         lat.close()
         lat._buf = None
     assert np.array_equal(out[0], out[1])
+
+
+def test_readback_waits_alone(lbsc):
+    """moments() behind many queued steps of a lattice large enough for several converting threads: they do not run while
+    the steps do (process CPU time well below two cores for the wait's time)."""
+    import time
+    rr, rb = W.droplet_fields(128, 128, 128, 30.0, seed=0)
+    lat = lbsc.Lattice(rr, rb).set_params(**CONTACT)
+    lat.step(32)
+    lat.moments()
+    lat.sync()
+    cpu, wall = time.process_time(), time.perf_counter()
+    lat.step(4096)  # about 0.4 s
+    lat.moments()
+    cpu, wall = time.process_time() - cpu, time.perf_counter() - wall
+    assert wall > 0.2
+    assert cpu < 2.0 * wall, (cpu, wall)
