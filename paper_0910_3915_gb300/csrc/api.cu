@@ -55,6 +55,7 @@ struct lb_ctx {
     int tile_y_req = 0, y_tiles_req = 0, nseg_req = 0;
     Schedule sched;  // ty = 0: not chosen since the last change
     long long steps = 0;
+    long long values_read = 0;  // by lb_moments
     // CUDA graphs of 2^i steps (i = 0 .. kGraphLevels - 1) for each starting buffer
     static constexpr int kGraphLevels = 5;  // (a sixth, of 32 steps, took half of the 0.44 ms that capturing them takes)
     cudaGraphExec_t graph[2][kGraphLevels] = {};
@@ -852,12 +853,18 @@ namespace {
 constexpr size_t kStageValues = 1 << 20;  // FP32 values of a half
 
 // Staging blocks (two halves of 4 MB) are kept between calls, at most four,
-// and released with the last context.
+// and released with the last context. Pinning one takes 0.3 ms, more than the
+// whole readback of a small field (32^3 0.1 ms, 0.38 with it; 64^3 0.25 and
+// 0.53), and saves 0.05 to 0.1 ms for every 2^20 values. So fields below
+// kStageValues only take a block that is there already until their context has
+// read kStageAfter values, about what the pinning costs, and go through pageable
+// memory before, as all do where there is no pinned memory to be had.
+constexpr long long kStageAfter = 1 << 22;
 struct Staging {
     std::mutex mu;
     std::vector<float*> free;
     int contexts = 0;
-    float* take()
+    float* take(bool make)
     {
         {
             std::lock_guard<std::mutex> lock(mu);
@@ -868,7 +875,9 @@ struct Staging {
             }
         }
         float* p = nullptr;
-        return cudaMallocHost((void**)&p, 2 * kStageValues * sizeof(float)) == cudaSuccess ? p : nullptr;
+        if (!make || cudaMallocHost((void**)&p, 2 * kStageValues * sizeof(float)) == cudaSuccess) return p;
+        cudaGetLastError();  // taken care of: the caller goes on without
+        return nullptr;
     }
     void give(float* p)
     {
@@ -907,9 +916,29 @@ struct Readback {
     double* dst;       // host
 };
 
-// Wait for stream st and fill the host arrays of n fields of N values each.
-cudaError_t read_back(const Readback* f, int n, long long N, cudaStream_t st)
+// read_back through one pageable array, a field at a time
+cudaError_t read_back_pageable(const Readback* f, int n, long long N, cudaStream_t st)
 {
+    float* tmp = new (std::nothrow) float[(size_t)N];
+    if (!tmp) return cudaErrorMemoryAllocation;
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < n && e == cudaSuccess; ++i) {
+        e = cudaMemcpyAsync(tmp, f[i].src, (size_t)N * sizeof(float), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e == cudaSuccess)
+            for (long long v = 0; v < N; ++v) f[i].dst[v] = tmp[v];
+    }
+    delete[] tmp;
+    return e;
+}
+
+// Wait for stream st and fill the host arrays of n fields of N values each,
+// `before` of which the context has read so far.
+cudaError_t read_back(const Readback* f, int n, long long N, cudaStream_t st, long long before)
+{
+    float* stage = staging().take(N >= (long long)kStageValues || before >= kStageAfter);
+    if (!stage) return read_back_pageable(f, n, N, st);
+
     struct Chunk {
         const float* src;
         double* dst;
@@ -919,8 +948,6 @@ cudaError_t read_back(const Readback* f, int n, long long N, cudaStream_t st)
     for (int i = 0; i < n; ++i)
         for (long long o = 0; o < N; o += kStageValues)
             chunks.push_back({f[i].src + o, f[i].dst + o, (size_t)(N - o < (long long)kStageValues ? N - o : kStageValues)});
-    float* stage = staging().take();
-    if (!stage) return cudaErrorMemoryAllocation;
     cudaEvent_t ev = nullptr;
     cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
@@ -1090,7 +1117,8 @@ int lb_moments(lb_ctx* c, double* rho_r, double* rho_b, double* u, double cons[8
     for (int d = 0; u && d < 3; ++d) fields[n++] = {c->W.u[d], u + d * N};
     if (n) LB_CUDA(c, dispatch_fields(c, u != nullptr));
     LB_CUDA(c, dispatch_cons(c));
-    if (n) LB_CUDA(c, read_back(fields, n, N, c->stream));
+    if (n) LB_CUDA(c, read_back(fields, n, N, c->stream, c->values_read));
+    c->values_read += n * N;
     double tmp[8];
     int rc = wait(c);
     if (rc == LB_OK) rc = take_cons(c, tmp);

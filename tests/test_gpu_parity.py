@@ -6,6 +6,9 @@ lattices from paper_0910_3915_gb300.workloads, identical on both sides.
 """
 import ctypes
 import math
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -805,3 +808,34 @@ def test_readback_waits_alone(lbsc):
     cpu, wall = time.process_time() - cpu, time.perf_counter() - wall
     assert wall > 0.2
     assert cpu < 2.0 * wall, (cpu, wall)
+
+
+READ_ONCE = r"""
+import sys, time
+sys.path.insert(0, sys.argv[1])
+import numpy as np
+from paper_0910_3915_gb300 import lbsc, workloads as W
+n = int(sys.argv[2])
+rr, rb = W.droplet_fields(n, n, n, 0.25 * n, seed=0)
+first, second = [], []
+for _ in range(12):
+    with lbsc.Lattice(rr, rb) as lat:
+        lat.step(2).sync()
+        for out in (first, second):
+            t = time.perf_counter()
+            r, b, _, cons = lat.moments()
+            out.append(time.perf_counter() - t)
+        assert abs(r.sum() - cons[0]) < 1e-6 * cons[0]
+print(np.median(first) * 1e6, np.median(second) * 1e6)
+"""
+
+
+@pytest.mark.parametrize("n", [32, 64])
+def test_first_readback_of_a_small_lattice(n):
+    """A program that keeps one lattice at a time and reads it: no staging block is pinned for the first moments() of each
+    (0.25 ms; the whole readback takes 0.1 ms at 32^3 and 0.25 at 64^3). In a process of its own, without other lattices."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", READ_ONCE, root, str(n)], capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-2000:]
+    first = float(out.stdout.split()[0])
+    assert first < {32: 240, 64: 400}[n], out.stdout  # us: half way between 116 and 365, 263 and 533
