@@ -355,8 +355,9 @@ static int tensor_map(lb_ctx* c, int buf, int ty)
     return rc;
 }
 
+// a step from buffer `src` on tiles_y row splits and nseg z segments
 template <class S>
-static StepArgs<S> step_args(lb_ctx* c, int src)
+static StepArgs<S> step_args(const lb_ctx* c, int src, int tiles_y, int nseg)
 {
     StepArgs<S> A;
     A.src = (const S*)c->f[src];
@@ -367,10 +368,10 @@ static StepArgs<S> step_args(lb_ctx* c, int src)
     A.L = c->L;
     A.P = c->kp;
     A.tiles_x = (c->nx + 31) / 32;
-    A.tiles_y = schedule(c).yt;
+    A.tiles_y = tiles_y;
     A.zlo = c->zlo;
     A.zhi = c->zhi;
-    A.nseg = schedule(c).nseg;
+    A.nseg = nseg;
     A.halo = c->halo;
     A.hkey = c->hkey;
     return A;
@@ -380,8 +381,8 @@ static StepArgs<S> step_args(lb_ctx* c, int src)
 template <class S>
 static cudaError_t launch_one_step(lb_ctx* c, int src, cudaStream_t st)
 {
-    const StepArgs<S> A = step_args<S>(c, src);
     const Schedule& d = schedule(c);
+    const StepArgs<S> A = step_args<S>(c, src, d.yt, d.nseg);
     if (d.ns) return (cudaError_t)tma_op<S>(0, c, c->general, d.ty, d.ns, c->tmap[src][tile_index(d.ty)], &A, st);
     return launch_step<S>(A, d.ty, c->general, tau_one(c), st);
 }
@@ -1402,6 +1403,7 @@ struct lb_batch {
     int nitems = 0;
     int tile_y_req = 0, seg_planes_req = 0;  // the caller's choices (0 = automatic)
     int tile_y = 8, seg_planes = 32, ctas_per_sm = 0, grid = 0;
+    int planned_grid = 0, planned_tile_y = 0;  // what the automatic seg_planes was chosen for (0: not chosen)
     int variant = LB_STEP_AUTO;
     bool tma = false;       // the TMA-staged batch kernel runs the steps
     bool tau1 = true;
@@ -1440,12 +1442,12 @@ static int batch_segments(const lb_ctx* c, int planes)
     return nseg < 1 ? 1 : (nseg > nzf ? nzf : nseg);
 }
 
-// the work list for `planes` planes an item, and the planes (two more an item
-// than it updates) of the CTA that has most when `grid` CTAs take it in turns
+// the work list for `planes` planes an item into `items`, or (items NULL) the planes (two more an
+// item than it updates) of the CTA that has most when `grid` CTAs take that list in turns
 static long long batch_items(const lb_batch* b, int planes, int grid, std::vector<int4>* items)
 {
-    std::vector<long long> load((size_t)grid, 0);
-    size_t n = 0;
+    std::vector<long long> load(items ? 0 : (size_t)grid, 0);
+    int at = 0;  // the CTA whose turn it is
     for (int i = 0; i < b->nbox; ++i) {
         const lb_ctx* c = b->box[i];
         const int cols = (c->nx + 31) / 32 * ((c->ny + b->tile_y - 1) / b->tile_y), nzf = c->zhi - c->zlo;
@@ -1453,9 +1455,13 @@ static long long batch_items(const lb_batch* b, int planes, int grid, std::vecto
         for (int s = 0; s < nseg; ++s) {
             const int za = c->zlo + (int)((long long)s * nzf / nseg), zb = c->zlo + (int)((long long)(s + 1) * nzf / nseg);
             if (za >= zb) continue;
-            for (int col = 0; col < cols; ++col, ++n) {
-                load[n % (size_t)grid] += zb - za + 2;
-                if (items) items->push_back(make_int4(i, col, za, zb));
+            for (int col = 0; col < cols; ++col) {
+                if (items) {
+                    items->push_back(make_int4(i, col, za, zb));
+                } else {
+                    load[at] += zb - za + 2;
+                    at = at + 1 < grid ? at + 1 : 0;
+                }
             }
         }
     }
@@ -1476,22 +1482,22 @@ static int batch_build_typed(lb_batch* b)
     // (the shared-memory attribute first: the occupancy of a kernel above 48 KB counts 0 without it)
     const bool want_tma = b->variant != LB_STEP_LDG;
     b->tile_y = b->tile_y_req ? b->tile_y_req : (want_tma && b->prec == LB_F32 ? 4 : 8);
-    b->tma = want_tma &&
-             tma_batch<S>(1, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr) ==
-                 (long long)cudaSuccess &&
-             tma_batch<S>(2, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr) > 0;
-    const int occ = b->ctas_per_sm > 0
-                        ? b->ctas_per_sm
-                        : (b->tma ? (int)tma_batch<S>(2, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0,
-                                                      nullptr, 0, nullptr)
-                                  : batch_occupancy<S>(b->tile_y, b->tau1));
+    auto tma_op = [&](int op) {
+        return tma_batch<S>(op, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr);
+    };
+    const int tma_occ = want_tma && tma_op(1) == (long long)cudaSuccess ? (int)tma_op(2) : 0;
+    b->tma = tma_occ > 0;
+    const int occ = b->ctas_per_sm > 0 ? b->ctas_per_sm : (b->tma ? tma_occ : batch_occupancy<S>(b->tile_y, b->tau1));
     b->grid = b->box[0]->nsm * (occ > 0 ? occ : 1);
     // Planes an item, where the caller leaves them open: those that give the
     // busiest CTA least. Long items repeat fewer planes, short ones share out
     // better: 12 boxes of edge 48-96 FP32 take 222 us a step with this choice, 225 with 16
-    // planes, 246 with 32
-    b->seg_planes = b->seg_planes_req ? b->seg_planes_req : 32;
-    if (!b->seg_planes_req) {
+    // planes, 246 with 32. The boxes, the tile height and the grid decide it, so a change of a
+    // box's parameters keeps the choice
+    if (b->seg_planes_req) {
+        b->seg_planes = b->seg_planes_req;
+        b->planned_grid = 0;
+    } else if (b->planned_grid != b->grid || b->planned_tile_y != b->tile_y) {
         long long least = 0;
         for (int planes : {64, 48, 32, 24, 20, 16, 12, 10, 8, 6, 4, 3, 2, 1}) {
             const long long most = batch_items(b, planes, b->grid, nullptr);
@@ -1499,13 +1505,14 @@ static int batch_build_typed(lb_batch* b)
             least = most;
             b->seg_planes = planes;
         }
+        b->planned_grid = b->grid;
+        b->planned_tile_y = b->tile_y;
     }
+    items.reserve((size_t)b->nitems);  // the list is as long again when only parameters changed
     batch_items(b, b->seg_planes, b->grid, &items);
     for (int i = 0; i < b->nbox; ++i)
-        for (int p = 0; p < 2; ++p) {
-            args[2 * i + p] = step_args<S>(b->box[i], p);
-            args[2 * i + p].tiles_y = (b->box[i]->ny + b->tile_y - 1) / b->tile_y;
-        }
+        for (int p = 0; p < 2; ++p)  // (the segments are the work list's)
+            args[2 * i + p] = step_args<S>(b->box[i], p, (b->box[i]->ny + b->tile_y - 1) / b->tile_y, 1);
     if (b->dargs) cudaFree(b->dargs);
     if (b->ditems) cudaFree(b->ditems);
     if (b->dmaps) cudaFree(b->dmaps);
@@ -1778,10 +1785,11 @@ struct AdjScratch {
 template <class S>
 static cudaError_t adj_step_into(lb_ctx* c, const void* src, void* dst, int ns, const CUtensorMap* maps, cudaStream_t st)
 {
-    StepArgs<S> A = step_args<S>(c, 0);
+    const Schedule& d = schedule(c);
+    StepArgs<S> A = step_args<S>(c, 0, d.yt, d.nseg);
     A.src = (const S*)src;
     A.dst = (S*)dst;
-    const int ty = schedule(c).ty;
+    const int ty = d.ty;
     if (ns) return (cudaError_t)tma_step<S>(0, ty, ns, tau_one(c), maps, &A, st);
     return launch_step<S>(A, ty, c->general, tau_one(c), st);
 }

@@ -86,3 +86,29 @@ def test_batch_refuses_a_box_stepped_alone(lbsc):
         batch.box(0).step(1)
     batch.step(3)
     batch.close()
+
+
+def test_set_params_of_many_boxes_costs_what_it_costs_of_few(lbsc):
+    """Setting one box's parameters does not search the whole batch's work list again: 64 boxes against 4, and the boxes
+    then step as lattices of their own with the same parameters do."""
+    import time
+    contact = dict(g_br=0.08, force_weights=1, force_scale=1.25)
+
+    def median(nbox):
+        fields = [W.droplet_fields(48, 40, 48, 12.0, seed=i) for i in range(nbox)]
+        b = lbsc.Batch(fields, [lbsc.Params(**contact)] * nbox)
+        ts = []
+        for i in range(nbox * 4):
+            t = time.perf_counter()
+            b.set_params(i % nbox, lbsc.Params(**dict(contact, g_br=0.07 + 0.0005 * (i % nbox))))
+            ts.append(time.perf_counter() - t)
+        b.step(40)
+        for i in (0, nbox - 1):
+            lat = lbsc.Lattice(*fields[i]).set_params(**dict(contact, g_br=0.07 + 0.0005 * i)).step(40)
+            assert np.array_equal(b.box(i).populations()[:, :, 1:-1], lat.populations()[:, :, 1:-1])
+            lat.close()
+        b.close()
+        return np.median(ts)
+
+    few, many = median(4), median(64)
+    assert many < 2.0 * few, (few, many)
