@@ -232,12 +232,27 @@ static double estimate(const lb_ctx* c, int ty, int ns, int occ, long long items
 // left open the least estimate among one to three waves of resident CTAs and
 // even row splits of up to a third more tiles than needed. Chosen once after
 // every change of schedule, parameters or geometry; it changes no value.
+constexpr int kFarPlanes = 40;
 static const Schedule& schedule(lb_ctx* c)
 {
     if (c->sched.ty) return c->sched;
     const int nzf = c->zhi - c->zlo, ntx = (c->nx + 31) / 32, ny = c->ny;
     Schedule best;
     double least = 0;
+    // Planar lattices far past L2: the rows of a tile's ring come from L2 only
+    // while the neighbouring CTAs are within a few planes of each other (the CTAs
+    // in flight move 12 to 30 MB a plane), and the longer they march the further
+    // apart they are; the estimate knows nothing of that. So segments there have
+    // kFarPlanes planes at most, FP32 takes two stages (two CTAs an SM instead of
+    // five) and 16-bit storage one. us a step without this rule and with it: FP32
+    // 320^3 1944 and 1605 (one stage with segments of 40 planes 1776), 256^3 879
+    // and 808, 400x400x200 2104 and 1566, 192^3 373 and 344, 512x512x40 519 and
+    // 483; BF16 320^3 1362 and 986, 400x400x200 1504 and 998. The lines: 176^3 (1.65 GB)
+    // FP32 275 without and 282 with, 1024x1024x12 504 and 531, BF16 128x128x1000,
+    // whose 64 columns are in flight together, 507 and 523.
+    const double pops = (double)c->fluid_nodes * 2 * Q * elem_size(c->prec);
+    const bool far = tau_one(c) && !c->general && c->variant == LB_STEP_AUTO && 2 * pops > 1.8e9 &&
+                     (c->prec == LB_F32 ? nzf >= 14 : nzf > kFarPlanes && (long long)ntx * ((ny + 7) / 8) >= c->nsm);
     const int tys[2] = {c->tile_y_req ? c->tile_y_req : 4, c->tile_y_req || c->prec == LB_F32 || !tau_one(c) ? 0 : 8};
     // TMA asked for by name takes three stages, else two
     for (int ty : tys) {
@@ -246,6 +261,7 @@ static const Schedule& schedule(lb_ctx* c)
         int stages[2] = {1, 2};
         if (c->variant == LB_STEP_TMA) stages[0] = 3;
         if (!tau_one(c) && c->variant == LB_STEP_AUTO) stages[0] = 2;  // holds v in fewer registers than one stage does
+        if (far) stages[0] = stages[1] = c->prec == LB_F32 ? 2 : 1;
         if (c->stages) stages[0] = stages[1] = c->stages;
         for (int i = 0; i < 2; ++i) {
             const int ns = stages[i];
@@ -261,10 +277,11 @@ static const Schedule& schedule(lb_ctx* c)
             const int yt1 = c->tile_y_req ? yt0 : (base + base / 3 < ny ? base + base / 3 : ny);
             for (int yt = yt0; yt <= yt1; ++yt) {
                 if (yt > yt0 && (ny + yt - 1) / yt < ty - 1) break;
-                for (int w = 1; w <= 3; ++w) {
-                    const long long col = (long long)ntx * yt;
+                for (int w = 1; w <= (far ? 16 : 3); ++w) {
+                    const long long col = (long long)ntx * yt, lo = far ? (nzf + kFarPlanes - 1) / kFarPlanes : 1;
                     long long seg = c->nseg_req ? c->nseg_req : (long long)w * c->nsm * occ / col;
-                    seg = seg < 1 ? 1 : (seg > nzf ? nzf : seg);
+                    seg = c->nseg_req || seg > lo ? seg : lo;
+                    seg = seg > nzf ? nzf : seg;
                     const double t = estimate(c, ty, ns, occ, col * seg, (int)((nzf + seg - 1) / seg) + 2);
                     if (!best.ty || t < least) {
                         best = Schedule{ty, yt, (int)seg, ns};

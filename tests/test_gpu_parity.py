@@ -839,3 +839,29 @@ def test_first_readback_of_a_small_lattice(n):
     assert out.returncode == 0, out.stderr[-2000:]
     first = float(out.stdout.split()[0])
     assert first < {32: 240, 64: 400}[n], out.stdout  # us: half way between 116 and 365, 263 and 533
+
+
+@pytest.mark.parametrize("precision,tile_y,stages", [("f32", 4, 2), ("bf16", 8, 1)])
+def test_automatic_schedule_of_a_lattice_past_l2(lbsc, precision, tile_y, stages):
+    """320^3: the automatic schedule takes no more than a tenth longer a step than segments of 40 planes, which keep
+    neighbouring tiles near each other, and gives the same values."""
+    import time
+    n = 320
+    rr = np.full((n, n, n), 0.4)
+    rr[:, ::7] = 0.1
+    rb = np.full((n, n, n), 0.3)
+    best = []
+    for named in (False, True):
+        lat = lbsc.Lattice(rr, rb, precision).set_params(**CONTACT)
+        if named:
+            lat.set_step_variant("auto", stages).set_tiling(tile_y, 0, 8)
+        lat.step(16).sync()
+        ts = []
+        for _ in range(4):
+            t = time.perf_counter()
+            lat.step(32).sync()
+            ts.append(time.perf_counter() - t)
+        best.append((min(ts) / 32, lat.conservation()))
+        lat.close()
+    assert best[0][0] < 1.1 * best[1][0], best
+    assert np.array_equal(best[0][1], best[1][1])
