@@ -1452,6 +1452,8 @@ static void batch_drop_graphs(lb_batch* b)
         }
 }
 
+constexpr long long kBatchWide = 9000;  // nodes of a plane (batch_build_typed)
+
 // nseg segments of about `planes` planes of a box's fluid planes
 static int batch_segments(const lb_ctx* c, int planes)
 {
@@ -1498,7 +1500,17 @@ static int batch_build_typed(lb_batch* b)
     // stage, 4- or 8-row tiles); LDG the load-from-global one
     // (the shared-memory attribute first: the occupancy of a kernel above 48 KB counts 0 without it)
     const bool want_tma = b->variant != LB_STEP_LDG;
-    b->tile_y = b->tile_y_req ? b->tile_y_req : (want_tma && b->prec == LB_F32 ? 4 : 8);
+    // FP32: 4 rows, which share out better (64 boxes of edge 48-96 take 1377 us a step, with 8 rows 1434), but 8 where the
+    // boxes are far past L2 (see schedule) and nearly all nodes lie in boxes of 96 x 96 and more, whose CTAs re-read fewer
+    // ring rows when they drift apart (16 boxes of 96^3: 674 and 733, 8 of 128^3: 814 and 885, 4 of 192^3: 1366 and 1719)
+    long long nodes = 0, wide = 0;
+    for (const lb_ctx* c : b->box) {
+        nodes += c->fluid_nodes;
+        if (c->nx * (long long)c->ny > kBatchWide) wide += c->fluid_nodes;
+    }
+    const bool far = want_tma && b->prec == LB_F32 && 2.0 * 2 * Q * elem_size(b->prec) * (double)nodes > 1.5e9;
+    const bool large = far && 10 * wide > 9 * nodes;
+    b->tile_y = b->tile_y_req ? b->tile_y_req : (want_tma && b->prec == LB_F32 && !large ? 4 : 8);
     auto tma_op = [&](int op) {
         return tma_batch<S>(op, b->tile_y, b->tau1, nullptr, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr);
     };
@@ -1515,8 +1527,13 @@ static int batch_build_typed(lb_batch* b)
         b->seg_planes = b->seg_planes_req;
         b->planned_grid = 0;
     } else if (b->planned_grid != b->grid || b->planned_tile_y != b->tile_y) {
+        // far past L2 FP32 items of 4 rows have 24 planes at most, so that neighbouring CTAs stay near each other (16 boxes of
+        // 96^3: 929 us a step with 64, 712 with 24; 12 mixed ones no difference). 8 rows re-read less, and large boxes have
+        // 32 at least
+        const int from = b->tma && far && b->tile_y == 4 ? 24 : 64, to = b->tma && large && b->tile_y == 8 ? 32 : 1;
         long long least = 0;
         for (int planes : {64, 48, 32, 24, 20, 16, 12, 10, 8, 6, 4, 3, 2, 1}) {
+            if (planes > from || planes < to) continue;
             const long long most = batch_items(b, planes, b->grid, nullptr);
             if (least && most >= least) continue;
             least = most;

@@ -112,3 +112,27 @@ def test_set_params_of_many_boxes_costs_what_it_costs_of_few(lbsc):
 
     few, many = median(4), median(64)
     assert many < 2.0 * few, (few, many)
+
+
+@pytest.mark.parametrize("edge,nbox", [(96, 16), (128, 8), (192, 3)])
+def test_automatic_schedule_of_large_boxes(lbsc, edge, nbox):
+    """Batches of large FP32 boxes, far past L2: the automatic tile height and planes an item take no more than a tenth
+    longer a step than 8 rows and 32 planes."""
+    import time
+    contact = dict(g_br=0.08, force_weights=1, force_scale=1.25)
+    fields = [W.droplet_fields(edge, edge, edge, 0.25 * edge, seed=0)] * nbox
+    b = lbsc.Batch(fields, [lbsc.Params(**contact)] * nbox)
+    best = []
+    for named in (False, True):
+        if named:
+            b.set_schedule(8, 32, 0)
+        b.step(32).conservation()
+        ts = []
+        for _ in range(4):
+            t = time.perf_counter()
+            b.step(64)
+            b.box(0).sync()
+            ts.append(time.perf_counter() - t)
+        best.append(min(ts) / 64)
+    b.close()
+    assert best[0] < 1.1 * best[1], best
