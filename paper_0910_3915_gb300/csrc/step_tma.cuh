@@ -286,11 +286,16 @@ __device__ __forceinline__ bool tma_item(const TmaMaps& maps, const StepArgs<S>&
         for (int q = 0; q < NIT; ++q) solid_it[q] = solid_own;
         if constexpr (kGeneral) {
             const uint32_t* mask = A.nbmask + wrapi(zp, nz) * plane;
-            nb = own_rd ? __ldg(mask + own_node) : kSelfSolid;
+            auto word = [&](int node) {
+                if constexpr (kCheckBounds)
+                    if (!in_bounds((long long)wrapi(zp, nz) * plane + node, (long long)plane * nz, A.err)) return kSelfSolid;
+                return __ldg(mask + node);
+            };
+            nb = own_rd ? word(own_node) : kSelfSolid;
             solid_own = (nb & kSelfSolid) != 0;
 #pragma unroll
             for (int q = 0; q < NIT; ++q)
-                if (it_code[q] >= 0) solid_it[q] = (__ldg(mask + it_node[q]) & kSelfSolid) != 0;
+                if (it_code[q] >= 0) solid_it[q] = (word(it_node[q]) & kSelfSolid) != 0;
         }
         const bool ok = mbar_wait(&bar[gi % NS], (gi / NS) & 1u);
         float2* spl = psi_plane(zp);

@@ -78,3 +78,29 @@ def test_bounds_checked_build_runs_clean_and_matches_release(tmp_path):
     assert not lbsc.build_flags() & lbsc.LB_BUILD_BOUNDS_CHECKED
     for i, c in enumerate(CASES):
         assert np.array_equal(dbg[f"c{i}"], run_case(lbsc, *c), equal_nan=True), c
+
+
+# general geometries on the TMA-staged kernel, whose mask words are checked too: every built height and stage count
+GENERAL_TMA = [
+    ("f32", (36, 20, 16), "auto", 1, 4, 0, 2, True),
+    ("f32", (70, 19, 16), "auto", 2, 4, 7, 3, True),
+    ("f16", (33, 17, 16), "auto", 1, 8, 0, 1, True),
+    ("f16", (96, 20, 16), "auto", 2, 4, 0, 16, True),
+    ("bf16", (65, 23, 16), "auto", 2, 8, 5, 2, True),
+    ("bf16", (36, 20, 16), "auto", 1, 4, 20, 4, True),
+]
+
+
+def test_bounds_checked_general_geometries_on_the_tma_kernel(tmp_path):
+    from paper_0910_3915_gb300 import build as B
+    from paper_0910_3915_gb300 import lbsc
+    out = tmp_path / "debug.npz"
+    env = dict(os.environ, LBSC_LIBRARY=B.build(debug_bounds=True))
+    child = CHILD.replace("import CASES,", "import GENERAL_TMA as CASES,")
+    r = subprocess.run([sys.executable, "-c", child, ROOT, str(out)], env=env, capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+    dbg = np.load(out)
+    lbsc.load()
+    for i, c in enumerate(GENERAL_TMA):
+        fluid = np.broadcast_to(geometry(*c[1]) == 0, dbg[f"c{i}"].shape)
+        assert np.array_equal(dbg[f"c{i}"][fluid], run_case(lbsc, *c)[fluid]), c
