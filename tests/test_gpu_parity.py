@@ -865,3 +865,25 @@ def test_automatic_schedule_of_a_lattice_past_l2(lbsc, precision, tile_y, stages
         lat.close()
     assert best[0][0] < 1.1 * best[1][0], best
     assert np.array_equal(best[0][1], best[1][1])
+
+
+@pytest.mark.parametrize("dims", [(33, 9, 12), (128, 129, 64), (300, 700, 5)])
+def test_readback_of_a_moving_state(lbsc, dims):
+    """Velocities that differ in every component and node, below, at and above a staging half: without interaction u is
+    sum(n c) / sum(n) of the same FP32 populations, to the rounding of 19 FP32 additions."""
+    nx, ny, nz = dims
+    rng = np.random.Generator(np.random.PCG64(nx))
+    n = np.zeros((2, 19, nz, ny, nx))
+    n[:] = rng.uniform(0.01, 0.05, size=n.shape).astype(np.float32)
+    lat = lbsc.Lattice(np.full((nz, ny, nx), 0.4), np.full((nz, ny, nx), 0.3)).set_populations(n)
+    r, b, u, _ = lat.moments(velocity=True)
+    c = np.stack(oracle.lattice()[0]).reshape(19, 3)
+    rho = n.sum(1)
+    j = np.einsum("kd,akzyx->dzyx", c, n)
+    fluid = slice(1, nz - 1)
+    # 19 (densities) and 38 (momentum, of values whose magnitudes sum to the density) additions of 2^-24 each
+    assert np.abs(r - rho[0])[fluid].max() <= 19 * 2.0 ** -24 * rho[0].max()
+    assert np.abs(b - rho[1])[fluid].max() <= 19 * 2.0 ** -24 * rho[1].max()
+    want = (j / rho.sum(0))[:, fluid]
+    assert np.abs(u[:, fluid] - want).max() <= (38 + 38 + 2) * 2.0 ** -24
+    assert np.all(u[:, [0, -1]] == 0)

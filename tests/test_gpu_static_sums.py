@@ -96,3 +96,38 @@ def test_a_large_field_without_finite_values_is_counted(masked):
     assert np.isnan(got[:5]).all()
     del n, solid
     torch.cuda.empty_cache()
+
+
+def test_sums_captured_in_a_graph():
+    """Under stream capture (the second kernel is launched dependently on the first): replayed twice on changed inputs, with
+    a second call in the same capture, the sums are those of calls outside a capture, bit for bit."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0910_3915_gb300 import lbsc
+    dims = [(97, 33, 32), (64, 9, 5)]
+    n = [torch.rand((2, 19, nz, ny, nx), dtype=torch.float64, device="cuda") for nx, ny, nz in dims]
+    out = [torch.zeros(8, dtype=torch.float64, device="cuda") for _ in dims]
+
+    def sums():
+        for a, (nx, ny, nz), o in zip(n, dims, out):
+            lbsc.conservation_static(a.data_ptr(), None, nx, ny, nz, o.data_ptr())
+
+    sums()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sums()
+    for k in range(2):
+        for a in n:
+            a.mul_(0.5).add_(0.01 * k)
+        sums()
+        torch.cuda.synchronize()
+        want = [o.cpu().numpy().copy() for o in out]
+        for o in out:
+            o.zero_()
+        graph.replay()
+        graph.replay()
+        torch.cuda.synchronize()
+        for o, w in zip(out, want):
+            assert np.array_equal(o.cpu().numpy(), w)
