@@ -1137,11 +1137,10 @@ int lb_moments(lb_ctx* c, double* rho_r, double* rho_b, double* u, double cons[8
     LB_CUDA(c, dispatch_cons(c));
     if (n) LB_CUDA(c, read_back(fields, n, N, c->stream, c->values_read));
     c->values_read += n * N;
+    const int rc = wait(c);
+    if (rc != LB_OK) return rc;
     double tmp[8];
-    int rc = wait(c);
-    if (rc == LB_OK) rc = take_cons(c, tmp);
-    if (cons && (rc == LB_OK || rc == LB_ERR_NAN)) memcpy(cons, tmp, sizeof(tmp));
-    return rc;
+    return take_cons(c, cons ? cons : tmp);  // filled whatever the state's verdict is
 }
 
 static int solve4(double M[4][4], double v[4], double s[4])
