@@ -407,13 +407,14 @@ __device__ __noinline__ void add_crossing_f64(float2* acc, int stride, int x, in
                                               const AngleArgs& A)
 {
     const double q0 = (double)p0 - A.level, q1 = (double)p1 - A.level, t = q0 / (q0 - q1);
-    const double p[3] = {x + t * (d == 0), y + t * (d == 1), z + t * (d == 2)};
+    double p[3] = {x + t * (d == 0), y + t * (d == 1), z + t * (d == 2)};
     if (d == 2 && q0 > 0) {
         const float2 top = acc[0];
         const Two v = two_f64(z + t);
         if (less2(Two{top.x, top.y}, v)) acc[0] = make_float2(v.h, v.l);
     }
     if (p[2] < A.zref) return;
+    for (int q = 0; q < 3; ++q) p[q] -= A.origin[q];
     const double rr = p[0] * p[0] + p[1] * p[1] + p[2] * p[2];
     const double v[14] = {1.0,         p[0] * p[0], p[0] * p[1], p[0] * p[2], p[0],      p[1] * p[1], p[1] * p[2],
                           p[1],        p[2] * p[2], p[2],        p[0] * rr,   p[1] * rr, p[2] * rr,   rr};
@@ -422,8 +423,8 @@ __device__ __noinline__ void add_crossing_f64(float2* acc, int stride, int x, in
 
 // An interface crossing between node (x, y, z) (phi = p0) and its neighbour
 // along axis d (phi = p1): the top crossing (along z, from phi > level
-// below to phi <= level above) and the sphere-fit sums of the crossing point at
-// or above the reference plane, into the thread's accumulators acc[i * stride].
+// below to phi <= level above) and the sphere-fit sums of the crossing point p at
+// or above the reference plane, less A.origin, into the thread's accumulators acc[i * stride].
 // Out of line: it is reached from a few places and rarely, and the row loop
 // fits the instruction cache without it.
 __device__ __noinline__ void add_crossing(float2* acc, int stride, int x, int y, int z, int d, float p0, float p1,
@@ -432,15 +433,16 @@ __device__ __noinline__ void add_crossing(float2* acc, int stride, int x, int y,
     const Two gap = norm2(two_sum(p0, -p1));
     if (!pairs_serve(fabsf(gap.h))) return add_crossing_f64(acc, stride, x, y, z, d, p0, p1, A);
     const Two t = div22(over(p0, A), gap);
-    const Two c[3] = {two_int(x), two_int(y), two_int(z)};
+    const Two zc = d == 2 ? norm2(two_int(z) + t) : two_int(z);
+    if (d == 2 && above(p0, A)) {  // phi > level below, <= level above
+        const float2 top = acc[0];
+        if (less2(Two{top.x, top.y}, zc)) acc[0] = make_float2(zc.h, zc.l);
+    }
+    if (less2(zc, Two{A.zh, A.zl})) return;
+    const Two c[3] = {two_int(x - A.origin[0]), two_int(y - A.origin[1]), two_int(z - A.origin[2])};
     Two p[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) p[q] = d == q ? norm2(c[q] + t) : c[q];
-    if (d == 2 && above(p0, A)) {  // phi > level below, <= level above
-        const float2 top = acc[0];
-        if (less2(Two{top.x, top.y}, p[2])) acc[0] = make_float2(p[2].h, p[2].l);
-    }
-    if (less2(p[2], Two{A.zh, A.zl})) return;
     auto add = [&](int i, Two v) { add_to(&acc[i * stride], v); };
     const Two xx = norm2(mul22(p[0], p[0])), yy = norm2(mul22(p[1], p[1])), zz = norm2(mul22(p[2], p[2]));
     const Two rr = norm2((xx + yy) + zz);
@@ -468,7 +470,7 @@ __device__ __noinline__ void add_crossing(float2* acc, int stride, int x, int y,
 //  [1]  positive length along x of the reference-plane interpolant of phi
 //       (the node at z0 adds its segment to x + 1, periodic);
 //  [2..15] sums over crossings along +x, +y, +z at or above the reference
-//       plane: 1, xx, xy, xz, x, yy, yz, y, zz, z, x rr, y rr, z rr, rr (rr = |p|^2);
+//       plane, of their points less A.origin: 1, xx, xy, xz, x, yy, yz, y, zz, z, x rr, y rr, z rr, rr (rr = |p|^2);
 //  [16] (max) max of phi over fluid nodes, [17] (max) of -phi (the contrast).
 // All in pairs of FP32 numbers: with FP64 sums (a drained queue took about 70
 // FP64 operations, 2240 cycles of an SM's one FP64 lane) the kernel took 53 us
@@ -477,7 +479,7 @@ __device__ __noinline__ void add_crossing(float2* acc, int stride, int x, int y,
 // instructions, a third of them for crossings; phi is 8 MB, in L2).
 // A thread's sums wait in shared memory, and a warp reduces a value only if one
 // of its lanes holds a contribution to it. The last block to finish adds the
-// blocks' rows, in order, and writes the 19 values lb_contact_angle works with.
+// blocks' rows, in order, and writes the 18 values lb_contact_angle works with.
 __global__ void __launch_bounds__(kAngleThreads, 3) angle_kernel(FieldArgs F, AngleArgs A, const float* P,
                                                               float2* __restrict__ part, unsigned int* __restrict__ ticket,
                                                               double* __restrict__ out)
@@ -1148,10 +1150,11 @@ cudaError_t launch_phi(const FieldArgs& F, const S* f, const Scratch& W, cudaStr
     return cudaGetLastError();
 }
 
-cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, double level, double* part,
-                         unsigned int* ticket, double* out, cudaStream_t st)
+cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, double level, const int (&origin)[3],
+                         double* part, unsigned int* ticket, double* out, cudaStream_t st)
 {
     AngleArgs A;
+    for (int q = 0; q < 3; ++q) A.origin[q] = origin[q];
     auto split = [](double v, float& h, float& l) {
         h = (float)v;
         l = (float)(v - (double)h);

@@ -19,10 +19,11 @@ constexpr int kPartVals = 19;           // doubles a row
 // The contact angle's level (lh + ll) and the least FP32 number above it, the
 // reference height zref (zh + zl), its plane z0 (nz where that lies outside)
 // and fraction there, in pairs of FP32 numbers, and level, zref and the
-// fraction in FP64 for the nodes that pairs do not serve.
+// fraction in FP64 for the nodes that pairs do not serve. The sphere fit's
+// sums are about the point `origin`.
 struct AngleArgs {
     float lh, ll, least, zh, zl, fzh, fzl;
-    int z0;
+    int z0, origin[3];
     double level, zref, fz;
 };
 
@@ -131,10 +132,10 @@ cudaError_t launch_fields(const FieldArgs& F, const S* f, const Scratch& W, bool
 // phi = rho_r - rho_b of every node into W.rho[0] (the contact angle's input)
 template <class S>
 cudaError_t launch_phi(const FieldArgs& F, const S* f, const Scratch& W, cudaStream_t st);
-// the contact angle's 18 values of phi in W.rho[0] (angle_kernel) into out; part: kAngleRow doubles a
-// block, ticket: a counter that is 0 between calls
-cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, double level, double* part,
-                         unsigned int* ticket, double* out, cudaStream_t st);
+// the contact angle's 18 values of phi in W.rho[0] (angle_kernel) into out, the fit's sums about origin; part:
+// kAngleRow doubles a block, ticket: a counter that is 0 between calls
+cudaError_t launch_angle(const FieldArgs& F, const Scratch& W, double zref, double level, const int (&origin)[3],
+                         double* part, unsigned int* ticket, double* out, cudaStream_t st);
 // pressure tensor of Sec. 4.1 (after launch_fields): every node, per-plane
 // sums (part: 8 nz split doubles of scratch), and fixed-point radial bins (see fields.cu)
 constexpr int kPressThreads = 128;

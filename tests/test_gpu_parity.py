@@ -887,3 +887,29 @@ def test_readback_of_a_moving_state(lbsc, dims):
     want = (j / rho.sum(0))[:, fluid]
     assert np.abs(u[:, fluid] - want).max() <= (38 + 38 + 2) * 2.0 ** -24
     assert np.all(u[:, [0, -1]] == 0)
+
+
+@pytest.mark.parametrize("dims,at", [((1024, 24, 64), 980.0), ((250, 40, 48), 236.5), ((128, 96, 64), 64.0), ((40, 36, 2000), 20.0),
+                                     ((3000, 20, 20), 2.0)])
+def test_contact_angle_sphere_fit_away_from_the_origin(lbsc, dims, at):
+    """A cap of radius 10 (16 in the middle lattice) anywhere in a long lattice: the sphere's centre and radius against the
+    oracle on coordinates that begin near the cap, on the same phi. Sums of 46 bits about a point within 8 spreads of the
+    crossings, through a 4 x 4 solve: 1e-7, as on the lattices above."""
+    nx, ny, nz = dims
+    R = 16.0 if nx == 128 else 0.42 * min(ny, 24)
+    z, y, x = np.meshgrid(np.arange(nz), np.arange(ny), np.arange(nx), indexing="ij")
+    zc = nz - 40.0 if nz == 2000 else 0.5
+    s = np.tanh((R - np.sqrt((x - at) ** 2 + (y - ny / 2) ** 2 + (z - zc) ** 2)) / 2.5)
+    lat = lbsc.Lattice(0.37 + 0.33 * s, 0.37 - 0.33 * s)
+    r, b, _, _ = lat.moments()
+    phi = (r.astype(np.float32) - b.astype(np.float32)).astype(np.float64)
+    solid = W.wall_mask(nx, ny, nz)
+    lo, hi = max(0, int(at) - 40), min(nx, int(at) + 40)  # the part of the lattice that holds every crossing
+    zlo = nz - 80 if nz == 2000 else 0
+    cut = (slice(zlo, nz), slice(0, ny), slice(lo, hi))
+    cut_solid = solid[cut].copy()
+    o = oracle.contact_angle(phi[cut].copy(), 0 * phi[cut], cut_solid, 2.0 if zlo == 0 else 1.0, 0.1)
+    d = lat.contact_angle(2.0, level=0.1)
+    assert o["n_points"] >= 100 and d["n_points"] == o["n_points"]
+    assert abs(d["xc"] - (o["xc"] + lo)) <= 1e-7 and abs(d["yc"] - o["yc"]) <= 1e-7 and abs(d["zc"] - (o["zc"] + zlo)) <= 1e-7
+    assert abs(d["r_fit"] - o["r_fit"]) <= 1e-7
