@@ -260,11 +260,12 @@ struct Dest {
         nb = 0;
         hoff = 0;
     }
-    // the node's offset in its plane after the step dx, dy, in nodes
+    // offset in the plane after the step dx, dy (kBytes: in bytes, up to 2^32)
+    __device__ __forceinline__ uint32_t in_plane(int dx, int dy) const { return (uint32_t)ro[dy + 1] + (uint32_t)xo[dx + 1]; }
+    // the same in nodes
     __device__ __forceinline__ int plane_node(int dx, int dy) const
     {
-        if constexpr (kBytes) return (int)((uint32_t)(ro[dy + 1] + xo[dx + 1]) / kPair);
-        else return ro[dy + 1] + xo[dx + 1];
+        return (int)(kBytes ? in_plane(dx, dy) / kPair : in_plane(dx, dy));
     }
     // the pair of velocity k's slot at x + (dx, dy, dz), or, on a wall link, of slot kbar at x
     __device__ __forceinline__ S* pair(S* dst, long long slot, int k, int kbar, int dx, int dy, int dz, bool wall) const
@@ -274,7 +275,7 @@ struct Dest {
             const size_t slot_b = (size_t)slot * kPair;
             char* const there = b + (size_t)zo[dz + 1] * kPair + (size_t)k * slot_b;
             char* const here = b + (size_t)zo[1] * kPair + (size_t)kbar * slot_b;
-            return (S*)((wall ? here : there) + (uint32_t)(wall ? ro[1] + xo[1] : ro[dy + 1] + xo[dx + 1]));
+            return (S*)((wall ? here : there) + (wall ? in_plane(0, 0) : in_plane(dx, dy)));
         } else {
             const int o = wall ? zo[1] + ro[1] + xo[1] : zo[dz + 1] + ro[dy + 1] + xo[dx + 1];
             return dst + 2 * (o + (long long)(wall ? kbar : k) * slot);
