@@ -574,14 +574,12 @@ static long long tma_dispatch(int op, int ty, int ns, bool t1, const CUtensorMap
 
 // The batched TMA kernel for one stage and 4- or 8-row tiles: op 0 launches
 // on `grid` CTAs (returns a cudaError_t), op 1 sets the shared-memory
-// attribute, op 2 returns resident CTAs per SM (0 if not built).
+// attribute, op 2 returns the CTAs per SM to launch (0 if not built).
 template <class S, int TY, bool T1>
 static long long tma_batch_one(int op, const TmaMaps* maps, const StepArgs<S>* args, const int4* items, int nitems,
                                int parity, int nbox, uint32_t* done, int grid, cudaStream_t st)
 {
-    // FP32 8-row tiles ask for 9000 bytes they do not use: three CTAs an SM either way, but with the SM's memory
-    // split for shared memory in full 64 boxes take 1344 us a step, else 1863
-    const size_t smem = TmaGeom<S, TY, 1, true>::SMEM + (TY == 8 && sizeof(S) == 4 ? 9000 : 0);
+    constexpr size_t smem = TmaGeom<S, TY, 1, true>::SMEM;
     if (op == 0) {
         batch_tma_kernel<S, TY, 1, T1><<<grid, 32 * TY, smem, st>>>(maps, args, items, nitems, parity, nbox, done);
         return cudaGetLastError();
@@ -593,7 +591,9 @@ static long long tma_batch_one(int op, const TmaMaps* maps, const StepArgs<S>* a
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_tma_kernel<S, TY, 1, T1>, 32 * TY, smem) !=
         cudaSuccess)
         return 0;
-    return n;
+    // three FP32 CTAs of 8-row tiles fit, but two re-read fewer ring rows: they stay nearer each other (64 boxes of edge
+    // 48-96 take 1434 us a step, 1863 with three; 8 boxes of 128^3 814 and 1052)
+    return TY == 8 && sizeof(S) == 4 && n > 2 ? 2 : n;
 }
 
 template <class S>
