@@ -306,8 +306,8 @@ def run_ours(args):
             lat.conservation()  # one kernel
             launches += 1
     # the last conservation sums and the contact angle in one pass over the populations
-    cons_end, angle = lat.measure(5.0)  # conservation (with phi), angle and finish kernels
-    launches += 3
+    cons_end, angle = lat.measure(5.0)  # conservation (with phi) and angle kernels
+    launches += 2
     t1.record(stream)
     torch.cuda.synchronize()
     replicas.barrier()

@@ -266,8 +266,9 @@ int lb_conservation(lb_ctx* ctx, double cons[8]);
 /* Contact angle of the r droplet on the bottom wall (Sec. 3): phi = rho_r -
  * rho_b = 0 located by linear interpolation, apex height h, base b' at the
  * reference plane `offset` above the wall plane (the paper uses 5 l.u.),
- * sphere radius r from that cap, base b at the wall from r and h, then theta.
- * Needs the default wall at z = 0 and offset >= 0. out->ok = 0 (and LB_OK)
+ * sphere radius r from that cap, base b at the wall from r and h, then theta;
+ * and the sphere fitted to the interface points. Lengths and fit from sums in pairs
+ * of FP32 numbers (about 46 bits) over FP32 phi. Needs the default wall at z = 0 and offset >= 0. out->ok = 0 (and LB_OK)
  * when no cap is found. */
 int lb_contact_angle(lb_ctx* ctx, double offset, lb_droplet* out);
 
@@ -291,9 +292,12 @@ int lb_measure(lb_ctx* ctx, double cons[8], double offset, lb_droplet* out);
  *        + 1/4 sum_(a, abar) g kappa sum_k G_k [psi^a(x) psi^abar(x+c_k) + psi^abar(x) psi^a(x+c_k)] c_ki c_kj
  * with u the velocity lb_moments reports, G_k and kappa the force's weights and
  * scale, and psi of a solid neighbour the wall pseudo-density (as in the
- * force). Solid nodes contribute nothing. Evaluated in FP64 from the stored
- * populations. Components are ordered xx, yy, zz, xy, xz, yz. Each call
- * allocates and frees its device scratch and synchronises the stream. */
+ * force). Solid nodes contribute nothing. Evaluated from the stored populations
+ * in pairs of FP32 numbers (about 46 bits; u and psi are FP32), in FP64 at nodes
+ * whose values FP32 does not hold. Components are ordered xx, yy, zz, xy, xz, yz.
+ * Each call synchronises the stream. lb_pressure_tensor allocates and frees its
+ * device array; the other two work in the context's scratch (lb_pressure_profile
+ * of a very tall lattice allocates). */
 
 /* P: host, 6*nx*ny*nz doubles, P[c*N + idx] (zeros on solid nodes). */
 int lb_pressure_tensor(lb_ctx* ctx, double* P);
@@ -304,7 +308,7 @@ int lb_pressure_tensor(lb_ctx* ctx, double* P);
  * then the fluid count (zeros for a solid plane). gamma_sum (may be NULL):
  * sum over planes with fluid of P_N - P_T, P_N = P_zz, P_T = (P_xx + P_yy)/2;
  * a box with m identical interfaces holds m gamma. The per-plane sums are
- * deterministic (one block per plane, fixed order). */
+ * deterministic (fixed ranges of a plane's nodes, added in a fixed order). */
 int lb_pressure_profile(lb_ctx* ctx, double* prof, double* gamma_sum);
 
 /* Radial profile about centre[3] (x, y, z lattice coordinates; distances use

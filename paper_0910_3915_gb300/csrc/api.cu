@@ -229,8 +229,8 @@ static double estimate(const lb_ctx* c, int ty, int ns, int occ, long long items
 }
 
 // The schedule of the context's steps: the caller's choices, and for what was
-// left open the least estimate among one to three waves of resident CTAs and
-// even row splits of up to a third more tiles than needed. Chosen once after
+// left open the least estimate among one to three waves of resident CTAs (16
+// for lattices far past L2) and even row splits of up to a third more tiles than needed. Chosen once after
 // every change of schedule, parameters or geometry; it changes no value.
 constexpr int kFarPlanes = 40;
 static const Schedule& schedule(lb_ctx* c)
