@@ -62,9 +62,9 @@ __device__ __forceinline__ bool node_solid(const FieldArgs& F, int x, int y, int
 // need more than FP32 are taken in pairs (Dekker 1971, Knuth's two-sum): a
 // value is h + l with l far below h, a sum carries the rounding error of h in
 // l. That keeps about 46 bits, 7 less than FP64; what they are formed from (psi, u, phi) is FP32. Against 64 bits
-// from the same populations (28 lattices of edges 24-128 and one of 1024, three precisions) the pressure tensor, its
+// from the same populations (27 lattices of edges 24-128 and one of 1024, three precisions) the pressure tensor, its
 // profile, bins and tensions are off by as much as with FP64 (6.4e-8 of the tensor's largest entry, 1.5e-7 in a plane's
-// mean), the contact angle by 5e-6 degrees, the fitted one by 1e-6, equal to 0.1%.
+// mean), the contact angle by 1e-5 degrees at most and the fitted one by 8e-6, within 0.3% of FP64's error.
 struct Two {
     float h, l;
 };
@@ -858,7 +858,9 @@ __global__ void __launch_bounds__(kPressThreads, 5) pressure_plane_kernel(FieldA
     const int lo = (int)((long long)blockIdx.y * nxy / split), hi = (int)((long long)(blockIdx.y + 1) * nxy / split);
     Two sum[7];
     for (int v = 0; v < 7; ++v) sum[v] = two(0.f);
-    double odd[7] = {0, 0, 0, 0, 0, 0, 0};  // nodes taken in FP64
+    // sums of the nodes taken in FP64, per thread: rare, so not in registers
+    __shared__ double odd[7][kPressThreads];
+    for (int v = 0; v < 7; ++v) odd[v][threadIdx.x] = 0.0;
     int count = 0;
     bool odd_nodes = false;
     for (int c = lo + threadIdx.x; c < hi; c += kPressThreads) {
@@ -872,14 +874,14 @@ __global__ void __launch_bounds__(kPressThreads, 5) pressure_plane_kernel(FieldA
         } else {
             double D[6];
             node_pressure_f64<S>(F, f, W, x, y, z, D);
-            for (int v = 0; v < 6; ++v) odd[v] += D[v];
+            for (int v = 0; v < 6; ++v) odd[v][threadIdx.x] += D[v];
             odd_nodes = true;
         }
         const Two phi = two_sum(W.rho[0][i], -W.rho[1][i]);
         if (fabsf(phi.h) < kSumLimit) {
             sum[6] = norm2(sum[6] + phi);
         } else {
-            odd[6] += (double)W.rho[0][i] - (double)W.rho[1][i];
+            odd[6][threadIdx.x] += (double)W.rho[0][i] - (double)W.rho[1][i];
             odd_nodes = true;
         }
         ++count;
@@ -903,7 +905,7 @@ __global__ void __launch_bounds__(kPressThreads, 5) pressure_plane_kernel(FieldA
     const bool any_odd = __syncthreads_or(odd_nodes);
     if (any_odd) {  // uniform
         for (int v = 0; v < 7; ++v) {
-            const double t = warp_sum(odd[v]);
+            const double t = warp_sum(odd[v][threadIdx.x]);
             if (lane == 0) sodd[warp][v] = t;
         }
         __syncthreads();
