@@ -242,7 +242,8 @@ static const Schedule& schedule(lb_ctx* c)
     // Planar lattices far past L2: the rows of a tile's ring come from L2 only
     // while the neighbouring CTAs are within a few planes of each other (the CTAs
     // in flight move 12 to 30 MB a plane), and the longer they march the further
-    // apart they are; the estimate knows nothing of that. So segments there have
+    // apart they are (FP32 256x256x128 in segments of 63 planes reads 1.35 times its
+    // populations from HBM, with this rule 1.06); the estimate knows nothing of that. So segments there have
     // kFarPlanes planes at most, FP32 takes two stages (two CTAs an SM instead of
     // five) and 16-bit storage one. us a step without this rule and with it: FP32
     // 320^3 1944 and 1605 (one stage with segments of 40 planes 1776), 256^3 879

@@ -478,7 +478,7 @@ __device__ __noinline__ void add_crossing(float2* acc, int stride, int x, int y,
 // All in pairs of FP32 numbers: with FP64 sums (a drained queue took about 70
 // FP64 operations, 2240 cycles of an SM's one FP64 lane) the kernel took 53 us
 // at 128^3, bound by the SMs that met the most crossings. A block takes rows
-// gridDim apart for the same reason: the drop's rows spread over all SMs. Now 27 us at 128^3 (9 million
+// gridDim apart for the same reason: the drop's rows spread over all SMs. Now 28 us at 128^3 (9 million
 // instructions, a third of them for crossings; phi is 8 MB, in L2).
 // A thread's sums wait in shared memory, and a warp reduces a value only if one
 // of its lanes holds a contribution to it. The last block to finish adds the
