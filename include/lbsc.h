@@ -434,7 +434,9 @@ int lb_batch_create(lb_batch** out, int nbox, const int* dims, const double* rho
 int lb_batch_set_params(lb_batch* b, int i, const lb_params* params);
 
 /* Work split: tile height (4, 8, 16), z planes per work item, CTAs per SM of
- * the persistent grid (0 = as many as fit). Results do not depend on it. */
+ * the persistent grid (0 = automatic: as many as fit, but two with FP32 8-row tiles on
+ * the TMA kernel). Without this call tile height and planes are chosen from the boxes' sizes.
+ * Results do not depend on it. */
 int lb_batch_set_schedule(lb_batch* b, int tile_y, int planes_per_item, int ctas_per_sm);
 
 /* Choose the batch's step kernel: LB_STEP_AUTO (default) and LB_STEP_TMA take
